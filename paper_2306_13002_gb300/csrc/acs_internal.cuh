@@ -43,6 +43,12 @@ acs_status launch_block(const double* A, const double* B, const double* G, doubl
                         const double* prm, int form, cudaStream_t s);
 acs_status launch_stencil_plain(const double* u, const double* a, double* out, const Geom& g,
                                 const StarCoef& c, cudaStream_t s);
+// The star stencil in fixed point (star_fixed.cuh): its integer weights (kind 0: not for it), and the launch.
+void star_fix(const StarCoef& c, StarFix& fx);
+acs_status launch_star_fixed(const double* u, const double* a, double* out, const Geom& g, const StarCoef& c,
+                             const StarFix& fx, const acs_tile& t, cudaStream_t s);
+acs_status launch_star_fixed_gen(const double* u, const double* a, double* out, const Geom& g, const StarCoef& c,
+                                 const StarFix& fx, const acs_tile& t, cudaStream_t s);
 acs_status launch_stencil_saturated(const double* u, const double* a, double* out, const Geom& g,
                                     const StarCoef& c, const acs_tile& t, cudaStream_t s);
 

@@ -95,6 +95,16 @@ struct StarCoef {
     Pipe pp;
 };
 
+// The weights as integers for the fixed-point star march (star_fixed.cuh): c = (wh 2^LB + wl) 2^-w
+// with wh signed, index 0 the centre, then one axis (kind 1: the three axes share their weights,
+// LB 29) or three (kind 2, LB 28). The joined sum counts in units of 2^(LB + 29 - w) = 2^shift of
+// the inputs' unit; `neg`: the weights were negated to make the centre's negative. kind 0: the
+// weights do not suit (star_fix).
+struct StarFix {
+    unsigned wh[13], wl[13];
+    int shift, kind, neg;
+};
+
 // Reciprocal of a double for the saturated RHS.
 //
 // A hardware estimate y0 ~ 1/x (rcp.approx.ftz.f64, roughly 20 correct bits) is refined by
@@ -137,6 +147,11 @@ __device__ __forceinline__ T stage_consts_read(const double* buf) {
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
     unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem_src) : "memory");
+}
+// The same, or eight zero bytes if !copy (gmem_src is then not read, but must be a valid address).
+__device__ __forceinline__ void cp_async8_or_zero(void* smem_dst, const void* gmem_src, bool copy) {
+    unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem_src), "r"(copy ? 8 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }

@@ -1,0 +1,434 @@
+// March of the saturated star stencil in block-scaled fixed point (fixed.cuh).
+//
+//   out(p) = a(p) * (C0 u(p) + sum_d sum_o c[d][o] (u(p+o e_d) + u(p-o e_d)))
+//
+// With the same four weights on every axis the 24 neighbours are first summed per distance and
+// five products remain; with distinct weights the 12 symmetric pairs are summed and 13 remain.
+// The weights are 59- or 60-bit integers with W0 = -(sum of the others), so a common offset of all
+// inputs (the bias, which keeps the integers unsigned) drops out of the sum exactly.
+//
+// Measured on GB300, 384^3, 32 x 8 tiles, tensor copies: 2388 us in FP64 (26 operations per point, 98 % of
+// the FP64 pipe) -> 628 us; 768^3 with distinct weights per axis 19.0 -> 6.65 ms. Error against
+// 64 bits (2-norm): uniform values 3.1e-16 -> 8.1e-17, a smooth wave 5.8e-15 -> 9.6e-17. What bounds it
+// now: about 250 instructions per point (130 on the ALU pipe, 70 on the FMA pipe) issued at half of
+// the peak rate, 16 warps per SM at 128 registers waiting on each other's results; launch bounds for
+// more warps spill and run 1.1 to 2 times longer. The 2 FP64 additions and one multiplication left
+// per point take a third of the FP64 pipe, memory 1.4 GB at a third of its rate.
+#pragma once
+
+#include "acs_internal.cuh"
+#include "fixed.cuh"
+#include "tma.cuh"
+
+namespace acs {
+
+// Inputs smaller than 2^-10 of the segment's scale (u(p) and its +x and +y neighbours, all
+// three) send the point to the FP64 form.
+constexpr u32 kStarBiasHi = 1u << 28;            // 2^60: the offset that keeps inputs unsigned
+constexpr u32 kStarSmallHi = 1u << 18;           // 2^50: the small-value bound
+constexpr int kStarIsoLB = 29, kStarGenLB = 28;  // bits of Wl (see StarFix)
+
+// The sum at one point in FP64, from global memory: the saturated form's operations in their order.
+static __device__ __noinline__ double star_point(const double* __restrict__ p, i64 isy, i64 isz, const StarCoef& cf) {
+    double t = cf.c0 * __ldg(p);
+#pragma unroll
+    for (int o = 1; o <= 4; ++o) t = fma(cf.c[o - 1], __ldg(p + o) + __ldg(p - o), t);
+#pragma unroll
+    for (int o = 1; o <= 4; ++o) t = fma(cf.c[4 + o - 1], __ldg(p + o * isy) + __ldg(p - o * isy), t);
+#pragma unroll
+    for (int o = 1; o <= 4; ++o) t = fma(cf.c[8 + o - 1], __ldg(p + o * isz) + __ldg(p - o * isz), t);
+    return t;
+}
+
+// A tile of BX x BY points; a thread owns two neighbours along x (16-byte shared loads) and takes two
+// planes per iteration. Eight ring slots: the planes kk .. kk+5 in fixed point, and kk+6, kk+7, which
+// are on their way from memory while planes kk and kk+1 are computed and converted in place after that.
+// The four planes below kk sit in registers.
+template <int BX, int BY>
+struct StarFixShape {
+    static constexpr int PX = BX + 8, PY = BY + 8, PLANE = PX * PY;
+    static constexpr int NT = BX * BY / 2;
+    static constexpr int NE = (PLANE + NT - 1) / NT;   // plane cells staged per thread
+    static constexpr int NSLOT = 8;
+    static constexpr int LIST = 4 * NT;   // points of one iteration
+    // Ring, one mbarrier per slot, two shared words, the list, and 128 bytes to align the ring.
+    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * PLANE + NSLOT + 1) + sizeof(u32) * LIST + 128;
+    static_assert((PLANE * sizeof(u64)) % 128 == 0, "every ring slot 128-byte aligned");
+};
+
+template <int BX, int BY, bool TMA, bool ISO>
+struct StarFixMarch {
+    using S = StarFixShape<BX, BY>;
+    static constexpr int PX = S::PX, PLANE = S::PLANE, NE = S::NE, NT = S::NT;
+
+    const double* __restrict__ u;
+    const double* __restrict__ a;
+    double* __restrict__ out;
+    const Geom& g;
+    const StarCoef& cf;
+    const StarFix& fx;
+    int i0, j0, k1;
+    u64* ring;
+    u64* bars;
+    u32* note;   // shared: [0] largest exponent word, [1] length of the list
+    u32* list;   // shared: points that are evaluated in FP64 at the segment's end
+    const CUtensorMap* map;
+    unsigned* tmo;
+    int tid, w, h, tx, ty;
+
+    __device__ __forceinline__ bool valid(int c) const { return ty < h && tx + c < w; }
+
+    // FP64 for the planes [k0, k1).
+    __device__ __forceinline__ void plain(int k0) const {
+        for (int kk = k0; kk < k1; ++kk)
+#pragma unroll 1
+            for (int c = 0; c < 2; ++c) {
+                if (!valid(c)) continue;
+                const i64 at = (i64)(kk + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + c + g.halo);
+                out[(i64)kk * g.osz + (i64)(j0 + ty) * g.osy + i0 + tx + c] =
+                    __ldg(a + at) * star_point(u + at, g.isy, g.isz, cf);
+            }
+    }
+
+    // Stages plane q (raw values) into its slot: one tensor copy, or this thread's cells with
+    // cp.async (zeros for the cells no point reads).
+    __device__ __forceinline__ void stage(int q, int slot, const u32 (&off)[NE], u32 keep, u32& flying) const {
+        u64* dst = ring + slot * PLANE;
+        if (TMA) {
+            flying |= 1u << slot;
+            if (tid == 0) {
+                fence_proxy_async();
+                uint64_t* bar = reinterpret_cast<uint64_t*>(bars + slot);
+                mbar_arrive_expect_tx(bar, PLANE * sizeof(u64));
+                tma_load_3d(dst, map, bar, i0 - 4 + g.halo, j0 - 4 + g.halo, q + g.halo);
+            }
+        } else {
+            const double* base = u + (i64)(q + g.halo) * g.isz + (i64)(j0 - 4 + g.halo) * g.isy + (i0 - 4 + g.halo);
+#pragma unroll
+            for (int n = 0; n < NE; ++n)
+                if (NE * NT == PLANE || n + 1 < NE || tid + n * NT < PLANE)
+                    cp_async8_or_zero(dst + tid + n * NT, base + off[n], (keep >> n) & 1u);
+            cp_async_commit();
+        }
+    }
+
+    // Marches from plane k0 at one scale; returns the first plane it did not finish.
+    // `phase`: the parity of each slot's next tensor copy (one bit per slot; every thread waits
+    // for every copy once); `flying`: the slots with a copy not waited for yet. `ok` turns false when a
+    // wait runs out.
+    __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
+        // The cells of a plane that some point reads: a caller may leave the others (corners of the
+        // halo) unset. On planes past the segment's end only the columns themselves are read.
+        u32 full = 0, core = 0, off[NE];
+#pragma unroll
+        for (int n = 0; n < NE; ++n) {
+            const int e = tid + n * NT;
+            const int yy = e / PX, xx = e - yy * PX;
+            const bool xin = xx >= 4 && xx < w + 4, yin = yy >= 4 && yy < h + 4;
+            const bool in = xx < w + 8 && yy < h + 8 && e < PLANE && (xin || yin);
+            off[n] = in ? (u32)(yy * (int)g.isy + xx) : 0u;
+            if (in) full |= 1u << n;
+            if (xin && yin) core |= 1u << n;
+        }
+        // Tensor copies bring every cell: only tiles at the grid's rim drop the ones not read.
+        const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 4 > g.nx || j0 + BY + 4 > g.ny);
+        if (TMA && !rim) full = ~0u;
+        auto keep = [&](int q) { return q < k1 ? full : core; };
+        const bool work = ty < h;
+        const u32 rs = smem_addr(ring), mine = rs + ((ty + 4) * PX + tx + 4) * 8;
+        const double* col0 = u + (i64)(k0 + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + g.halo);
+        auto below = [&](int q, int c) {   // the column's value q planes below k0
+            return valid(c) ? (u64)__double_as_longlong(__ldg(col0 - q * g.isz + c)) : 0ull;
+        };
+        auto cells = [&](int slot, auto&& f) {   // f(bit, cell) over this thread's cells of a slot
+            const u32 c = rs + (slot * PLANE + tid) * 8;
+#pragma unroll
+            for (int n = 0; n < NE; ++n)
+                if (NE * NT == PLANE || n + 1 < NE || tid + n * NT < PLANE) {
+                    u64 v = lds1(c + 8 * n * NT);
+                    f(n, v);
+                    sts1(c + 8 * n * NT, v);
+                }
+        };
+        auto landed = [&](int slot) {
+            if (!TMA || !ok) return;
+            ok = mbar_wait_bounded(reinterpret_cast<uint64_t*>(bars + slot), (phase >> slot) & 1u, tmo);
+            if (ok) phase ^= 1u << slot, flying &= ~(1u << slot);
+        };
+
+        // Prologue: planes k0 .. k0+5 under way; the largest exponent in them and in the
+        // column's four values below.
+        int next = k0;   // the next plane to stage
+        for (; next < k0 + 6 && next < k1 + 4; ++next) stage(next, next - k0, off, keep(next), flying);
+        if (tid < 2) note[tid] = 0;
+        u32 top = 0;
+        auto see = [&](u64 v) { top = max(top, (hi32(v) & 0x7fffffffu) | (lo32(v) != 0 ? 1u : 0u)); };
+        u64 past[4][2];   // [distance below - 1][column]
+#pragma unroll
+        for (int q = 1; q <= 4; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                past[q - 1][c] = below(q, c);
+                see(past[q - 1][c]);
+            }
+        if (!TMA) cp_async_wait_all();
+#pragma unroll 1
+        for (int q = 0; q < next - k0; ++q) {
+            landed(q);
+            const u32 m = keep(k0 + q);
+            cells(q, [&](int n, u64& v) {
+                if (!TMA || (m >> n) & 1u) see(v);
+            });
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        __syncthreads();
+        if ((tid & 31) == 0) atomicMax(note, top);
+        __syncthreads();
+        if (!ok) note[0] = 0x7fffffffu;
+        __syncthreads();
+        top = note[0];
+        const bool zero = top == 0;
+        int E0 = (int)(top >> 20);
+        const bool fits = zero || (E0 >= kFixMinExp && E0 <= kFixMaxExp);   // not if a wait ran out, either
+        if (zero) E0 = kFixMinExp;
+        int bad = 0;
+        constexpr u32 bias = kStarBiasHi + kStarSmallHi;
+        // This thread's cells of plane q from raw to fixed point, in place.
+        auto convert = [&](int slot, int q) {
+            if (zero) {
+                const u32 m = keep(q);
+                cells(slot, [&](int n, u64& v) {
+                    if ((v << 1) != 0 && (!TMA || (m >> n) & 1u)) bad = -1;
+                    v = (u64)bias << 32;
+                });
+            } else if (rim || (TMA && q >= k1)) {
+                const u32 m = keep(q);
+                cells(slot, [&](int n, u64& v) { v = to_fixed((m >> n) & 1u ? v : 0ull, E0, bias, bad); });
+            } else {
+                cells(slot, [&](int, u64& v) { v = to_fixed(v, E0, bias, bad); });
+            }
+            if (TMA) fence_proxy_async();
+        };
+        int kk = k0;
+        if (fits) {
+#pragma unroll 1
+            for (int q = 0; q < next - k0; ++q) convert(q, k0 + q);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) past[q][c] = to_fixed(past[q][c], E0, bias, bad);
+        }
+        const FixOut fo = fix_out(E0 - 1023 - 59 + fx.shift, fx.neg != 0);
+        const u32 small = zero ? 0u : 2 * kStarSmallHi;
+        // + 1: the two floors in the joined sum lose half a unit each on average.
+        const u64 round = zero ? 0 : 1;
+        const i64 at0 = (i64)(k0 + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + g.halo);
+        const double* ap = a + at0;
+        double* op = out + (i64)k0 * g.osz + (i64)(j0 + ty) * g.osy + i0 + tx;
+        const bool v0 = valid(0), v1 = valid(1);
+        // Pairs of a and out as 16-byte accesses where their addresses allow it (tx is even).
+        auto even = [](const void* at, i64 sy, i64 sz) { return ((uintptr_t)at & 15) == 0 && ((sy | sz) & 1) == 0; };
+        const bool a16 = even(a + at0 - tx - ty * g.isy, g.isy, g.isz), o16 = even(op - tx - ty * g.osy, g.osy, g.osz);
+        int cur = 0;   // the slot of plane kk
+        __syncthreads();
+#pragma unroll 1
+        for (; fits && kk < k1; kk += 2) {
+            const bool two = kk + 1 < k1;
+            double av[2][2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                av[j][0] = av[j][1] = 0.0;
+                if (j && !two) continue;
+                if (v1 && a16) {
+                    const double2 t = __ldg(reinterpret_cast<const double2*>(ap + j * g.isz));
+                    av[j][0] = t.x;
+                    av[j][1] = t.y;
+                } else if (v0) {
+                    av[j][0] = __ldg(ap + j * g.isz);
+                    if (v1) av[j][1] = __ldg(ap + j * g.isz + 1);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j)   // planes kk+6 and kk+7 into the slots of kk-2 and kk-1
+                if (next + j < k1 + 4) stage(next + j, (cur + 6 + j) & 7, off, keep(next + j), flying);
+            next = min(next + 2, k1 + 4);
+            if (work) {
+                u32 s[6];   // planes kk .. kk+5 at the thread's points
+#pragma unroll
+                for (int j = 0; j < 6; j += 2) {
+                    s[j] = mine + ((cur + j) & 7) * (PLANE * 8);
+                    s[j + 1] = s[j] + PLANE * 8;
+                }
+                u64 here[2][2];
+                u32 least = ~0u;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    u64 row[10];
+#pragma unroll
+                    for (int x = 0; x < 10; x += 2) {
+                        const U64x2 t = lds2(s[j] + (x - 4) * 8);
+                        row[x] = t.x;
+                        row[x + 1] = t.y;
+                    }
+                    here[j][0] = row[4];
+                    here[j][1] = row[5];
+                    FixAcc t[2] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+                    u32 nh[2], nl[2];
+#pragma unroll
+                    for (int o = 1; o <= 4; ++o) {
+                        const U64x2 yp2 = lds2(s[j] + o * PX * 8), ym2 = lds2(s[j] - o * PX * 8);
+                        const U64x2 zp2 = lds2(s[j + o]);
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const u64 xp = row[4 + c + o], xm = row[4 + c - o];
+                            const u64 yp = c ? yp2.y : yp2.x, ym = c ? ym2.y : ym2.x;
+                            const u64 zp = c ? zp2.y : zp2.x;
+                            const u64 zm = o <= j ? here[0][c] : past[o - 1 - j][c];
+                            if (o == 1) {
+                                nh[c] = hi32(row[4 + c]);
+                                nl[c] = lo32(row[4 + c]);
+                                least = min(least, nh[c] ^ kStarBiasHi);
+                            }
+                            if (ISO) {
+                                const u64 sm = (xp + xm + yp) + (ym + zp + zm);
+                                fix_mac(t[c], sm, fx.wh[o], fx.wl[o]);
+                                if (o % 2 == 0) {
+                                    nh[c] += hi32(sm);
+                                    nl[c] += lo32(sm);
+                                }
+                            } else {
+                                const u64 sx = xp + xm, sy = yp + ym, sz = zp + zm;
+                                fix_mac(t[c], sx, fx.wh[o], fx.wl[o]);
+                                fix_mac(t[c], sy, fx.wh[4 + o], fx.wl[4 + o]);
+                                fix_mac(t[c], sz, fx.wh[8 + o], fx.wl[8 + o]);
+                                if (o % 2 == 0) {
+                                    nh[c] += hi32(sx) + hi32(sy) + hi32(sz);
+                                    nl[c] += lo32(sx) + lo32(sy) + lo32(sz);
+                                }
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        fix_mac(t[c], row[4 + c], fx.wh[0], fx.wl[0]);
+                        fix_neg(t[c], nh[c], nl[c]);
+                        constexpr int LB = ISO ? kStarIsoLB : kStarGenLB;
+                        const u64 sum = (t[c].hh << 3) + ((t[c].hl + hi32(t[c].ll)) >> (LB - 3)) +
+                                        (u64)((i64)t[c].lh >> 29) + round;
+av[j][c] *= from_fixed((i64)sum, fo);
+                    }
+                    if (j && !two) continue;
+                    if (v1 && o16) {
+                        *reinterpret_cast<double2*>(op + j * g.osz) = make_double2(av[j][0], av[j][1]);
+                    } else if (v0) {
+                        op[j * g.osz] = av[j][0];
+                        if (v1) op[j * g.osz + 1] = av[j][1];
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    past[3][c] = past[1][c];
+                    past[2][c] = past[0][c];
+                    past[1][c] = here[0][c];
+                    past[0][c] = here[1][c];
+                }
+                if (least < small) {   // a point whose neighbours are small, too, goes on the list
+#pragma unroll 1
+                    for (int p = 0; p < 4; ++p) {
+                        const int j = p >> 1, c = p & 1;
+                        if (!(c ? v1 : v0) || (j && !two)) continue;
+                        const u32 q = mine + (((cur + j) & 7) * PLANE + c) * 8;
+                        if (((hi32(lds1(q)) ^ kStarBiasHi) | (hi32(lds1(q + 8)) ^ kStarBiasHi) |
+                             (hi32(lds1(q + PX * 8)) ^ kStarBiasHi)) >= small)
+                            continue;
+                        const u32 at = atomicAdd(note + 1, 1u);
+                        if (at < (u32)S::LIST)
+                            list[at] = ((u32)(kk + j - k0) * BY + ty) * BX + tx + c;
+                        else
+                            bad = -1;
+                    }
+                }
+            }
+            // Planes kk+6 and kk+7 to fixed point (read from the next iteration on).
+            if (!TMA) cp_async_wait_all();
+#pragma unroll 1
+            for (int j = 6; j < 8; ++j)
+                if (kk + j < k1 + 4) {
+                    landed((cur + j) & 7);
+                    convert((cur + j) & 7, kk + j);
+                }
+            if (!ok) bad = -1;
+            ap += 2 * g.isz;
+            op += 2 * g.osz;
+            cur = (cur + 2) & 7;
+            if (__syncthreads_or(bad < 0)) {
+                if (note[1] <= (u32)S::LIST) kk += 2;   // else these two planes are done again
+                break;
+            }
+        }
+        kk = min(kk, k1);
+        // The listed points (of finished planes), by all threads.
+        __syncthreads();
+        const u32 listed = min(note[1], (u32)S::LIST);
+        for (u32 n = tid; n < listed; n += NT) {
+            const int x = list[n] % BX, y = list[n] / BX % BY, q = k0 + (int)(list[n] / (BX * BY));
+            if (q >= kk) continue;
+            const i64 at = (i64)(q + g.halo) * g.isz + (i64)(j0 + y + g.halo) * g.isy + (i0 + x + g.halo);
+            out[(i64)q * g.osz + (i64)(j0 + y) * g.osy + i0 + x] = __ldg(a + at) * star_point(u + at, g.isy, g.isz, cf);
+        }
+        return kk;
+    }
+};
+
+// One block's work: the BX x BY column tile at (i0, j0), z-planes [k0, k1). Ends with all threads
+// past a barrier after their last shared-memory read. A segment that meets a value beyond its scale
+// (or too many points below it) ends early and the next one starts with a scale of its own;
+// after several short ones the rest of the planes is evaluated in FP64.
+template <int BX, int BY, bool TMA, bool ISO>
+__device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, const double* __restrict__ a,
+                                                 double* __restrict__ out, const Geom& g, const StarCoef& cf,
+                                                 const StarFix& fx, int i0, int j0, int k0, int k1, double* smem,
+                                                 const CUtensorMap* map, unsigned* tmo) {
+    using S = StarFixShape<BX, BY>;
+    const int tid = threadIdx.x;
+    // A tile cut by the grid's x edge packs its column pairs into the first threads (see star_march).
+    const int w = min(BX, g.nx - i0), h = min(BY, g.ny - j0), wp = (w + 1) / 2;
+    u64* ring = reinterpret_cast<u64*>(align128(smem));
+    u64* bars = ring + S::NSLOT * S::PLANE;
+    const StarFixMarch<BX, BY, TMA, ISO> m{u,    a,   out, g,   cf,  fx, i0, j0, k1, ring,
+                                           bars, reinterpret_cast<u32*>(bars + S::NSLOT), reinterpret_cast<u32*>(bars + S::NSLOT + 1), map, tmo, tid, w, h,
+                                           2 * (w == BX ? tid % (BX / 2) : tid % wp),
+                                           w == BX ? tid / (BX / 2) : tid / wp};
+    if (TMA) {
+        if (tid == 0) {
+            for (int s = 0; s < S::NSLOT; ++s) mbar_init(reinterpret_cast<uint64_t*>(bars + s), 1);
+            fence_mbar_init();
+        }
+        __syncthreads();
+    }
+    u32 phase = 0, flying = 0;
+    bool ok = true;
+    int kk = k0;
+    for (int left = 4; kk < k1; --left) {
+        const int done = m.segment(kk, phase, flying, ok);
+        __syncthreads();   // the ring and the notes are free again
+        left += (done - kk) / 16;
+        if (done == kk || left <= 0 || !ok) {
+            m.plain(done);
+            break;
+        }
+        kk = done;
+    }
+    if (TMA) {
+        // Copies may still be in flight after a wait that ran out: one more bounded wait each.
+        if (tid == 0 && !ok)
+            for (int s = 0; s < S::NSLOT; ++s)
+                if ((flying >> s) & 1u) mbar_wait_bounded(reinterpret_cast<uint64_t*>(bars + s), (phase >> s) & 1u, tmo);
+        __syncthreads();
+        if (tid == 0)
+            for (int s = 0; s < S::NSLOT; ++s) mbar_inval(reinterpret_cast<uint64_t*>(bars + s));
+        __syncthreads();
+    }
+}
+
+}  // namespace acs

@@ -145,6 +145,9 @@ acs_status launch_stencil_plain(const double* u, const double* a, double* out, c
 
 acs_status launch_stencil_saturated(const double* u, const double* a, double* out, const Geom& g, const StarCoef& c,
                                     const acs_tile& t, cudaStream_t s) {
+    StarFix fx;
+    star_fix(c, fx);
+    if (fx.kind && g.isy < (1 << 22)) return launch_star_fixed(u, a, out, g, c, fx, t, s);
     if (t.bx == 32 && t.by == 8) return launch_star_t<32, 8>(u, a, out, g, c, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 4) return launch_star_t<32, 4>(u, a, out, g, c, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 16) return launch_star_t<32, 16>(u, a, out, g, c, t.kchunk, t.flags, s);
