@@ -35,6 +35,12 @@ acs_status ensure_smem(const void* fn, size_t bytes);
 acs_status launch_rhs_plain(const double* U, double* R, const Geom& g, const RhsConst& k, cudaStream_t s);
 acs_status launch_rhs_saturated(const double* U, double* R, const Geom& g, const RhsConst& k,
                                 const acs_tile& t, cudaStream_t s);
+// The RHS in fixed point (rhs_fixed.cuh): its constants (kc: kf with |s_d|), and the launch.
+void rhs_fix(const RhsConst& kf, RhsFix& fx, RhsConst& kc);
+acs_status launch_rhs_fixed(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+                            const RhsFix& fx, const acs_tile& t, cudaStream_t s);
+acs_status launch_rhs_fixed_gen(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+                                const RhsFix& fx, const acs_tile& t, cudaStream_t s);
 acs_status launch_rhs_ladder(const double* U, double* R, const Geom& g, const RhsConst& k, int form, cudaStream_t s);
 size_t rhs_host_ws_bytes(const Geom& g, int slab);
 acs_status rhs_host_run(const double* U, double* R, const Geom& g, const RhsConst& k, const acs_tile& t, int slab,

@@ -57,6 +57,42 @@ __device__ __forceinline__ void balanced_segments(const BalancedPlan& s, int b, 
     }
 }
 
+// The same segments one at a time (the march is then compiled once, not at each of the three calls).
+struct BalancedWalk {
+    int n;        // segments given so far
+    i64 L, L1;    // the share of the tops still to do
+};
+__device__ __forceinline__ bool balanced_next(const BalancedPlan& s, int b, BalancedWalk& w, i64& col, int& z0, int& z1) {
+    const int n = w.n++;
+    if (n < s.f) {
+        col = (i64)n * s.G + b;
+        z0 = 0;
+        z1 = s.Z;
+        return true;
+    }
+    if (s.R == 0) return false;
+    const i64 c0 = (i64)s.f * s.G;
+    if (b < s.R) {
+        col = c0 + b;
+        z0 = 0;
+        z1 = s.P;
+        return n == s.f && s.P > 0;
+    }
+    const int H = s.Z - s.P, T = s.G - s.R, t = b - s.R;
+    if (n == s.f) {
+        w.L = (i64)s.R * H * t / T;
+        w.L1 = (i64)s.R * H * (t + 1) / T;
+    }
+    if (w.L >= w.L1) return false;
+    const i64 c = w.L / H;
+    const int a = (int)(w.L - c * H);
+    col = c0 + c;
+    z0 = s.P + a;
+    z1 = s.P + (int)min((i64)H, a + (w.L1 - w.L));
+    w.L += z1 - z0;
+    return true;
+}
+
 // FP64 instruction selection for the saturated kernels. Measured on GB300: an FP64
 // instruction whose operands are two per-thread registers and nothing else from a register
 // (DADD, DMUL, or a DFMA whose third operand is an immediate or a kernel argument) issues at
@@ -95,6 +131,15 @@ struct StarCoef {
     Pipe pp;
 };
 
+// Constants of the fixed-point RHS march (rhs_fixed.cuh): eps and |s_d| as 62-bit integers
+// (h 2^31 + l) 2^(ex - 62), and the magnitudes its rules compare. ok 0: the parameters do not suit.
+struct RhsFix {
+    int eh, el, ex_eps;
+    int sh[3], sl[3], ex_s[3];
+    float g1, smax, smin, eps;
+    int ok;
+};
+
 // The weights as integers for the fixed-point star march (star_fixed.cuh): c = (wh 2^LB + wl) 2^-w
 // with wh signed, index 0 the centre, then one axis (kind 1: the three axes share their weights,
 // LB 29) or three (kind 2, LB 28). The joined sum counts in units of 2^(LB + 29 - w) = 2^shift of
@@ -118,15 +163,18 @@ struct StarFix {
 // Outside [2^-1000, 2^1001) (zero, subnormal, huge, inf, NaN) it falls back to an IEEE
 // division; the test of the exponent is integer work only.
 // `one` is 1.0 (in a register, see Pipe).
-__device__ __forceinline__ double rcp_refined(double x, double one) {
-    const int hi = __double2hiint(x);
-    const int bexp = (hi >> 20) & 0x7ff;
-    if (bexp < 23 || bexp > 2023) return 1.0 / x;
+__device__ __forceinline__ double rcp_inside(double x, double one) {   // |x| in [2^-1000, 2^1001)
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     double e = fma(-x, y, one);
     e = fma(e, e, e);
     return fma(y, e, y);
+}
+__device__ __forceinline__ double rcp_refined(double x, double one) {
+    const int hi = __double2hiint(x);
+    const int bexp = (hi >> 20) & 0x7ff;
+    if (bexp < 23 || bexp > 2023) return 1.0 / x;
+    return rcp_inside(x, one);
 }
 
 // Copies a struct of doubles (kernel-argument constants) through shared memory into

@@ -50,6 +50,17 @@ __device__ __forceinline__ u64 lds1(u32 addr) {
     return r;
 }
 
+__device__ __forceinline__ int lds_int(u32 addr) {
+    int r;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(r) : "r"(addr) : "memory");
+    return r;
+}
+__device__ __forceinline__ int4 lds_int4(u32 addr) {
+    int4 r;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr) : "memory");
+    return r;
+}
+
 __device__ __forceinline__ u64 pack64(u32 hi, u32 lo) { return ((u64)hi << 32) | lo; }
 __device__ __forceinline__ u32 hi32(u64 v) { return (u32)(v >> 32); }
 __device__ __forceinline__ u32 lo32(u64 v) { return (u32)v; }

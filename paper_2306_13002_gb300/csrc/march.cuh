@@ -51,11 +51,11 @@ __host__ __device__ inline bool rhs_isotropic(const RhsConst& k) {
     return k.sx == k.sy && k.sy == k.sz && as >= 0x1p-64 && as <= 0x1p64;
 }
 
-template <bool ISO = false>
+template <bool ISO = false, bool INSIDE = false>   // INSIDE: rho known to need no division
 __device__ __forceinline__ void point_flux(double rho, double mx, double my, double mz, double E, const RhsConst& k,
                                            double fx[4], double fy[4], double fz[4]) {
     const Pipe& q = k.pp;
-    const double r0 = rcp_refined(rho, q.one);
+    const double r0 = INSIDE ? rcp_inside(rho, q.one) : rcp_refined(rho, q.one);
     const double r = ISO ? pmul(r0, k.sx, q) : r0;
     const double vx = pmul(mx, r, q), vy = pmul(my, r, q), vz = pmul(mz, r, q);
     const double mxvx = pmul(mx, vx, q);

@@ -1,0 +1,478 @@
+// March of the saturated RHS in block-scaled fixed point (fixed.cuh): the fluxes of a point are computed
+// in FP64 as before (point_flux), everything that adds neighbours runs on the integer pipes.
+//
+//   R_c = -( sum of the flux differences + eps (S2 - 4 S1 + 18 U_c) )
+//
+// Of the 114 FP64 operations of a point (equal spacing) 23 remain; the 91 that difference fluxes and
+// form the dissipation are sums of at most 13 terms with small whole weights, exact in 64-bit
+// integers. The scale of the fluxes (|s| = 1/(2h)) is folded in where they are formed, for unequal
+// spacing as well (30 operations).
+//
+// Scales: one exponent each for rho, the momenta and E, from the first planes of a segment, with
+// the ranges of rho and E below them (they enter the bounds of the fluxes, and a point's own values
+// must not lose their low bits); the fluxes' scales follow from these bounds. A plane that leaves
+// the ranges ends the segment.
+#pragma once
+
+#include "fixed.cuh"
+#include "march.cuh"
+
+namespace acs {
+
+// t * 2^e2 rounded to FP64 (half away from zero) with its sign flipped, on the integer pipes. No
+// branches here or in the flux: the five components' chains interleave.
+__device__ __forceinline__ double minus_from_fixed(i64 t, int e2) {
+    const u32 sg = (u32)((int)hi32((u64)t) >> 31);
+    const u64 m = ((u64)t ^ pack64(sg, sg)) + (sg & 1u);
+    const bool low = hi32(m) == 0;
+    const u32 mh = low ? lo32(m) : hi32(m), ml = low ? 0u : lo32(m);
+    // exponent field of a value with bit 63 (low: 31) set, less the hidden bit
+    const int top = (low ? 1023 + 31 - 1 : 1023 + 63 - 1) + e2;
+    const int lz = __clz((int)mh);
+    const u32 nh = __funnelshift_l(ml, mh, lz), nl = ml << (lz & 31);
+    const u64 r = pack64((nh >> 11) + ((u32)(top - lz) << 20), __funnelshift_r(nl, nh, 11)) + ((nl >> 10) & 1u);
+    return mh == 0 ? 0.0 : __hiloint2double((int)(hi32(r) | (~sg & 0x80000000u)), (int)lo32(r));
+}
+
+// floor-like d * w / 2^63 for w = wh 2^31 + wl, both parts below 2^31 (error below two units).
+__device__ __forceinline__ i64 mul63(i64 d, int wh, int wl) {
+    const int dh = (int)hi32((u64)d);
+    const u32 dl = lo32((u64)d);
+    return (i64)dh * wh + (((i64)dh * wl) >> 31) + (i64)(((u64)dl * (u32)wh) >> 32);
+}
+
+// Fluxes of a point scaled by |s_d| per axis (unequal spacing), otherwise as point_flux.
+__device__ __forceinline__ void point_flux_scaled(double rho, double mx, double my, double mz, double E,
+                                                  const RhsConst& k, double fx[4], double fy[4], double fz[4]) {
+    const Pipe& q = k.pp;
+    const double r = rcp_inside(rho, q.one);
+    const double vx = pmul(mx, r, q), vy = pmul(my, r, q), vz = pmul(mz, r, q);
+    const double twoKE = fma(mz, vz, fma(my, vy, pmul(mx, vx, q)));
+    const double P = fma(k.nhg1, twoKE, pmul(k.g1, E, q)), EP = padd(E, P, q);
+    const double ax = pmul(vx, k.sx, q), ay = pmul(vy, k.sy, q), az = pmul(vz, k.sz, q);
+    fx[0] = fma(mx, ax, pmul(P, k.sx, q));
+    fx[1] = pmul(my, ax, q);
+    fx[2] = pmul(mz, ax, q);
+    fx[3] = pmul(EP, ax, q);
+    fy[0] = pmul(mx, ay, q);
+    fy[1] = fma(my, ay, pmul(P, k.sy, q));
+    fy[2] = pmul(mz, ay, q);
+    fy[3] = pmul(EP, ay, q);
+    fz[0] = pmul(mx, az, q);
+    fz[1] = pmul(my, az, q);
+    fz[2] = fma(mz, az, pmul(P, k.sz, q));
+    fz[3] = pmul(EP, az, q);
+}
+
+// Six ring slots of U (raw as they land, fixed point once their fluxes are formed), the x and y
+// fluxes of one plane, constants, mbarriers and the scan's results.
+template <int BX, int BY>
+struct RhsFixShape {
+    static constexpr int PX = BX + 4, PY = BY + 4, PLANE = PX * PY, CELLS = 5 * PLANE;
+    static constexpr int NT = BX * BY, NSLOT = 6;
+    static constexpr int NE = (CELLS + NT - 1) / NT;
+    static constexpr int FX = 4 * BY * (BX + 2), FY = 4 * (BY + 2) * BX;
+    static constexpr int CONST_ELEMS = 16;
+    // ... constants of the launch, mbarriers, the scan's results, constants of the segment
+    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * CELLS + FX + FY + CONST_ELEMS + NSLOT + 4 + 10);
+    static constexpr int MINB = NT <= 128 ? 4 : 2;
+    static_assert((CELLS * sizeof(u64)) % 128 == 0, "every ring slot 128-byte aligned");
+    static_assert(NT >= 2 * (BX + BY) && (2 * BX) % 32 == 0, "flux ring needs 2(BX+BY) threads, y-ring whole warps");
+    static_assert(sizeof(RhsConst) <= CONST_ELEMS * sizeof(double), "constant staging area");
+    static_assert(BYTES >= RhsShape<BX, BY>::BYTES, "the FP64 march runs in the same shared memory");
+};
+
+// A segment's constants, in shared memory: the march has few registers to spare.
+struct RhsScale {
+    int join[3][4];               // rho, momenta, E: RhsJoin
+    int cu[3], lo[3];             // conversion exponents of U, least exponents (none for the momenta)
+    int cf[2];                    // conversion exponents of the momentum and energy fluxes
+};
+static_assert(sizeof(RhsScale) == 80, "RhsFixShape reserves ten words");
+
+// Shifts and exponent that join a component's flux sum a and dissipation d: z = (a >> sa) + (d >> sd),
+// in units of 2^e.
+struct RhsJoin {
+    int sa, sd, e;
+};
+__device__ __forceinline__ RhsJoin rhs_join(int ea, int ed) {
+    const int e = max(ea, ed) + 1;
+    return RhsJoin{min(e - ea, 63), min(e - ed, 63), e};
+}
+
+template <int BX, int BY, bool TMA, bool ISO>
+struct RhsFixMarch {
+    using S = RhsFixShape<BX, BY>;
+    static constexpr int PX = S::PX, PLANE = S::PLANE, NE = S::NE, NT = S::NT, NSLOT = S::NSLOT;
+
+    const double* __restrict__ U;
+    double* __restrict__ R;
+    const Geom& g;
+    const RhsConst& kc;   // with |s_d| in place of s_d
+    const RhsFix& fx;
+    int i0, j0, k1;
+    double* smem;
+    const CUtensorMap* map;
+    unsigned* tmo;
+
+    __device__ __forceinline__ uint64_t* bar(int slot) const {
+        return reinterpret_cast<uint64_t*>(smem + NSLOT * S::CELLS + S::FX + S::FY + S::CONST_ELEMS) + slot;
+    }
+
+    // Marches from plane k0; returns the first plane not finished. `phase`, `flying`, `ok`: as
+    // StarFixMarch::segment. `room`: bits of headroom for the scales.
+    __device__ __forceinline__ int segment(int k0, int room, u32& phase, u32& flying, bool& ok) const {
+        const int tid = threadIdx.y * BX + threadIdx.x;
+        const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX * 8;
+        int* note = reinterpret_cast<int*>(bar(NSLOT));   // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E
+        // Tiles cut by the grid's edges: points packed as in rhs_march, one halo column more than the
+        // valid ones; rows up to the one past the last valid row.
+        const int w = min(BX, g.nx - i0), h = min(BY, g.ny - j0);
+        const int wf = w < BX ? w + 1 : BX;
+        const int tx = w < BX ? tid % wf : tid % BX, ty = w < BX ? tid / wf : tid / BX;
+        const bool fluxer = ty < BY && ty <= h && (tx < w || ty < h);   // not the corner past both edges
+        const bool active = fluxer && tx < w && ty < h;
+        const u32 own = ((ty + 2) * PX + tx + 2) * 8;
+
+        u32 full = 0, core = 0;
+#pragma unroll
+        for (int n = 0; n < NE; ++n) {
+            const int e = tid + n * NT, r = e % PLANE;
+            const int yy = r / PX, xx = r - yy * PX;
+            const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2;
+            if (xx < w + 4 && yy < h + 4 && e < S::CELLS && (xin || yin)) full |= 1u << n;
+            if (xin && yin && e < S::CELLS) core |= 1u << n;
+        }
+        const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 2 > g.nx || j0 + BY + 2 > g.ny);
+        if (TMA && !rim) full = ~0u;
+        auto keep = [&](int q) { return q >= k0 && q < k1 ? full : core; };
+        auto slot_of = [&](int q) { return (q - k0 + 2) % NSLOT; };
+        auto stage = [&](int q) {
+            const int slot = slot_of(q);
+            if (TMA) {
+                flying |= 1u << slot;
+                if (tid == 0) {
+                    fence_proxy_async();
+                    mbar_arrive_expect_tx(bar(slot), S::CELLS * 8);
+                    tma_load_4d(smem + slot * S::CELLS, map, bar(slot), i0 - 2 + g.halo, j0 - 2 + g.halo, q + g.halo, 0);
+                }
+            } else {
+                const double* base = U + (i64)(q + g.halo) * g.isz + (i64)(j0 - 2 + g.halo) * g.isy + (i0 - 2 + g.halo);
+                const u32 m = keep(q);
+#pragma unroll
+                for (int n = 0; n < NE; ++n) {
+                    const int e = tid + n * NT;
+                    if (e >= S::CELLS) break;
+                    const int c = e / PLANE, r = e % PLANE;
+                    const bool in = (m >> n) & 1u;
+                    cp_async8_or_zero(smem + slot * S::CELLS + e, base + (in ? c * g.isc + (r / PX) * g.isy + r % PX : 0), in);
+                }
+                cp_async_commit();
+            }
+        };
+        auto landed = [&](int slot) {
+            if (!TMA || !ok) return;
+            ok = mbar_wait_bounded(bar(slot), (phase >> slot) & 1u, tmo);
+            if (ok) phase ^= 1u << slot, flying &= ~(1u << slot);
+        };
+        // f(n, cell, kind) over this thread's cells of a slot; kind 0 rho, 1 momentum, 2 E
+        auto kind_of = [&](int n) {
+            const int e = tid + n * NT;
+            return (n + 1) * NT <= PLANE ? 0 : n * NT >= PLANE && (n + 1) * NT <= 4 * PLANE ? 1 : n * NT >= 4 * PLANE ? 2
+                   : e < PLANE ? 0 : e < 4 * PLANE ? 1 : 2;
+        };
+
+        // Prologue: the first six planes under way; exponent ranges of the first five.
+        int next = k0 - 2;
+        for (; next < k0 + 4 && next < k1 + 2; ++next) stage(next);
+        if (tid < 5) note[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
+        __syncthreads();
+        int rng[5] = {0, 0x7ff, 0, 0, 0x7ff};
+        if (!TMA) cp_async_wait_all();
+        const int scanned = min(5, next - k0 + 2);
+#pragma unroll 1
+        for (int p = 0; p < scanned; ++p) {
+            landed(p);
+            const u32 m = keep(k0 - 2 + p);
+#pragma unroll
+            for (int n = 0; n < NE; ++n) {
+                if (!((m >> n) & 1u) || tid + n * NT >= S::CELLS) continue;
+                const u64 v = lds1(rs + (p * S::CELLS + tid + n * NT) * 8);
+                const int e = (int)((hi32(v) << 1) >> 21), kd = kind_of(n);
+                if (kd == 0) {
+                    rng[0] = max(rng[0], e);
+                    rng[1] = min(rng[1], e);
+                } else if (kd == 1) {
+                    rng[2] = max(rng[2], e);
+                } else {
+                    rng[3] = max(rng[3], e);
+                    rng[4] = min(rng[4], e);
+                }
+            }
+        }
+#pragma unroll
+        for (int n = 0; n < 5; ++n) {
+            const bool mn = n == 1 || n == 4;
+            const int v = mn ? __reduce_min_sync(0xffffffffu, rng[n]) : __reduce_max_sync(0xffffffffu, rng[n]);
+            if ((tid & 31) == 0) {
+                if (mn)
+                    atomicMin(note + n, v);
+                else
+                    atomicMax(note + n, v);
+            }
+        }
+        if (!ok) note[0] = 0x7ff;
+        __syncthreads();
+        // Exponents: |rho| in [2^rlo, 2^rhi), |m| < 2^mhi, |E| in [2^elo, 2^ehi).
+        const int rhi = note[0] - 1022 + room, rlo = note[1] - 1023 - 1 - room, mhi = max(note[2], 1023 + rlo - 60) - 1022 + room,
+                  ehi = note[3] - 1022 + room, elo = note[4] - 1023 - 1 - room;
+        bool fits = note[0] < 0x7ff && note[2] < 0x7ff && note[3] < 0x7ff && abs(rhi) < 200 && abs(ehi) < 200 &&
+                    abs(mhi) < 200 && rhi - rlo <= 8 + 2 * room && ehi - elo <= 8 + 2 * room;
+        int efm = 0, efe = 0;
+        if (fits) {
+            // Bounds of the fluxes, and whether quantising against them stays below what FP64 rounds
+            // anyway at the least rho and E: the dissipation (eps 18 U 2^-53) for the mass and energy
+            // components, the pressure ((gamma - 1) E 2^-53) for the momenta.
+            const float vmax = ldexpf(1.f, mhi - rlo), mv = ldexpf(vmax, mhi);
+            const float P = fabsf(fx.g1) * (ldexpf(1.f, ehi) + 1.5f * mv);
+            const float bm = (mv + P) * fx.smax * 1.01f, be = (ldexpf(1.f, ehi) + P) * vmax * fx.smax * 1.01f;
+            const float pl = fx.smin * fabsf(fx.g1) * ldexpf(1.f, elo);
+            fits = isfinite(bm) && isfinite(be) && fx.eps * ldexpf(1.f, rlo) >= fx.smax * ldexpf(0x1p-10f, mhi) &&
+                   fx.eps * ldexpf(1.f, elo) >= be * 0x1p-10f && pl >= bm * 0x1p-8f && pl * 0x1p5f >= fx.eps * ldexpf(1.f, mhi);
+            efm = ilogbf(bm) + 1;
+            efe = ilogbf(be) + 1;
+        }
+        if (!fits) {
+            for (int p = scanned; p < next - k0 + 2; ++p) landed(p);
+            return k0;
+        }
+        // Conversion exponents (leading bit at 59; one more bit of room for U, whose dissipation sums
+        // to 12 times its largest value) and the units of the sums.
+        const int cr = rhi + 1023, cm = mhi + 1023, ce = ehi + 1023, cfm = efm + 1022, cfe = efe + 1022;
+        const int ur = rhi - 59, um = mhi - 59, ue = ehi - 59;
+        const int dx = 2 + 1 + fx.ex_eps;   // dissipation / 4, mul63
+        const int es = max(max(fx.ex_s[0], fx.ex_s[1]), fx.ex_s[2]);
+        RhsScale* const scale = reinterpret_cast<RhsScale*>(note + 8);
+        const u32 sc = smem_addr(scale);
+        if (tid == 0) {
+            const RhsJoin j[3] = {rhs_join(um + 1 + es + (ISO ? 0 : 2), ur + dx), rhs_join(efm - 60, um + dx),
+                                  rhs_join(efe - 60, ue + dx)};
+            for (int n = 0; n < 3; ++n) {
+                scale->join[n][0] = j[n].sa;
+                scale->join[n][1] = j[n].sd;
+                scale->join[n][2] = j[n].e;
+                scale->cu[n] = n == 0 ? cr : n == 1 ? cm : ce;
+                scale->lo[n] = n == 0 ? rlo + 1023 : n == 1 ? 0 : elo + 1023;
+            }
+            scale->cf[0] = cfm;
+            scale->cf[1] = cfe;
+        }
+        __syncthreads();
+
+        auto raw = [&](u32 at) { return __longlong_as_double((long long)lds1(at)); };
+        auto flux = [&](u32 at, double* fxv, double* fyv, double* fzv) {
+            const RhsConst k = stage_consts_read<RhsConst>(smem + NSLOT * S::CELLS + S::FX + S::FY);
+            const double rho = raw(at), mx = raw(at + PLANE * 8), my = raw(at + 2 * PLANE * 8), mz = raw(at + 3 * PLANE * 8),
+                         E = raw(at + 4 * PLANE * 8);
+            if (ISO)
+                point_flux<true, true>(rho, mx, my, mz, E, k, fxv, fyv, fzv);
+            else
+                point_flux_scaled(rho, mx, my, mz, E, k, fxv, fyv, fzv);
+        };
+        int bad = 0;
+        auto fixm = [&](double v) { return to_fixed((u64)__double_as_longlong(v), lds_int(sc + 72), 0, bad); };
+        auto fixe = [&](double v) { return to_fixed((u64)__double_as_longlong(v), lds_int(sc + 76), 0, bad); };
+
+        u64 pa[4] = {0, 0, 0, 0}, pb[4] = {0, 0, 0, 0}, fzp[4] = {0, 0, 0, 0};   // flux sums of q-1 and q-2, F_z of q-1
+        int cur = 0;   // slot of plane q
+        int q = k0 - 2;
+        auto back = [&](int d) { return rs + (cur - d < 0 ? cur - d + NSLOT : cur - d) * (S::CELLS * 8); };
+#pragma unroll 1
+        for (; q < k1 + 2; ++q) {
+            const u32 sq = rs + cur * (S::CELLS * 8);
+            if (q >= k0 + 3) {
+                if (!TMA) cp_async_wait_all();
+                landed(cur);
+            }
+            // In element-wise staging other threads' copies are visible after this barrier only.
+            if (!TMA) __syncthreads();
+            bad = 0;
+            const bool zflux = q >= k0 - 1 && q <= k1, xy = q >= k0 && q < k1;
+            u64 ix[4], iy[4], iz[4], rg[4];
+            int rat = -1;   // where this thread's ring fluxes go
+            if (zflux && fluxer) {
+                double a[4], b[4], c[4];
+                flux(sq + own, a, b, c);
+                ix[0] = fixm(a[0]), ix[1] = fixm(a[1]), ix[2] = fixm(a[2]), ix[3] = fixe(a[3]);
+                iy[0] = ISO ? ix[1] : fixm(b[0]), iy[1] = fixm(b[1]), iy[2] = fixm(b[2]), iy[3] = fixe(b[3]);
+                iz[0] = ISO ? ix[2] : fixm(c[0]), iz[1] = ISO ? iy[2] : fixm(c[1]), iz[2] = fixm(c[2]), iz[3] = fixe(c[3]);
+            }
+            if (xy) {
+                if (tid < 2 * BX) {
+                    const int rx = tid >> 1, ry = (tid & 1) ? BY : -1;
+                    if (rx < w && (ry < 0 || h == BY)) {
+                        double a[4], b[4], c[4];
+                        flux(sq + ((ry + 2) * PX + rx + 2) * 8, a, b, c);
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(b[n]) : fixe(b[n]);
+                        rat = (ry + 1) * BX + rx;
+                    }
+                } else if (tid < 2 * (BX + BY)) {
+                    const int t = tid - 2 * BX, ry = t >> 1, rx = (t & 1) ? BX : -1;
+                    if (ry < h && (rx < 0 || w == BX)) {
+                        double a[4], b[4], c[4];
+                        flux(sq + ((ry + 2) * PX + rx + 2) * 8, a, b, c);
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(a[n]) : fixe(a[n]);
+                        rat = ry * (BX + 2) + rx + 1;
+                    }
+                }
+            }
+            __syncthreads();   // plane q's raw values, plane q-1's fluxes and plane q-5 have been read
+            if (next < k1 + 2 && next <= q + 1) stage(next++);
+            if (xy) {
+                if (fluxer) {
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        sts1(fxs + ((n * BY + ty) * (BX + 2) + tx + 1) * 8, ix[n]);
+                        sts1(fys + ((n * (BY + 2) + ty + 1) * BX + tx) * 8, iy[n]);
+                    }
+                }
+                if (rat >= 0) {
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+                        sts1(tid < 2 * BX ? fys + (n * (BY + 2) * BX + rat) * 8 : fxs + (n * BY * (BX + 2) + rat) * 8, rg[n]);
+                }
+            }
+            {   // plane q to fixed point, in place
+                const u32 m = rim || !TMA || !xy ? keep(q) : ~0u;
+                u64 v[NE];
+#pragma unroll
+                for (int n = 0; n < NE; ++n)
+                    v[n] = (n + 1) * NT <= S::CELLS || tid + n * NT < S::CELLS ? lds1(sq + (tid + n * NT) * 8) : 0ull;
+                if (m != ~0u) {
+#pragma unroll
+                    for (int n = 0; n < NE; ++n) {   // cells no point reads: a value in range
+                        const int kd = kind_of(n);
+                        if (!((m >> n) & 1u)) v[n] = kd == 1 ? 0ull : (u64)(u32)lds_int(sc + 60 + 4 * kd) << 52;
+                    }
+                }
+#pragma unroll
+                for (int n = 0; n < NE; ++n) {
+                    const int kd = kind_of(n);
+                    const int cu = lds_int(sc + 48 + 4 * kd);
+                    if ((n + 1) * NT <= S::CELLS || tid + n * NT < S::CELLS) {
+                        if ((n + 1) * NT > 4 * PLANE || n * NT < PLANE)
+                            bad |= (int)((hi32(v[n]) << 1) >> 21) - lds_int(sc + 60 + 4 * kd);
+                        sts1(sq + (tid + n * NT) * 8, to_fixed(v[n], cu, 0, bad));
+                    }
+                }
+                if (TMA) fence_proxy_async();
+            }
+            if (!ok) bad = -1;
+            // Plane q in fixed point, its fluxes; a value out of range ends the segment before it is used.
+            if (__syncthreads_or(bad < 0)) break;
+            const int kk = q - 2;
+            if (active) {
+                u64 pc[4] = {0, 0, 0, 0};
+                if (xy) {
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const u32 xr = fxs + ((n * BY + ty) * (BX + 2) + tx) * 8, yr = fys + (n * (BY + 2) + ty) * BX * 8 + tx * 8;
+                        pc[n] = (lds1(xr + 16) - lds1(xr)) + (lds1(yr + 2 * BX * 8) - lds1(yr)) - fzp[n];
+                    }
+                }
+                if (kk >= k0) {
+                    const u32 s0 = back(2) + own, sm1 = back(3) + own, sm2 = back(4) + own, sp1 = back(1) + own, sp2 = sq + own;
+                    double* Rp = R + (i64)kk * g.osz + (i64)(j0 + ty) * g.osy + (i0 + tx);
+                    i64 z[5];
+                    int ze[5];
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) {
+                        constexpr int C = PLANE * 8;
+                        const u64 mid = lds1(s0 + c * C);
+                        const u64 s2 = (lds1(s0 + c * C - 16) + lds1(s0 + c * C + 16) + lds1(s0 + c * C - 16 * PX)) +
+                                       (lds1(s0 + c * C + 16 * PX) + lds1(sm2 + c * C) + lds1(sp2 + c * C));
+                        const u64 s1 = (lds1(s0 + c * C - 8) + lds1(s0 + c * C + 8) + lds1(s0 + c * C - 8 * PX)) +
+                                       (lds1(s0 + c * C + 8 * PX) + lds1(sm1 + c * C) + lds1(sp1 + c * C));
+                        const u64 d4 = (u64)((i64)s2 >> 2) - s1 + (mid << 2) + (u64)((i64)mid >> 1);
+                        const i64 ds = mul63((i64)d4, fx.eh, fx.el);
+                        i64 a;
+                        if (c == 0) {
+                            const u64 ax = lds1(s0 + C + 8) - lds1(s0 + C - 8), ay = lds1(s0 + 2 * C + 8 * PX) - lds1(s0 + 2 * C - 8 * PX),
+                                      az = lds1(sp1 + 3 * C) - lds1(sm1 + 3 * C);
+                            if (ISO)
+                                a = mul63((i64)(ax + ay + az), fx.sh[0], fx.sl[0]);
+                            else
+                                a = (mul63((i64)ax, fx.sh[0], fx.sl[0]) >> min(es - fx.ex_s[0] + 2, 63)) +
+                                    (mul63((i64)ay, fx.sh[1], fx.sl[1]) >> min(es - fx.ex_s[1] + 2, 63)) +
+                                    (mul63((i64)az, fx.sh[2], fx.sl[2]) >> min(es - fx.ex_s[2] + 2, 63));
+                        } else {
+                            a = (i64)pb[c - 1];
+                        }
+                        const int4 j = lds_int4(sc + (c == 0 ? 0 : c == 4 ? 32 : 16));
+                        z[c] = (a >> j.x) + (ds >> j.y);
+                        ze[c] = j.z;
+                    }
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
+                }
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    pb[n] = pa[n] + (zflux ? iz[n] : 0);
+                    pa[n] = pc[n];
+                    if (zflux) fzp[n] = iz[n];
+                }
+            }
+            cur = cur + 1 == NSLOT ? 0 : cur + 1;
+        }
+        // Copies not waited for yet: planes after q that a segment cut short had under way.
+        for (int p = max(q + 1, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
+        if (!TMA) cp_async_wait_all();
+        return min(max(q - 2, k0), k1);
+    }
+};
+
+// One block's work: the BX x BY column tile at (i0, j0), z-planes [k0, k1). Ends with all threads past
+// a barrier after their last shared-memory access. The planes of segments that do not fit run in the
+// FP64 march.
+template <int BX, int BY, bool TMA, bool ISO>
+__device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, double* __restrict__ R, const Geom& g,
+                                                const RhsConst& kf, const RhsConst& kc, const RhsFix& fx, int i0, int j0,
+                                                int k0, int k1, double* smem, const CUtensorMap* map, unsigned* tmo) {
+    using S = RhsFixShape<BX, BY>;
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    const RhsFixMarch<BX, BY, TMA, ISO> m{U, R, g, kc, fx, i0, j0, k1, smem, map, tmo};
+    stage_consts_write(smem + S::NSLOT * S::CELLS + S::FX + S::FY, kc, tid);
+    if (TMA && tid == 0) {
+        for (int s = 0; s < S::NSLOT; ++s) mbar_init(m.bar(s), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    u32 phase = 0, flying = 0;
+    bool ok = !TMA || (smem_addr(smem) & 127u) == 0;
+    int kk = k0;
+    for (int left = 4, room = 0; kk < k1 && ok; --left, room = 1) {
+        const int done = m.segment(kk, room, phase, flying, ok);
+        __syncthreads();   // shared memory is free again
+        left += (done - kk) / 16;
+        const bool stop = done == kk || left <= 0;
+        kk = done;
+        if (stop) break;
+    }
+    if (TMA) {
+        if (tid == 0 && !ok)
+            for (int s = 0; s < S::NSLOT; ++s)
+                if ((flying >> s) & 1u) mbar_wait_bounded(m.bar(s), (phase >> s) & 1u, tmo);
+        __syncthreads();
+        if (tid == 0)
+            for (int s = 0; s < S::NSLOT; ++s) mbar_inval(m.bar(s));
+        __syncthreads();
+    }
+    if (kk < k1) {
+        rhs_march<BX, BY, TMA, ISO>(U, R, g, kf, i0, j0, kk, k1, smem, map, tmo);
+        __syncthreads();
+    }
+}
+
+}  // namespace acs

@@ -1,0 +1,89 @@
+// Kernels and launchers of the fixed-point RHS march; rhs_fixed_iso.cu and rhs_fixed_gen.cu each compile
+// one of its two spacing forms.
+#pragma once
+
+#include <cmath>
+#include <cstring>
+
+#include "rhs_fixed.cuh"
+
+namespace acs {
+namespace {
+
+template <int BX, int BY, bool TMA, bool ISO>
+__global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
+    rhs_fixed_kernel(const double* __restrict__ U, double* __restrict__ R, const __grid_constant__ Geom g,
+                     const __grid_constant__ RhsConst kf, const __grid_constant__ RhsConst kc,
+                     const __grid_constant__ RhsFix fx, int kchunk, const __grid_constant__ CUtensorMap map,
+                     unsigned* tmo) {
+    extern __shared__ __align__(128) double smem[];
+    const int k0 = blockIdx.z * kchunk;
+    rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kf, kc, fx, blockIdx.x * BX, blockIdx.y * BY, k0, min(k0 + kchunk, g.nz),
+                                      smem, &map, tmo);
+}
+
+template <int BX, int BY, bool TMA, bool ISO>
+__global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
+    rhs_fixed_balanced_kernel(const double* __restrict__ U, double* __restrict__ R, const __grid_constant__ Geom g,
+                              const __grid_constant__ RhsConst kf, const __grid_constant__ RhsConst kc,
+                              const __grid_constant__ RhsFix fx, const __grid_constant__ BalancedPlan plan,
+                              const __grid_constant__ CUtensorMap map, unsigned* tmo) {
+    extern __shared__ __align__(128) double smem[];
+    BalancedWalk walk{0, 0, 0};
+    i64 col;
+    int z0, z1;
+    while (balanced_next(plan, blockIdx.x, walk, col, z0, z1))
+        rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kf, kc, fx, (int)(col % plan.ntx) * BX, (int)(col / plan.ntx) * BY, z0,
+                                          z1, smem, &map, tmo);
+}
+
+template <int BX, int BY, bool TMA, bool ISO>
+acs_status launch_rhs_fixed_t(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+                              const RhsFix& fx, int kchunk, int flags, const CUtensorMap& map, cudaStream_t s) {
+    using S = RhsFixShape<BX, BY>;
+    unsigned* tmo = wait_timeout_counter();
+    if (!tmo) return fail(ACS_ERR_CUDA, "cannot address the wait-timeout counter");
+    const int ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY;
+    const dim3 block(BX, BY, 1);
+    if (flags & ACS_TILE_BALANCED) {
+        const void* fn = (const void*)rhs_fixed_balanced_kernel<BX, BY, TMA, ISO>;
+        acs_status st = ensure_smem(fn, S::BYTES);
+        if (st != ACS_OK) return st;
+        const i64 C = (i64)ntx * nty;
+        i64 G = resident_blocks(fn, S::NT, S::BYTES);
+        if (G <= 0) return fail(ACS_ERR_CUDA, "occupancy query failed for rhs_fixed_balanced_kernel");
+        if (G > C * g.nz) G = C * g.nz;
+        const BalancedPlan plan = balanced_plan(C, ntx, g.nz, (int)G);
+        rhs_fixed_balanced_kernel<BX, BY, TMA, ISO><<<(unsigned)G, block, S::BYTES, s>>>(U, R, g, kf, kc, fx, plan, map, tmo);
+        return launch_status("rhs_fixed_balanced_kernel");
+    }
+    const void* fn = (const void*)rhs_fixed_kernel<BX, BY, TMA, ISO>;
+    acs_status st = ensure_smem(fn, S::BYTES);
+    if (st != ACS_OK) return st;
+    if (kchunk <= 0) kchunk = default_kchunk(g.nz, (i64)ntx * nty, S::MINB);
+    const dim3 grid(ntx, nty, (g.nz + kchunk - 1) / kchunk);
+    rhs_fixed_kernel<BX, BY, TMA, ISO><<<grid, block, S::BYTES, s>>>(U, R, g, kf, kc, fx, kchunk, map, tmo);
+    return launch_status("rhs_fixed_kernel");
+}
+
+template <int BX, int BY, bool ISO>
+acs_status launch_rhs_fixed_tile(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+                                 const RhsFix& fx, const acs_tile& t, cudaStream_t s) {
+    CUtensorMap map;
+    memset(&map, 0, sizeof(map));
+    if ((t.flags & ACS_TILE_TMA) && encode_plane_map(U, g, 5, BX + 4, BY + 4, &map) == ACS_OK)
+        return launch_rhs_fixed_t<BX, BY, true, ISO>(U, R, g, kf, kc, fx, t.kchunk, t.flags, map, s);
+    return launch_rhs_fixed_t<BX, BY, false, ISO>(U, R, g, kf, kc, fx, t.kchunk, t.flags, map, s);
+}
+
+// The march is built for 16 x 16 and 16 x 8 (larger tiles leave room for one block on an SM): a
+// requested tile of 256 points or more runs as the first, a smaller one as the second.
+template <bool ISO>
+acs_status launch_rhs_fixed_form(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+                                 const RhsFix& fx, const acs_tile& t, cudaStream_t s) {
+    return t.bx * t.by >= 256 ? launch_rhs_fixed_tile<16, 16, ISO>(U, R, g, kf, kc, fx, t, s)
+                              : launch_rhs_fixed_tile<16, 8, ISO>(U, R, g, kf, kc, fx, t, s);
+}
+
+}  // namespace
+}  // namespace acs

@@ -139,6 +139,16 @@ size_t rhs_smem_bytes(int bx, int by) {
 
 acs_status launch_rhs_saturated(const double* U, double* R, const Geom& g, const RhsConst& k, const acs_tile& t,
                                 cudaStream_t s) {
+    RhsFix fx;
+    RhsConst kc;
+    rhs_fix(k, fx, kc);
+    // The fixed-point march starts four planes before its first result (the FP64 march one), so it needs
+    // a few planes per resident block: 64^3 (3.4 planes) 71.6 -> 46.7 us, 48^3 (1.4) 42.6 -> 43.4, 32^3
+    // (0.4) 17.5 -> 22.0. Counted in 16 x 16 columns whatever the tile, so that a grid's results do not
+    // depend on its launch shape.
+    const i64 work = (i64)((g.nx + 15) / 16) * ((g.ny + 15) / 16) * g.nz;
+    if (fx.ok && work >= 4 * (i64)num_sms() && rhs_tile_supported(t.bx, t.by))
+        return launch_rhs_fixed(U, R, g, k, kc, fx, t, s);
     if (t.bx == 32 && t.by == 8) return launch_t<32, 8>(U, R, g, k, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 4) return launch_t<32, 4>(U, R, g, k, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 16) return launch_t<32, 16>(U, R, g, k, t.kchunk, t.flags, s);

@@ -47,10 +47,12 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
                                const __grid_constant__ StarFix fx, const __grid_constant__ BalancedPlan plan,
                                const __grid_constant__ CUtensorMap map, unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
-    balanced_segments(plan, blockIdx.x, [&](i64 col, int z0, int z1) {
+    BalancedWalk walk{0, 0, 0};
+    i64 col;
+    int z0, z1;
+    while (balanced_next(plan, blockIdx.x, walk, col, z0, z1))
         star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, (int)(col % plan.ntx) * BX,
                                           (int)(col / plan.ntx) * BY, z0, z1, smem, &map, tmo);
-    });
 }
 
 template <int BX, int BY, int MINB, bool TMA, bool ISO>

@@ -120,7 +120,9 @@ def test_star_fixed_non_finite_and_unset_corners(tile):
     fine = np.isfinite(ref)
     assert 0 < np.count_nonzero(~fine) < ref.size // 10 and np.array_equal(fine, np.isfinite(got))
     zero = np.where(np.isfinite(u), u, 0.0)
-    assert np.all((np.abs(got - ref) <= 2.0 ** -46 * _star_scale(zero, a, TAYLOR))[fine])
+    with np.errstate(all="ignore"):
+        near = np.abs(got - ref) <= 2.0 ** -46 * _star_scale(zero, a, TAYLOR)
+    assert np.all(near[fine])
 
 
 @pytest.mark.parametrize("tile", [None, (16, 16, 0, 0)])
@@ -136,3 +138,119 @@ def test_star_fixed_non_finite_and_unset_corners(tile):
 def test_star_fixed_weights(c, tile):
     u, a = inputs.stencil_fields(37, 21, 19, seed=91)
     _check_star(u - 0.5, a, np.array(c), tile, "weights")
+
+
+# ------------------------------------------------------------------------------------------ RHS
+
+RHS_TILES = [None, (16, 16, 6, 2), (32, 8, 0, 1), (16, 8, 0, 3), (16, 8, 5, 0)]
+
+
+def _rhs_scale(U, gamma, eps, h):
+    """sum|terms| of every component: fluxes with every addend's magnitude, and the dissipation's."""
+    g1 = abs(gamma - 1.0)
+    A = np.abs(U)
+    with np.errstate(all="ignore"):
+        v = A[1:4] / A[0]
+        P = g1 * (A[4] + 0.5 * (A[1:4] * v).sum(0))
+        F = [np.stack([A[1 + d]] + [A[1 + c] * v[d] + (P if c == d else 0.0) for c in range(3)] + [(A[4] + P) * v[d]])
+             for d in range(3)]
+    inner = (slice(None),) + (slice(2, -2),) * 3
+    tot = np.zeros_like(U[inner])
+    for d in range(3):
+        ax = 3 - d
+
+        def at(x, o):
+            return np.roll(x, -o, axis=ax)[inner]
+
+        tot += (at(F[d], 1) + at(F[d], -1)) / (2 * abs(h[d]))
+        tot += abs(eps) * (at(A, 2) + 4 * at(A, 1) + 6 * at(A, 0) + 4 * at(A, -1) + at(A, -2))
+    return tot
+
+
+def _rhs(U, tile, gamma, eps, h):
+    _, Z, Y, X = U.shape
+    R = torch.full((5, Z - 4, Y - 4, X - 4), float("nan"), dtype=torch.float64, device="cuda")
+    binding.acs_rhs_saturated(to_dev(U), R, gamma, eps, h, tile=tile)
+    torch.cuda.synchronize()
+    return R.cpu().numpy()
+
+
+def _check_rhs(U, tile, what, gamma=1.4, eps=0.25, h=(1.0, 1.0, 1.0)):
+    got, ref = _rhs(U, tile, gamma, eps, h), oracle.rhs(U, gamma=gamma, eps=eps, h=h, threads=8)
+    bad = ~(np.abs(got - ref) <= 2.0 ** -46 * _rhs_scale(U, gamma, eps, h))
+    assert not bad.any(), (what, tile, int(bad.sum()), np.argwhere(bad)[:3], got[bad][:3], ref[bad][:3])
+
+
+def _flow(kind, nx, ny, nz, seed):
+    U = inputs.rhs_field(nx, ny, nz, halo=2, seed=seed)
+    z, y, x = np.meshgrid(*(np.arange(n) for n in U.shape[1:]), indexing="ij")
+    rng = np.random.default_rng(seed)
+    if kind == "shock":             # a jump of 2^12 in density and energy
+        jump = np.where(x + y + z > (nx + ny + nz) // 2, 2.0 ** 12, 1.0)
+        U = U * jump
+    elif kind == "ramp":            # outgrows the scale every other plane
+        U = U * 2.0 ** (0.5 * z)
+    elif kind == "fall":
+        U = U * 2.0 ** (-0.5 * z)
+    elif kind == "rest":
+        U[1:4] = 0.0
+    elif kind == "slow":            # momenta far below the other components
+        U[1:4] *= 2.0 ** -70
+    elif kind == "fast":            # momenta far above
+        U[1:4] *= 2.0 ** 20
+    elif kind == "lumps":
+        U[1:4] *= 2.0 ** rng.integers(-60, 1, U[1:4].shape)
+        U[0] *= 2.0 ** rng.integers(-4, 4, U[0].shape)
+    elif kind == "negative":        # nothing keeps the signs of a state apart
+        U = U * rng.choice([-1.0, 1.0], U.shape)
+    elif kind == "large":
+        U = U * 2.0 ** 150
+    elif kind == "small":
+        U = U * 2.0 ** -190
+    return U
+
+
+@pytest.mark.parametrize("tile", RHS_TILES)
+@pytest.mark.parametrize("kind", ["plain", "shock", "ramp", "fall", "rest", "slow", "fast", "lumps", "negative", "large",
+                                  "small"])
+def test_rhs_fixed_ranges(kind, tile):
+    """Grids large enough for the fixed-point march (two planes per resident block)."""
+    _check_rhs(_flow(kind, 83, 70, 37, 21), tile, kind)
+
+
+@pytest.mark.parametrize("tile", RHS_TILES)
+@pytest.mark.parametrize("prm", [
+    {"gamma": 5.0 / 3.0, "eps": 0.03, "h": (0.37, 0.37, 0.37)}, {"gamma": 1.1, "eps": 0.25, "h": (0.2, 1.0, 3.0)},
+    {"eps": 1e-9}, {"eps": 0.0}, {"eps": -0.25}, {"h": (-1.0, 1.0, 1.0)}, {"gamma": 1.0}, {"gamma": 0.5},
+    {"eps": 40.0}, {"h": (2.0 ** -80,) * 3, "eps": 2.0 ** 78}, {"h": (1e-5, 1.0, 1.0)},
+])
+def test_rhs_fixed_parameters(prm, tile):
+    _check_rhs(_flow("plain", 67, 50, 49, 22), tile, str(prm), **prm)
+
+
+@pytest.mark.parametrize("tile", RHS_TILES)
+@pytest.mark.parametrize("dims", [(17, 16, 400), (31, 33, 160), (64, 48, 60), (1, 1, 700), (15, 90, 120), (160, 2, 70)])
+def test_rhs_fixed_tile_edges(dims, tile):
+    """One, all but one and all columns and rows of the last tile."""
+    _check_rhs(_flow("plain", *dims, 23), tile, dims, h=(1.0, 0.5, 2.0))
+    _check_rhs(_flow("plain", *dims, 24), tile, dims)
+
+
+@pytest.mark.parametrize("tile", RHS_TILES)
+def test_rhs_fixed_non_finite_and_unset_corners(tile):
+    U = _flow("plain", 70, 61, 40, 25)
+    z, y, x = np.meshgrid(*(np.arange(n) for n in U.shape[1:]), indexing="ij")
+    outside = sum(((v < 2) | (v >= n - 2)).astype(int) for v, n in zip((z, y, x), U.shape[1:]))
+    clean = U.copy()
+    U[:, outside >= 2] = np.nan
+    got, ref = _rhs(U, tile, 1.4, 0.25, (1.0,) * 3), oracle.rhs(clean, threads=8)
+    scale = _rhs_scale(clean, 1.4, 0.25, (1.0,) * 3)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -46 * scale)
+    U[0, 20, 30, 33], U[4, 9, 50, 60], U[2, 38, 12, 7] = np.nan, np.inf, -np.inf
+    U[0, 30, 10, 50] = 0.0
+    got, ref = _rhs(U, tile, 1.4, 0.25, (1.0,) * 3), oracle.rhs(U, threads=8)
+    fine = np.isfinite(ref)
+    assert 0 < np.count_nonzero(~fine) < ref.size // 10 and np.array_equal(fine, np.isfinite(got))
+    with np.errstate(all="ignore"):
+        far = np.abs(got - ref) <= 2.0 ** -46 * scale * 4.0   # neighbours of the changed cells have larger terms
+    assert np.all(far[fine & (scale < 30.0)])
