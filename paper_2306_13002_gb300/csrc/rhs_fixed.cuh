@@ -132,7 +132,8 @@ struct RhsFixMarch {
         const int tx = w < BX ? tid % wf : tid % BX, ty = w < BX ? tid / wf : tid / BX;
         const bool fluxer = ty < BY && ty <= h && (tx < w || ty < h);   // not the corner past both edges
         const bool active = fluxer && tx < w && ty < h;
-        const u32 own = ((ty + 2) * PX + tx + 2) * 8;
+        constexpr u32 safe = (2 * PX + 2) * 8;   // the tile's first point
+        const u32 own = ((ty + 2) * PX + tx + 2) * 8, mine = fluxer ? own : safe;
 
         u32 full = 0, core = 0;
 #pragma unroll
@@ -300,32 +301,38 @@ struct RhsFixMarch {
             const bool zflux = q >= k0 - 1 && q <= k1, xy = q >= k0 && q < k1;
             u64 ix[4], iy[4], iz[4], rg[4];
             int rat = -1;   // where this thread's ring fluxes go
-            if (zflux && fluxer) {
+            auto own_flux = [&]() {
                 double a[4], b[4], c[4];
-                flux(sq + own, a, b, c);
+                flux(sq + mine, a, b, c);
                 ix[0] = fixm(a[0]), ix[1] = fixm(a[1]), ix[2] = fixm(a[2]), ix[3] = fixe(a[3]);
                 iy[0] = ISO ? ix[1] : fixm(b[0]), iy[1] = fixm(b[1]), iy[2] = fixm(b[2]), iy[3] = fixe(b[3]);
                 iz[0] = ISO ? ix[2] : fixm(c[0]), iz[1] = ISO ? iy[2] : fixm(c[1]), iz[2] = fixm(c[2]), iz[3] = fixe(c[3]);
-            }
-            if (xy) {
-                if (tid < 2 * BX) {
+            };
+            // The ring's points outside the tile, next to the thread's own (y-ring: rows -1 and BY, the
+            // first 2 BX threads; x-ring: columns -1 and BX, the next 2 BY). Both fluxes in one stretch of
+            // code, so that their chains of FP64 operations overlap: the ring's warps are the ones every
+            // step waits for. Threads without a point take a cell that every tile has.
+            if (zflux) {
+                if (xy && tid < 2 * BX) {
                     const int rx = tid >> 1, ry = (tid & 1) ? BY : -1;
-                    if (rx < w && (ry < 0 || h == BY)) {
-                        double a[4], b[4], c[4];
-                        flux(sq + ((ry + 2) * PX + rx + 2) * 8, a, b, c);
+                    const bool in = rx < w && (ry < 0 || h == BY);
+                    if (in) rat = (ry + 1) * BX + rx;
+                    double a[4], b[4], c[4];
+                    flux(sq + (in ? ((ry + 2) * PX + rx + 2) * 8 : safe), a, b, c);
+                    own_flux();
 #pragma unroll
-                        for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(b[n]) : fixe(b[n]);
-                        rat = (ry + 1) * BX + rx;
-                    }
-                } else if (tid < 2 * (BX + BY)) {
+                    for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(b[n]) : fixe(b[n]);
+                } else if (xy && tid < 2 * (BX + BY)) {
                     const int t = tid - 2 * BX, ry = t >> 1, rx = (t & 1) ? BX : -1;
-                    if (ry < h && (rx < 0 || w == BX)) {
-                        double a[4], b[4], c[4];
-                        flux(sq + ((ry + 2) * PX + rx + 2) * 8, a, b, c);
+                    const bool in = ry < h && (rx < 0 || w == BX);
+                    if (in) rat = ry * (BX + 2) + rx + 1;
+                    double a[4], b[4], c[4];
+                    flux(sq + (in ? ((ry + 2) * PX + rx + 2) * 8 : safe), a, b, c);
+                    own_flux();
 #pragma unroll
-                        for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(a[n]) : fixe(a[n]);
-                        rat = ry * (BX + 2) + rx + 1;
-                    }
+                    for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(a[n]) : fixe(a[n]);
+                } else if (fluxer) {
+                    own_flux();
                 }
             }
             __syncthreads();   // plane q's raw values, plane q-1's fluxes and plane q-5 have been read
