@@ -14,6 +14,8 @@
 // the ranges ends the segment.
 #pragma once
 
+#include <type_traits>
+
 #include "fixed.cuh"
 #include "march.cuh"
 
@@ -285,56 +287,109 @@ struct RhsFixMarch {
         auto fixe = [&](double v) { return to_fixed((u64)__double_as_longlong(v), lds_int(sc + 76), 0, bad); };
 
         u64 pa[4] = {0, 0, 0, 0}, pb[4] = {0, 0, 0, 0}, fzp[4] = {0, 0, 0, 0};   // flux sums of q-1 and q-2, F_z of q-1
+        u64 ix[4], iy[4], iz[4], rg[4];   // fluxes of plane q: the thread's own point, its ring point
         int cur = 0;   // slot of plane q
         int q = k0 - 2;
         auto back = [&](int d) { return rs + (cur - d < 0 ? cur - d + NSLOT : cur - d) * (S::CELLS * 8); };
+        auto z_plane = [&](int p) { return p >= k0 - 1 && p <= k1; };
+        auto xy_plane = [&](int p) { return p >= k0 && p < k1; };
+        // The ring's point outside the tile: rows -1 and BY for the first 2 BX threads, columns -1 and BX
+        // for the next 2 BY. Threads without a point take a cell that every tile has.
+        const int ring = tid < 2 * BX ? 1 : tid < 2 * (BX + BY) ? 2 : 0;
+        int rat = -1;   // where its fluxes go
+        u32 rfrom = safe;
+        if (ring == 1) {
+            const int rx = tid >> 1, ry = (tid & 1) ? BY : -1;
+            if (rx < w && (ry < 0 || h == BY)) {
+                rat = (ry + 1) * BX + rx;
+                rfrom = ((ry + 2) * PX + rx + 2) * 8;
+            }
+        } else if (ring == 2) {
+            const int t = tid - 2 * BX, ry = t >> 1, rx = (t & 1) ? BX : -1;
+            if (ry < h && (rx < 0 || w == BX)) {
+                rat = ry * (BX + 2) + rx + 1;
+                rfrom = ((ry + 2) * PX + rx + 2) * 8;
+            }
+        }
+        // Fluxes of the plane at sn. The ring's and the own one stand in one stretch of code, so that
+        // their chains of FP64 operations overlap: the ring's warps are the ones every step waits for.
+        auto fluxes = [&](u32 sn, auto kind) {
+            constexpr int RING = decltype(kind)::value;
+            double a[4], b[4], c[4], d[4], e[4], f[4];
+            if (RING) flux(sn + rfrom, d, e, f);
+            flux(sn + mine, a, b, c);
+            ix[0] = fixm(a[0]), ix[1] = fixm(a[1]), ix[2] = fixm(a[2]), ix[3] = fixe(a[3]);
+            iy[0] = ISO ? ix[1] : fixm(b[0]), iy[1] = fixm(b[1]), iy[2] = fixm(b[2]), iy[3] = fixe(b[3]);
+            iz[0] = ISO ? ix[2] : fixm(c[0]), iz[1] = ISO ? iy[2] : fixm(c[1]), iz[2] = fixm(c[2]), iz[3] = fixe(c[3]);
+            if (RING)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(RING == 1 ? e[n] : d[n]) : fixe(RING == 1 ? e[n] : d[n]);
+        };
+        // x and y flux differences of plane q; the flux sums move on by one plane.
+        u64 po[4];   // the complete flux sums of plane q-2
+        auto gather = [&](bool xy, bool zflux) {
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                u64 pc = 0;
+                if (xy) {
+                    const u32 xr = fxs + ((n * BY + ty) * (BX + 2) + tx) * 8, yr = fys + (n * (BY + 2) + ty) * BX * 8 + tx * 8;
+                    pc = (lds1(xr + 16) - lds1(xr)) + (lds1(yr + 2 * BX * 8) - lds1(yr)) - fzp[n];
+                }
+                po[n] = pb[n];
+                pb[n] = pa[n] + (zflux ? iz[n] : 0);
+                pa[n] = pc;
+                if (zflux) fzp[n] = iz[n];
+            }
+        };
+        auto emit = [&]() {   // the result at plane q-2
+            const int kk = q - 2;
+            const u32 s0 = back(2) + own, sm1 = back(3) + own, sm2 = back(4) + own, sp1 = back(1) + own, sp2 = back(0) + own;
+            double* Rp = R + (i64)kk * g.osz + (i64)(j0 + ty) * g.osy + (i0 + tx);
+            i64 z[5];
+            int ze[5];
+#pragma unroll
+            for (int c = 0; c < 5; ++c) {
+                constexpr int C = PLANE * 8;
+                const u64 mid = lds1(s0 + c * C);
+                const u64 s2 = (lds1(s0 + c * C - 16) + lds1(s0 + c * C + 16) + lds1(s0 + c * C - 16 * PX)) +
+                               (lds1(s0 + c * C + 16 * PX) + lds1(sm2 + c * C) + lds1(sp2 + c * C));
+                const u64 s1 = (lds1(s0 + c * C - 8) + lds1(s0 + c * C + 8) + lds1(s0 + c * C - 8 * PX)) +
+                               (lds1(s0 + c * C + 8 * PX) + lds1(sm1 + c * C) + lds1(sp1 + c * C));
+                const u64 d4 = (u64)((i64)s2 >> 2) - s1 + (mid << 2) + (u64)((i64)mid >> 1);
+                const i64 ds = mul63((i64)d4, fx.eh, fx.el);
+                i64 a;
+                if (c == 0) {
+                    const u64 ax = lds1(s0 + C + 8) - lds1(s0 + C - 8), ay = lds1(s0 + 2 * C + 8 * PX) - lds1(s0 + 2 * C - 8 * PX),
+                              az = lds1(sp1 + 3 * C) - lds1(sm1 + 3 * C);
+                    if (ISO)
+                        a = mul63((i64)(ax + ay + az), fx.sh[0], fx.sl[0]);
+                    else
+                        a = (mul63((i64)ax, fx.sh[0], fx.sl[0]) >> min(es - fx.ex_s[0] + 2, 63)) +
+                            (mul63((i64)ay, fx.sh[1], fx.sl[1]) >> min(es - fx.ex_s[1] + 2, 63)) +
+                            (mul63((i64)az, fx.sh[2], fx.sl[2]) >> min(es - fx.ex_s[2] + 2, 63));
+                } else {
+                    a = (i64)po[c - 1];
+                }
+                const int4 j = lds_int4(sc + (c == 0 ? 0 : c == 4 ? 32 : 16));
+                z[c] = (a >> j.x) + (ds >> j.y);
+                ze[c] = j.z;
+            }
+#pragma unroll
+            for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
+        };
+        auto arrive = [&](int p, int slot) {   // plane p's raw values are in its slot
+            if (p >= k0 + 3) {
+                if (!TMA) cp_async_wait_all();
+                landed(slot);
+            }
+            if (!TMA) __syncthreads();   // other threads' element copies are visible after a barrier only
+        };
+        const bool whole = w == BX && h == BY;
+        arrive(q, cur);
 #pragma unroll 1
         for (; q < k1 + 2; ++q) {
             const u32 sq = rs + cur * (S::CELLS * 8);
-            if (q >= k0 + 3) {
-                if (!TMA) cp_async_wait_all();
-                landed(cur);
-            }
-            // In element-wise staging other threads' copies are visible after this barrier only.
-            if (!TMA) __syncthreads();
-            bad = 0;
-            const bool zflux = q >= k0 - 1 && q <= k1, xy = q >= k0 && q < k1;
-            u64 ix[4], iy[4], iz[4], rg[4];
-            int rat = -1;   // where this thread's ring fluxes go
-            auto own_flux = [&]() {
-                double a[4], b[4], c[4];
-                flux(sq + mine, a, b, c);
-                ix[0] = fixm(a[0]), ix[1] = fixm(a[1]), ix[2] = fixm(a[2]), ix[3] = fixe(a[3]);
-                iy[0] = ISO ? ix[1] : fixm(b[0]), iy[1] = fixm(b[1]), iy[2] = fixm(b[2]), iy[3] = fixe(b[3]);
-                iz[0] = ISO ? ix[2] : fixm(c[0]), iz[1] = ISO ? iy[2] : fixm(c[1]), iz[2] = fixm(c[2]), iz[3] = fixe(c[3]);
-            };
-            // The ring's points outside the tile, next to the thread's own (y-ring: rows -1 and BY, the
-            // first 2 BX threads; x-ring: columns -1 and BX, the next 2 BY). Both fluxes in one stretch of
-            // code, so that their chains of FP64 operations overlap: the ring's warps are the ones every
-            // step waits for. Threads without a point take a cell that every tile has.
-            if (zflux) {
-                if (xy && tid < 2 * BX) {
-                    const int rx = tid >> 1, ry = (tid & 1) ? BY : -1;
-                    const bool in = rx < w && (ry < 0 || h == BY);
-                    if (in) rat = (ry + 1) * BX + rx;
-                    double a[4], b[4], c[4];
-                    flux(sq + (in ? ((ry + 2) * PX + rx + 2) * 8 : safe), a, b, c);
-                    own_flux();
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(b[n]) : fixe(b[n]);
-                } else if (xy && tid < 2 * (BX + BY)) {
-                    const int t = tid - 2 * BX, ry = t >> 1, rx = (t & 1) ? BX : -1;
-                    const bool in = ry < h && (rx < 0 || w == BX);
-                    if (in) rat = ry * (BX + 2) + rx + 1;
-                    double a[4], b[4], c[4];
-                    flux(sq + (in ? ((ry + 2) * PX + rx + 2) * 8 : safe), a, b, c);
-                    own_flux();
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(a[n]) : fixe(a[n]);
-                } else if (fluxer) {
-                    own_flux();
-                }
-            }
+            const bool zflux = z_plane(q), xy = xy_plane(q);
             __syncthreads();   // plane q's raw values, plane q-1's fluxes and plane q-5 have been read
             if (next < k1 + 2 && next <= q + 1) stage(next++);
             if (xy) {
@@ -348,7 +403,7 @@ struct RhsFixMarch {
                 if (rat >= 0) {
 #pragma unroll
                     for (int n = 0; n < 4; ++n)
-                        sts1(tid < 2 * BX ? fys + (n * (BY + 2) * BX + rat) * 8 : fxs + (n * BY * (BX + 2) + rat) * 8, rg[n]);
+                        sts1(ring == 1 ? fys + (n * (BY + 2) * BX + rat) * 8 : fxs + (n * BY * (BX + 2) + rat) * 8, rg[n]);
                 }
             }
             {   // plane q to fixed point, in place
@@ -379,59 +434,45 @@ struct RhsFixMarch {
             if (!ok) bad = -1;
             // Plane q in fixed point, its fluxes; a value out of range ends the segment before it is used.
             if (__syncthreads_or(bad < 0)) break;
-            const int kk = q - 2;
-            if (active) {
-                u64 pc[4] = {0, 0, 0, 0};
-                if (xy) {
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) {
-                        const u32 xr = fxs + ((n * BY + ty) * (BX + 2) + tx) * 8, yr = fys + (n * (BY + 2) + ty) * BX * 8 + tx * 8;
-                        pc[n] = (lds1(xr + 16) - lds1(xr)) + (lds1(yr + 2 * BX * 8) - lds1(yr)) - fzp[n];
-                    }
+            bad = 0;
+            // Then plane q-2's result from integers and plane q+1's fluxes in FP64: independent, and in one
+            // stretch of code where the whole tile takes part, so that the two pipes work at once.
+            const int nslot = cur + 1 == NSLOT ? 0 : cur + 1;
+            const u32 sn = rs + nslot * (S::CELLS * 8);
+            using I0 = std::integral_constant<int, 0>;
+            using I1 = std::integral_constant<int, 1>;
+            using I2 = std::integral_constant<int, 2>;
+            if (TMA && whole && q - 2 >= k0 && q + 1 < k1) {
+                gather(true, true);
+                arrive(q + 1, nslot);
+                if (ring == 1) {
+                    fluxes(sn, I1{});
+                    emit();
+                } else if (ring == 2) {
+                    fluxes(sn, I2{});
+                    emit();
+                } else {
+                    fluxes(sn, I0{});
+                    emit();
                 }
-                if (kk >= k0) {
-                    const u32 s0 = back(2) + own, sm1 = back(3) + own, sm2 = back(4) + own, sp1 = back(1) + own, sp2 = sq + own;
-                    double* Rp = R + (i64)kk * g.osz + (i64)(j0 + ty) * g.osy + (i0 + tx);
-                    i64 z[5];
-                    int ze[5];
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) {
-                        constexpr int C = PLANE * 8;
-                        const u64 mid = lds1(s0 + c * C);
-                        const u64 s2 = (lds1(s0 + c * C - 16) + lds1(s0 + c * C + 16) + lds1(s0 + c * C - 16 * PX)) +
-                                       (lds1(s0 + c * C + 16 * PX) + lds1(sm2 + c * C) + lds1(sp2 + c * C));
-                        const u64 s1 = (lds1(s0 + c * C - 8) + lds1(s0 + c * C + 8) + lds1(s0 + c * C - 8 * PX)) +
-                                       (lds1(s0 + c * C + 8 * PX) + lds1(sm1 + c * C) + lds1(sp1 + c * C));
-                        const u64 d4 = (u64)((i64)s2 >> 2) - s1 + (mid << 2) + (u64)((i64)mid >> 1);
-                        const i64 ds = mul63((i64)d4, fx.eh, fx.el);
-                        i64 a;
-                        if (c == 0) {
-                            const u64 ax = lds1(s0 + C + 8) - lds1(s0 + C - 8), ay = lds1(s0 + 2 * C + 8 * PX) - lds1(s0 + 2 * C - 8 * PX),
-                                      az = lds1(sp1 + 3 * C) - lds1(sm1 + 3 * C);
-                            if (ISO)
-                                a = mul63((i64)(ax + ay + az), fx.sh[0], fx.sl[0]);
-                            else
-                                a = (mul63((i64)ax, fx.sh[0], fx.sl[0]) >> min(es - fx.ex_s[0] + 2, 63)) +
-                                    (mul63((i64)ay, fx.sh[1], fx.sl[1]) >> min(es - fx.ex_s[1] + 2, 63)) +
-                                    (mul63((i64)az, fx.sh[2], fx.sl[2]) >> min(es - fx.ex_s[2] + 2, 63));
-                        } else {
-                            a = (i64)pb[c - 1];
-                        }
-                        const int4 j = lds_int4(sc + (c == 0 ? 0 : c == 4 ? 32 : 16));
-                        z[c] = (a >> j.x) + (ds >> j.y);
-                        ze[c] = j.z;
-                    }
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
+            } else {
+                if (active) {
+                    gather(xy, zflux);
+                    if (q - 2 >= k0) emit();
                 }
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    pb[n] = pa[n] + (zflux ? iz[n] : 0);
-                    pa[n] = pc[n];
-                    if (zflux) fzp[n] = iz[n];
+                if (q + 1 < k1 + 2) {
+                    arrive(q + 1, nslot);
+                    if (z_plane(q + 1)) {
+                        if (xy_plane(q + 1) && ring == 1)
+                            fluxes(sn, I1{});
+                        else if (xy_plane(q + 1) && ring == 2)
+                            fluxes(sn, I2{});
+                        else if (fluxer)
+                            fluxes(sn, I0{});
+                    }
                 }
             }
-            cur = cur + 1 == NSLOT ? 0 : cur + 1;
+            cur = nslot;
         }
         // Copies not waited for yet: planes after q that a segment cut short had under way.
         for (int p = max(q + 1, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
