@@ -262,9 +262,10 @@ size_t acs_batch_workspace_bytes(int n);
  * acs_batch_prepare - check n >= 1 items of one kind (each as its single-grid entry point
  * would, including the alias check), order them largest first, and upload the unit table
  * into `ws` (16-byte aligned device memory of at least acs_batch_workspace_bytes(n) bytes:
- * ACS_ERR_ALIGN / ACS_ERR_WORKSPACE otherwise). `tile` NULL = 32 x 8 with z-chunks of 16
- * planes; tile->flags may be ACS_TILE_TMA for a star-stencil batch, which encodes a tensor map
- * per grid into the workspace (grids of even row and plane pitch are then staged by tensor
+ * ACS_ERR_ALIGN / ACS_ERR_WORKSPACE otherwise). `tile` NULL = 16 x 8 with z-chunks of 32
+ * planes and ACS_TILE_TMA (star stencil) or 16 x 16 with z-chunks of 24 (RHS; the columns of an RHS
+ * batch are 16 x 16 whatever the tile); tile->flags may be ACS_TILE_TMA for a star-stencil batch,
+ * which encodes a tensor map per grid into the workspace (grids of even row and plane pitch are then staged by tensor
  * copies, the others element-wise). On success fills `plan`.
  */
 acs_status acs_batch_prepare(const acs_batch_item *items, int n, int kind, const acs_tile *tile, void *ws,
@@ -288,7 +289,7 @@ acs_status acs_batch_launch(const acs_batch_plan *plan, const void *params, acs_
  * that want a graph use acs_batch_prepare + acs_batch_launch. Calls from several host threads
  * are serialised from upload to launch by a library mutex; calls share the array, so calls
  * whose kernels overlap on the GPU (streams not ordered against each other) race.
- * `tile` NULL = 32 x 8, z-chunks of 16; `params` as for the kind.
+ * `tile` NULL = as acs_batch_prepare, staged element-wise; `params` as for the kind.
  */
 #define ACS_BATCH_STATIC_MAX 256
 acs_status acs_batch_run_static(const acs_batch_item *items, int n, int kind, const acs_tile *tile,

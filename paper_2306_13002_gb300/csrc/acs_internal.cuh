@@ -69,6 +69,8 @@ struct BatchPlanHost {
 size_t batch_ws_bytes(int n);
 acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int n, int kind, const acs_tile& tile,
                               unsigned char* ws, size_t ws_bytes, cudaStream_t s, BatchPlanHost& plan);
+bool batch_fixed_launch(const BatchPlanHost& p, unsigned long long* counter, const RhsConst& rk, const StarCoef& sc,
+                        cudaStream_t s, acs_status& st);
 acs_status batch_launch(const BatchPlanHost& p, const RhsConst& rk, const StarCoef& sc, cudaStream_t s);
 acs_status batch_run_static(const acs_batch_item* items, const Geom* geo, int n, int kind, const acs_tile& tile,
                             const RhsConst& rk, const StarCoef& sc, cudaStream_t s);

@@ -24,45 +24,12 @@
 #include <numeric>
 #include <vector>
 
+#include "batch_desc.cuh"
 #include "march.cuh"
 
 namespace acs {
 
-struct BatchDesc {
-    const double* in0;  // U (RHS) or u (stencil)
-    const double* in1;  // unused (RHS) or a (stencil)
-    double* out;
-    Geom g;
-    int ntx, nty, nkc, kchunk;   // this grid's z-chunk (see batch_pack)
-    int tma, pad;                // tma: this grid's planes are staged by its tensor map
-};
-static_assert(sizeof(BatchDesc) <= 112, "the static batch scratch is sized for 112-byte descriptors");
-
-struct BatchHeader {
-    unsigned long long counter;
-    long long total;
-    int n, kind, bx, by, kchunk, maps_off;   // maps_off: byte offset of the tensor maps (0: none)
-    long long pad1[3];
-};
-static_assert(sizeof(BatchHeader) == 64, "batch header is 64 bytes");
-
 namespace {
-
-constexpr size_t kHeader = 64;
-
-__host__ __device__ inline size_t desc_bytes(int n) { return ((size_t)n * sizeof(BatchDesc) + 15) & ~(size_t)15; }
-
-__device__ __forceinline__ int find_item(const long long* __restrict__ prefix, int n, long long u) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] <= u)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
 
 // The star stencil stages planes two steps ahead here (StarShape DEPTH 2): small grids give
 // many edge tiles whose few active warps cannot hide one plane's copy latency per step.
@@ -75,27 +42,13 @@ __global__ void __launch_bounds__(BX * BY, KIND == ACS_KIND_RHS ? RhsShape<BX, B
                  unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
     __shared__ long long s_unit;
-    const BatchHeader* h = reinterpret_cast<const BatchHeader*>(ws);
-    const BatchDesc* items = reinterpret_cast<const BatchDesc*>(ws + kHeader);
-    const int n = h->n;
-    const long long* prefix = reinterpret_cast<const long long*>(ws + kHeader + desc_bytes(n));
-    const long long total = h->total;
+    const BatchView b = batch_view(ws);
     const bool leader = threadIdx.x == 0 && threadIdx.y == 0;
     for (;;) {
-        if (leader) s_unit = (long long)atomicAdd(counter, 1ULL);
-        __syncthreads();
-        const long long u = s_unit;
-        __syncthreads();
-        if (u >= total) break;
-        const int it = find_item(prefix, n, u);
-        const BatchDesc d = items[it];
-        long long lu = u - prefix[it];
-        const int tx = (int)(lu % d.ntx);
-        lu /= d.ntx;
-        const int ty = (int)(lu % d.nty);
-        const int kc = (int)(lu / d.nty);
-        const int k0 = kc * d.kchunk;
-        const int k1 = min(k0 + d.kchunk, d.g.nz);
+        BatchUnit u;
+        if (!batch_next(b, counter, &s_unit, leader, u)) break;
+        const BatchDesc d = b.items[u.item];
+        const int tx = u.tx, ty = u.ty, k0 = u.k0, k1 = u.k1;
         if (KIND == ACS_KIND_RHS) {
             if (rhs_isotropic(rk))   // uniform over the launch: the batch shares one set of constants
                 rhs_march<BX, BY, false, true>(d.in0, d.out, d.g, rk, tx * BX, ty * BY, k0, k1, smem, nullptr, nullptr);
@@ -103,7 +56,7 @@ __global__ void __launch_bounds__(BX * BY, KIND == ACS_KIND_RHS ? RhsShape<BX, B
                 rhs_march<BX, BY, false, false>(d.in0, d.out, d.g, rk, tx * BX, ty * BY, k0, k1, smem, nullptr,
                                                 nullptr);
         } else if (d.tma) {
-            const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(ws + h->maps_off) + it;
+            const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(ws + b.head->maps_off) + u.item;
             if (leader) tensormap_acquire(map);
             star_march<BX, BY, true, kBatchStarDepth>(d.in0, d.in1, d.out, d.g, sc, tx * BX, ty * BY, k0, k1, smem,
                                                        map, tmo);
@@ -278,8 +231,12 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     return ACS_OK;
 }
 
-acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int n, int kind, const acs_tile& tile,
+acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int n, int kind, const acs_tile& asked,
                               unsigned char* ws, size_t ws_bytes, cudaStream_t s, BatchPlanHost& plan) {
+    // Columns of an RHS batch are 16 x 16, the shape the fixed-point march is built for (whether the
+    // parameters suit it is known at the launch only).
+    acs_tile tile = asked;
+    if (kind == ACS_KIND_RHS) tile.bx = tile.by = 16;
     std::vector<unsigned char> image;
     long long total = 0;
     acs_status st = batch_pack(items, geo, n, kind, tile, (uintptr_t)ws, image, total);
@@ -300,6 +257,8 @@ acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int 
 acs_status batch_launch(const BatchPlanHost& p, const RhsConst& rk, const StarCoef& sc, cudaStream_t s) {
     unsigned long long* counter = reinterpret_cast<unsigned long long*>(p.ws);
     if (cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return launch_status("cudaMemsetAsync");
+    acs_status st;
+    if (batch_fixed_launch(p, counter, rk, sc, s, st)) return st;
     if (p.kind == ACS_KIND_RHS) return dispatch<ACS_KIND_RHS>(p, counter, rk, sc, s);
     return dispatch<ACS_KIND_STENCIL>(p, counter, rk, sc, s);
 }

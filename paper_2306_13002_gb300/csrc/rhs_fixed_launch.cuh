@@ -76,13 +76,10 @@ acs_status launch_rhs_fixed_tile(const double* U, double* R, const Geom& g, cons
     return launch_rhs_fixed_t<BX, BY, false, ISO>(U, R, g, kf, kc, fx, t.kchunk, t.flags, map, s);
 }
 
-// The march is built for 16 x 16 and 16 x 8 (larger tiles leave room for one block on an SM): a
-// requested tile of 256 points or more runs as the first, a smaller one as the second.
 template <bool ISO>
 acs_status launch_rhs_fixed_form(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
                                  const RhsFix& fx, const acs_tile& t, cudaStream_t s) {
-    return t.bx * t.by >= 256 ? launch_rhs_fixed_tile<16, 16, ISO>(U, R, g, kf, kc, fx, t, s)
-                              : launch_rhs_fixed_tile<16, 8, ISO>(U, R, g, kf, kc, fx, t, s);
+    return launch_rhs_fixed_tile<16, 16, ISO>(U, R, g, kf, kc, fx, t, s);
 }
 
 }  // namespace

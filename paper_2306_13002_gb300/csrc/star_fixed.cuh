@@ -409,6 +409,10 @@ __device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, c
     u32 phase = 0, flying = 0;
     bool ok = true;
     int kk = k0;
+    if (g.isy >= (1 << 22)) {   // staging offsets are 32 bits
+        m.plain(k0);
+        kk = k1;
+    }
     for (int left = 4; kk < k1; --left) {
         const int done = m.segment(kk, phase, flying, ok);
         __syncthreads();   // the ring and the notes are free again
