@@ -23,6 +23,8 @@
 #include <string>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "acs_internal.cuh"
 
 namespace acs {
@@ -153,6 +155,276 @@ __global__ void mlp_grad_adam(const float* __restrict__ X, const float* __restri
     prm[p] -= lr * mh / (sqrtf(vh) + 1e-8f);
 }
 
+// All epochs in one launch, for models of 64 hidden units whose training set fits shared memory.
+//
+// A cluster of eight blocks: each keeps the whole model and the standardised features in shared
+// memory, runs forward and backward passes of an eighth of the samples, and owns an eighth of the
+// hidden units' parameters (with their Adam moments in registers). Activations and updated
+// parameters go between the blocks through the L2, ordered by two cluster barriers per epoch. Every
+// sum runs over the same terms in the same order as in the kernels above, so the trained model has
+// the same bits.
+//
+// The three launches per epoch took 100 us for 400 samples of 20 features (400 x 64 threads that wait on
+// L2 for every weight, then one thread per parameter over 400 samples): 203 ms for 2000 epochs, now
+// 46 ms. What bounds it now is latency: the sums' chains of 64 and 400 dependent additions, whose order
+// is kept, and two cluster barriers with a trip through the L2 per epoch.
+constexpr int kTrainBlocks = 8, kTrainThreads = 512, kTrainH = 64, kTrainRows = kTrainH / kTrainBlocks;
+constexpr int kTrainPad = kTrainH + 1;   // row pitch of the activations a thread reads along
+
+struct TrainShape {
+    int n, F, NS;   // samples, features, samples per block
+    size_t xs, all, cols, dy, w1t, w2, w2t, vec, floats;
+    __host__ __device__ TrainShape(int n_, int F_) : n(n_), F(F_), NS((n_ + kTrainBlocks - 1) / kTrainBlocks) {
+        xs = 0;                                  // standardised features, n x F
+        all = (xs + (size_t)n * F + 3) & ~(size_t)3;   // H1 of all samples; the block's own activations before that
+        const size_t own = (size_t)NS * (2 * kTrainH + kTrainPad) + NS;   // h1, d2 (rows of 64 floats), h2, dy
+        cols = all + ((size_t)n * kTrainH > own ? (size_t)n * kTrainH : own);   // own columns of DH2, DH1, H2
+        cols = (cols + 3) & ~(size_t)3;
+        dy = cols + (size_t)n * 3 * kTrainRows;
+        w1t = dy + n;                            // W1 transposed, W2, W2 transposed, b1 b2 w3 b3
+        w2 = w1t + (size_t)F * kTrainH;
+        w2t = w2 + kTrainH * kTrainH;
+        vec = w2t + kTrainH * kTrainPad;
+        floats = vec + 3 * kTrainH + 1;
+    }
+};
+
+// Adam's update of one parameter, as in mlp_grad_adam.
+__device__ __forceinline__ float adam_step(float p, float& m, float& v, float g, int step, float lr) {
+    const float b1 = 0.9f, b2 = 0.999f;
+    const float mm = b1 * m + (1.f - b1) * g;
+    const float vv = b2 * v + (1.f - b2) * g * g;
+    m = mm;
+    v = vv;
+    const float mh = mm / (1.f - powf(b1, (float)step));
+    const float vh = vv / (1.f - powf(b2, (float)step));
+    return p - lr * mh / (sqrtf(vh) + 1e-8f);
+}
+
+__global__ void __launch_bounds__(kTrainThreads)
+    mlp_train_cluster(const float* __restrict__ X, const float* __restrict__ T, const float* __restrict__ Wt, float* prm,
+                      float* H1, float* H2, float* DH1, float* DH2, float* DY, int F, int n, int epochs, float lr) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ float sh[];
+    constexpr int H = kTrainH;
+    const TrainShape S(n, F);
+    const Layout L(F, H);
+    const int tid = threadIdx.x, blk = (int)cluster.block_rank();
+    const int s_lo = min(blk * S.NS, n), ns = min(S.NS, n - s_lo);
+    float *xs = sh + S.xs, *h1a = sh + S.all, *c2 = sh + S.cols, *c1 = c2 + (size_t)n * kTrainRows, *ch = c1 + (size_t)n * kTrainRows;
+    float *dyv = sh + S.dy, *W1T = sh + S.w1t, *W2 = sh + S.w2, *W2T = sh + S.w2t, *b1 = sh + S.vec, *b2 = b1 + H, *w3 = b2 + H,
+          *b3 = w3 + H;
+    float *h1o = h1a, *d2o = h1o + (size_t)S.NS * H, *h2o = d2o + (size_t)S.NS * H, *dyo = h2o + (size_t)S.NS * kTrainPad;
+
+    for (int e = tid; e < n * F; e += kTrainThreads) {
+        const int f = e % F;
+        xs[e] = (X[e] - prm[L.mu + f]) / prm[L.sd + f];
+    }
+    auto load_model = [&]() {
+        for (int e = tid; e < H * F; e += kTrainThreads) W1T[(e % F) * H + e / F] = __ldcg(prm + L.W1 + e);
+        for (int e = tid; e < H * H; e += kTrainThreads) {
+            const float w = __ldcg(prm + L.W2 + e);
+            W2[e] = w;
+            W2T[(e % H) * kTrainPad + e / H] = w;
+        }
+        if (tid < H) {
+            b1[tid] = __ldcg(prm + L.b1 + tid);
+            b2[tid] = __ldcg(prm + L.b2 + tid);
+            w3[tid] = __ldcg(prm + L.w3 + tid);
+        }
+        if (tid == 0) b3[0] = __ldcg(prm + L.b3);
+    };
+    load_model();
+
+    // The parameters of this block: rows [j0, j0 + 8) of W1, W2, b1, b2 and of w3 (block 0 also b3).
+    // Threads [0, 128) take 2 x 2 of W2 each; the others one of W1, b1, b2, w3, b3 at a time.
+    const int j0 = blk * kTrainRows;
+    float p4[4], m4[4] = {0, 0, 0, 0}, v4[4] = {0, 0, 0, 0};
+    const int jq = (tid / 32) * 2, k2 = (tid % 32) * 2;
+    if (tid < 128)
+        for (int q = 0; q < 4; ++q) p4[q] = prm[L.W2 + (size_t)(j0 + jq + q / 2) * H + k2 + q % 2];
+    const int others = kTrainRows * F + 3 * kTrainRows + (blk == 0 ? 1 : 0);
+    constexpr int kOther = kTrainThreads - 128, kMost = 2;   // others <= 8 * 93 + 25
+    size_t po[kMost];
+    float pv[kMost], mv[kMost], vv[kMost];
+    for (int r = 0; r < kMost; ++r) {
+        const int o = tid - 128 + r * kOther;
+        mv[r] = vv[r] = 0.f;
+        po[r] = 0;
+        if (tid < 128 || o >= others) continue;
+        const int q = o - kTrainRows * F;
+        po[r] = q < 0 ? L.W1 + (size_t)(j0 + o / F) * F + o % F
+                : q < kTrainRows ? L.b1 + j0 + q : q < 2 * kTrainRows ? L.b2 + j0 + q - kTrainRows
+                : q < 3 * kTrainRows ? L.w3 + j0 + q - 2 * kTrainRows : L.b3;
+        pv[r] = prm[po[r]];
+    }
+    __syncthreads();
+    cluster.sync();   // nobody updates a parameter before all blocks have read the model
+
+    const int j = tid % H, grp = tid / H;
+    constexpr int G = kTrainThreads / H;   // samples worked on at once
+    // a[i] += sum_k w[k][j] v[s_i][k], k in order; four of v at a time (one value serves a whole warp)
+    auto along = [&](const float* w, int pitch, const float* v, float (&a)[8], int base) {
+#pragma unroll 4
+        for (int k = 0; k < H; k += 4) {
+            const float w0 = w[k * pitch + j], w1 = w[(k + 1) * pitch + j], w2 = w[(k + 2) * pitch + j], w3k = w[(k + 3) * pitch + j];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(v + min(base + grp + i * G, ns - 1) * H + k);
+                a[i] += w0 * x.x;
+                a[i] += w1 * x.y;
+                a[i] += w2 * x.z;
+                a[i] += w3k * x.w;
+            }
+        }
+    };
+    for (int ep = 1; ep <= epochs; ++ep) {
+        // Forward and backward passes of the block's samples, a thread per hidden unit.
+        for (int base = 0; base < ns; base += 8 * G) {   // (up to eight samples per thread at a time)
+            float a[8], r1[8], r2[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[i] = b1[j];
+            // (rows of samples past the block's own are read, inside shared memory, and not used)
+            int f = 0;
+            if (F % 4 == 0) {
+                for (; f < F; f += 4) {
+                    const float w0 = W1T[f * H + j], w1 = W1T[(f + 1) * H + j], w2 = W1T[(f + 2) * H + j], w3f = W1T[(f + 3) * H + j];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int s = min(base + grp + i * G, ns - 1);
+                        const float4 x = *reinterpret_cast<const float4*>(xs + (size_t)(s_lo + s) * F + f);
+                        a[i] += w0 * x.x;
+                        a[i] += w1 * x.y;
+                        a[i] += w2 * x.z;
+                        a[i] += w3f * x.w;
+                    }
+                }
+            }
+            for (; f < F; ++f) {
+                const float w = W1T[f * H + j];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] += w * xs[(size_t)(s_lo + min(base + grp + i * G, ns - 1)) * F + f];
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int s = base + grp + i * G;
+                r1[i] = a[i] > 0.f ? a[i] : 0.f;
+                if (s < ns) {
+                    h1o[s * H + j] = r1[i];
+                    H1[(size_t)(s_lo + s) * H + j] = r1[i];
+                }
+                a[i] = b2[j];
+            }
+            __syncthreads();
+            along(W2T, kTrainPad, h1o, a, base);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int s = base + grp + i * G;
+                r2[i] = a[i] > 0.f ? a[i] : 0.f;
+                if (s < ns) {
+                    h2o[s * kTrainPad + j] = r2[i];
+                    H2[(size_t)(s_lo + s) * H + j] = r2[i];
+                }
+            }
+            __syncthreads();
+            const int sy = base + tid;
+            if (tid < 8 * G && sy < ns) {
+                float y = b3[0];
+#pragma unroll 8
+                for (int k = 0; k < H; ++k) y += w3[k] * h2o[sy * kTrainPad + k];
+                const float dy = 2.f * Wt[s_lo + sy] * (y - T[s_lo + sy]) / (float)n;
+                dyo[sy] = dy;
+                DY[s_lo + sy] = dy;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int s = base + grp + i * G;
+                if (s < ns) {
+                    const float gq = r2[i] > 0.f ? dyo[s] * w3[j] : 0.f;
+                    d2o[s * H + j] = gq;
+                    DH2[(size_t)(s_lo + s) * H + j] = gq;
+                }
+                a[i] = 0.f;
+            }
+            __syncthreads();
+            along(W2, H, d2o, a, base);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int s = base + grp + i * G;
+                if (s < ns) DH1[(size_t)(s_lo + s) * H + j] = r1[i] > 0.f ? a[i] : 0.f;
+            }
+            __syncthreads();
+        }
+        cluster.sync();
+        // Activations of all samples: H1 whole, the block's columns of the others.
+        {
+            float4* d = reinterpret_cast<float4*>(h1a);
+            const float4* src = reinterpret_cast<const float4*>(H1);
+            for (int e = tid; e < n * H / 4; e += kTrainThreads) d[e] = __ldcg(src + e);
+            for (int e = tid; e < n * kTrainRows; e += kTrainThreads) {
+                const size_t at = (size_t)(e / kTrainRows) * H + j0 + e % kTrainRows;
+                c2[e] = __ldcg(DH2 + at);
+                c1[e] = __ldcg(DH1 + at);
+                ch[e] = __ldcg(H2 + at);
+            }
+            for (int e = tid; e < n; e += kTrainThreads) dyv[e] = __ldcg(DY + e);
+        }
+        __syncthreads();
+        if (tid < 128) {
+            float g4[4] = {0, 0, 0, 0};
+#pragma unroll 8
+            for (int s = 0; s < n; ++s) {
+                const float2 d = *reinterpret_cast<const float2*>(c2 + s * kTrainRows + jq);
+                const float2 x = *reinterpret_cast<const float2*>(h1a + s * H + k2);
+                g4[0] += d.x * x.x;
+                g4[1] += d.x * x.y;
+                g4[2] += d.y * x.x;
+                g4[3] += d.y * x.y;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                p4[q] = adam_step(p4[q], m4[q], v4[q], g4[q], ep, lr);
+                prm[L.W2 + (size_t)(j0 + jq + q / 2) * H + k2 + q % 2] = p4[q];
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < kMost; ++r) {
+                const int o = tid - 128 + r * kOther, q = o - kTrainRows * F;
+                if (o >= others) continue;
+                float g = 0.f;
+                if (q < 0) {
+                    const int f = o % F, jl = o / F;
+#pragma unroll 8
+                    for (int s = 0; s < n; ++s) g += c1[s * kTrainRows + jl] * xs[s * F + f];
+                } else if (q < 2 * kTrainRows) {
+                    const float* c = q < kTrainRows ? c1 + q : c2 + q - kTrainRows;
+#pragma unroll 8
+                    for (int s = 0; s < n; ++s) g += c[s * kTrainRows];
+                } else if (q < 3 * kTrainRows) {
+#pragma unroll 8
+                    for (int s = 0; s < n; ++s) g += dyv[s] * ch[s * kTrainRows + q - 2 * kTrainRows];
+                } else {
+#pragma unroll 8
+                    for (int s = 0; s < n; ++s) g += dyv[s];
+                }
+                pv[r] = adam_step(pv[r], mv[r], vv[r], g, ep, lr);
+                prm[po[r]] = pv[r];
+            }
+        }
+        cluster.sync();
+        load_model();
+        __syncthreads();
+    }
+}
+
+// Whether the one-launch training takes this model and training set.
+bool train_fits(int n, int F, int H) {
+    return H == kTrainH && n >= kTrainBlocks && kTrainRows * F + 3 * kTrainRows + 1 <= 2 * (kTrainThreads - 128) &&
+           TrainShape(n, F).floats * sizeof(float) <= 227 * 1024;
+}
+
 __global__ void copy_column(const float* __restrict__ X, int F, int col, int n, float* out) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) out[s] = X[(size_t)s * F + col];
@@ -250,6 +522,26 @@ acs_status ranker_train(const float* feats, const float* times, int n, int F, in
     const int tb = H < 32 ? 32 : ((H + 31) / 32) * 32;
     const size_t sh_f = sizeof(float) * (F + 2 * H), sh_b = sizeof(float) * H;
     const unsigned pg = (unsigned)((L.P + 255) / 256);
+    if (epochs > 0 && train_fits(n, F, H) && ((uintptr_t)w.H1 & 15) == 0) {
+        const size_t bytes = TrainShape(n, F).floats * sizeof(float);
+        acs_status st = ensure_smem((const void*)mlp_train_cluster, 227 * 1024);
+        if (st != ACS_OK) return st;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kTrainBlocks);
+        cfg.blockDim = dim3(kTrainThreads);
+        cfg.dynamicSmemBytes = bytes;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kTrainBlocks;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, mlp_train_cluster, feats, (const float*)w.T, (const float*)w.W, params, w.H1, w.H2, w.DH1,
+                               w.DH2, w.DY, F, n, epochs, lr) == cudaSuccess)
+            return launch_status("mlp_train_cluster");
+        cudaGetLastError();   // no room for the cluster: the launches below
+    }
     for (int e = 1; e <= epochs; ++e) {   // epochs == 0: the initial model only
         mlp_forward<<<n, tb, sh_f, s>>>(feats, params, F, H, w.H1, w.H2, w.Y, 1);
         mlp_backward_sample<<<n, tb, sh_b, s>>>(w.T, w.W, params, F, H, n, w.H1, w.H2, w.Y, w.DH1, w.DH2, w.DY);
