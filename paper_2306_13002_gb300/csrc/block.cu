@@ -15,11 +15,9 @@
 //  CSE+BULK    all 151 loads of the point (A, B on three planes, G) before the first store
 //              (Sec. VI-B, the shape of Listing 3); 151 live doubles exceed the register file
 //              share of a thread, as the paper saw for bulk load (+103 registers, Table IV).
-//  saturated   constants folded once, G(p) and the diagonal terms computed once, every
-//              operation issued as an FMA, __restrict__ pointers so that loads may move ahead
-//              of earlier stores within the register budget. (A z-marching form with one
-//              thread per block entry reads each input once but measured slower on GB300:
-//              this body is FP64-bound, not memory-bound.)
+//  saturated   constants folded once, the products of an input plane shared by the three output
+//              planes that use them, every operation issued as an FMA, __restrict__ pointers so
+//              that loads may move ahead of earlier stores within the register budget.
 #include "acs_internal.cuh"
 
 namespace acs {
@@ -111,53 +109,77 @@ __global__ void __launch_bounds__(256) block_cse_kernel(const double* A, const d
     }
 }
 
-// Saturated form: one thread per point; the loop-invariant products are folded once
-// (t2, -t1, -t2, 2 t1, -q4 t2, t1 q3) and held in registers like the Pipe constants, G(p)
-// and its diagonal terms are computed once, every add, subtract and multiply is issued as an
-// FMA (Pipe), and the pointers are __restrict__, so the
-// compiler may hoist loads of later entries over earlier stores as far as registers allow
-// (bulk load bounded by the register file instead of all 151 loads at once).
-// The register bound (four 256-thread blocks per SM, 64 registers) is tuned: it lets the
-// compiler keep about twice as many loads in flight as the default allocation (40 registers,
-// six blocks per SM, 0.69 ms at 128^3) and measured 0.58 ms.
+// 2 v exactly, on the integer pipes (v + v for every v, infinities and NaN included).
+__device__ __forceinline__ double twice(double v) {
+    unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned e = (hi << 1) >> 21;
+    if (e - 1u < 2045u) {
+        hi += 0x100000u;
+    } else if (e == 0) {   // zero or subnormal: the significand moves, into the exponent if need be
+        hi = (hi & 0x80000000u) | (hi << 1) | (lo >> 31);
+        lo <<= 1;
+    } else if (e == 2046) {
+        hi = (hi & 0x80000000u) | 0x7ff00000u;
+        lo = 0;
+    }
+    return __hiloint2double((int)hi, (int)lo);
+}
+
+// Saturated form, one thread per (i, j) and input plane: the products of a plane's A and B entries serve
+// three output planes (the statements L at k+1, D at k and W at k-1 that read them), so every input is
+// read once and one product is shared,
+//     n = -t1 B,   L(k+1) = -t2 A + n,   W(k-1) = t2 A + n,   D(k) = -q4 t2 A - 2 n,
+// four FP64 operations per entry (the doubling is exact and integer) against six with a thread per
+// output point. The loop-invariant products are folded once and held in registers like the Pipe
+// constants, and every add, subtract and multiply is issued as an FMA (Pipe).
+// FP64-bound before and after: 128^3, 167 -> 119.5 operations per point, 584 -> 440 us (96 % of the pipe),
+// 64^3 84 -> 66 us. The register bound (four 256-thread blocks per SM, 64 registers) is tuned:
+// 2 / 3 / 4 / 5 / 6 / 8 blocks ran 641 / 495 / 440 / 450 / 494 / 496 us.
 __global__ void __launch_bounds__(256, 4) block_saturated_kernel(const double* __restrict__ A,
                                                               const double* __restrict__ B,
                                                               const double* __restrict__ G,
                                                               double* __restrict__ out, Geom g, BlkArgs a) {
     // The folded constants and Pipe staged through shared memory into registers (see Pipe).
-    __shared__ double cs[11];
+    __shared__ double cs[10];
     if (threadIdx.x == 0 && threadIdx.y == 0) {
         const double t1 = a.dt * a.q1, t2 = a.dt * a.q2;
-        const double v[11] = {1.0, -1.0, -0.0, t2, -t1, -t2, 2.0 * t1, -a.q4 * t2, t1 * a.q3, 2.0, 1.0};
-        for (int q = 0; q < 11; ++q) cs[q] = v[q];
+        const double v[10] = {1.0, -1.0, -0.0, t2, -t1, -t2, -a.q4 * t2, t1 * a.q3, 2.0, 1.0};
+        for (int q = 0; q < 10; ++q) cs[q] = v[q];
     }
     __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= g.nx || j >= g.ny) return;
     const Pipe pp = Pipe{cs[0], cs[1], cs[2]};
-    const double t2 = cs[3], nt1 = cs[4], nt2 = cs[5], tw1 = cs[6], nq4t2 = cs[7], t1q3 = cs[8], two = cs[9],
-                 one = cs[10];
-    for (int k = blockIdx.z; k < g.nz; k += gridDim.z) {
+    const double t2 = cs[3], nt1 = cs[4], nt2 = cs[5], nq4t2 = cs[6], t1q3 = cs[7], two = cs[8], one = cs[9];
+    for (int kz = blockIdx.z; kz < g.nz + 2; kz += gridDim.z) {
+        const int k = kz - 1;   // input plane -1 .. nz
+        const bool low = k + 1 < g.nz, mid = k >= 0 && k < g.nz, up = k >= 1;   // which outputs it serves
         const i64 p = (i64)(k + g.halo) * g.isz + (i64)(j + g.halo) * g.isy + (i64)(i + g.halo);
-        const i64 o = (i64)k * g.osz + (i64)j * g.osy + i;
-        const double tg = pmul(t1q3, __ldg(G + p), pp);
-        const double dg = fma(two, tg, one);
+        double* o = out + (i64)k * g.osz + (i64)j * g.osy + i;
+        const double tgl = low ? pmul(t1q3, __ldg(G + p + g.isz), pp) : 0.0;
+        const double dg = mid ? fma(two, pmul(t1q3, __ldg(G + p), pp), one) : 0.0;
+        const double tgu = up ? pmul(t1q3, __ldg(G + p - g.isz), pp) : 0.0;
 #pragma unroll
         for (int q = 0; q < 25; ++q) {
-            const double* Aq = A + (i64)q * g.isc + p;
-            const double* Bq = B + (i64)q * g.isc + p;
-            double L = fma(nt2, __ldg(Aq - g.isz), pmul(nt1, __ldg(Bq - g.isz), pp));
-            double D = fma(tw1, __ldg(Bq), pmul(nq4t2, __ldg(Aq), pp));
-            double W = fma(t2, __ldg(Aq + g.isz), pmul(nt1, __ldg(Bq + g.isz), pp));
-            if ((q / 5) == (q % 5)) {
-                L = psub(L, tg, pp);
-                W = psub(W, tg, pp);
-                D = padd(D, dg, pp);
+            const double va = __ldg(A + (i64)q * g.isc + p);
+            const double n = pmul(nt1, __ldg(B + (i64)q * g.isc + p), pp);
+            const bool diag = (q / 5) == (q % 5);
+            if (low) {
+                double L = fma(nt2, va, n);
+                if (diag) L = psub(L, tgl, pp);
+                o[(i64)q * g.osc + g.osz] = L;
             }
-            out[(i64)q * g.osc + o] = L;
-            out[(i64)(25 + q) * g.osc + o] = D;
-            out[(i64)(50 + q) * g.osc + o] = W;
+            if (mid) {
+                double D = fma(nq4t2, va, -twice(n));
+                if (diag) D = padd(D, dg, pp);
+                o[(i64)(25 + q) * g.osc] = D;
+            }
+            if (up) {
+                double W = fma(t2, va, n);
+                if (diag) W = psub(W, tgu, pp);
+                o[(i64)(50 + q) * g.osc - g.osz] = W;
+            }
         }
     }
 }
@@ -173,7 +195,11 @@ acs_status launch_block(const double* A, const double* B, const double* G, doubl
         case ACS_FORM_AS_WRITTEN: block_plain_kernel<<<grid, block, 0, s>>>(A, B, G, out, g, a); break;
         case ACS_FORM_CSE: block_cse_kernel<false><<<grid, block, 0, s>>>(A, B, G, out, g, a); break;
         case ACS_FORM_CSE_BULK: block_cse_kernel<true><<<grid, block, 0, s>>>(A, B, G, out, g, a); break;
-        case ACS_FORM_SATURATED: block_saturated_kernel<<<grid, block, 0, s>>>(A, B, G, out, g, a); break;
+        case ACS_FORM_SATURATED: {
+            const dim3 planes(grid.x, grid.y, g.nz + 2 < 65535 ? g.nz + 2 : 65535);
+            block_saturated_kernel<<<planes, block, 0, s>>>(A, B, G, out, g, a);
+            break;
+        }
         default: return fail(ACS_ERR_INVALID, "block body form %d is not built (use 0, 1, 3 or 5)", form);
     }
     return launch_status("block kernel");
