@@ -254,3 +254,43 @@ def test_rhs_fixed_non_finite_and_unset_corners(tile):
     with np.errstate(all="ignore"):
         far = np.abs(got - ref) <= 2.0 ** -46 * scale * 4.0   # neighbours of the changed cells have larger terms
     assert np.all(far[fine & (scale < 30.0)])
+
+
+# --------------------------------------------------------------------------- ranker training
+
+@pytest.mark.parametrize("n,F", [(8, 1), (9, 5), (63, 20), (64, 20), (65, 20), (400, 20), (430, 7), (100, 92), (57, 93),
+                                 (1200, 20)])
+def test_ranker_one_launch_training(n, F):
+    """The one-launch training (64 hidden units, what fits shared memory; the last two sizes are past its
+    limits) against Adam steps formed here from acs_ranker_gradient at the same parameters. Each update
+    is lr times a ratio of moments computed in about ten FP32 roundings (below 1e-6 of it), and each
+    parameter is rounded once per epoch; 1e-5 lr and 2^-22 |p| per epoch bound both, with room for the
+    later gradients, which see the differences of earlier steps."""
+    rng = np.random.default_rng(n)
+    H, lr, epochs, FW = 64, 3e-3, 6, 1.0
+    X = to_dev(rng.uniform(0.0, 100.0, (n, F)).astype(np.float32))
+    T = to_dev((2.0 + rng.uniform(0.0, 1.0, n)).astype(np.float32))
+    P = binding.acs_ranker_param_count(F, H)
+    ws = torch.empty(binding.acs_ranker_workspace_bytes(n, F, H) // 4 + 4, dtype=torch.float32, device="cuda")
+
+    def train(e):
+        params = torch.full((P,), float("nan"), dtype=torch.float32, device="cuda")
+        binding.acs_ranker_train(X, T, params, ws, hidden=H, epochs=e, lr=lr, fast_weight=FW)
+        return params
+
+    p = train(0)
+    m = np.zeros(P)
+    v = np.zeros(P)
+    g = torch.empty(P, dtype=torch.float32, device="cuda")
+    fixed = 2 * F + 2   # the statistics are not trained
+    for e in range(1, epochs + 1):
+        binding.acs_ranker_gradient(X, T, p, g, ws, hidden=H, fast_weight=FW)
+        gn = g.cpu().numpy().astype(np.float64)
+        m, v = 0.9 * m + 0.1 * gn, 0.999 * v + 0.001 * gn * gn
+        step = lr * (m / (1 - 0.9 ** e)) / (np.sqrt(v / (1 - 0.999 ** e)) + 1e-8)
+        step[:fixed] = 0.0
+        p = train(e)
+        want = (train(e - 1).cpu().numpy().astype(np.float64) - step)
+        got = p.cpu().numpy()
+        assert np.all(np.abs(got - want) <= e * (1e-5 * lr + 2.0 ** -22 * np.abs(want))), (e, np.abs(got - want).max())
+    assert torch.equal(p, train(epochs))
