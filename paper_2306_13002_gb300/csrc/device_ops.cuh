@@ -197,9 +197,8 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem_src) : "memory");
 }
 // The same, or eight zero bytes if !copy (gmem_src is then not read, but must be a valid address).
-__device__ __forceinline__ void cp_async8_or_zero(void* smem_dst, const void* gmem_src, bool copy) {
-    unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem_src), "r"(copy ? 8 : 0) : "memory");
+__device__ __forceinline__ void cp_async8_or_zero(unsigned smem_dst, const void* gmem_src, bool copy) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_dst), "l"(gmem_src), "r"(copy ? 8 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }

@@ -14,8 +14,6 @@
 // the ranges ends the segment.
 #pragma once
 
-#include <type_traits>
-
 #include "fixed.cuh"
 #include "march.cuh"
 
@@ -72,7 +70,8 @@ template <int BX, int BY>
 struct RhsFixShape {
     static constexpr int PX = BX + 4, PY = BY + 4, PLANE = PX * PY, CELLS = 5 * PLANE;
     static constexpr int NT = BX * BY, NSLOT = 6;
-    static constexpr int NE = (CELLS + NT - 1) / NT;
+    static constexpr int NR = 2 * (BX + BY), NC = NT - NR;   // threads of the flux ring, and of the cells
+    static constexpr int NE = (CELLS + NC - 1) / NC;
     static constexpr int FX = 4 * BY * (BX + 2), FY = 4 * (BY + 2) * BX;
     static constexpr int CONST_ELEMS = 16;
     // ... constants of the launch, mbarriers, the scan's results, constants of the segment
@@ -105,7 +104,7 @@ __device__ __forceinline__ RhsJoin rhs_join(int ea, int ed) {
 template <int BX, int BY, bool TMA, bool ISO>
 struct RhsFixMarch {
     using S = RhsFixShape<BX, BY>;
-    static constexpr int PX = S::PX, PLANE = S::PLANE, NE = S::NE, NT = S::NT, NSLOT = S::NSLOT;
+    static constexpr int PX = S::PX, PLANE = S::PLANE, NE = S::NE, NC = S::NC, NSLOT = S::NSLOT;
 
     const double* __restrict__ U;
     double* __restrict__ R;
@@ -137,14 +136,16 @@ struct RhsFixMarch {
         constexpr u32 safe = (2 * PX + 2) * 8;   // the tile's first point
         const u32 own = ((ty + 2) * PX + tx + 2) * 8, mine = fluxer ? own : safe;
 
+        // The first NR threads compute the ring's fluxes; the others stage and convert the cells.
+        const int cell = tid - S::NR;
         u32 full = 0, core = 0;
 #pragma unroll
         for (int n = 0; n < NE; ++n) {
-            const int e = tid + n * NT, r = e % PLANE;
+            const int e = cell + n * NC, r = e % PLANE;
             const int yy = r / PX, xx = r - yy * PX;
-            const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2;
-            if (xx < w + 4 && yy < h + 4 && e < S::CELLS && (xin || yin)) full |= 1u << n;
-            if (xin && yin && e < S::CELLS) core |= 1u << n;
+            const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2, mine = cell >= 0 && e < S::CELLS;
+            if (mine && xx < w + 4 && yy < h + 4 && (xin || yin)) full |= 1u << n;
+            if (mine && xin && yin) core |= 1u << n;
         }
         const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 2 > g.nx || j0 + BY + 2 > g.ny);
         if (TMA && !rim) full = ~0u;
@@ -160,15 +161,29 @@ struct RhsFixMarch {
                     tma_load_4d(smem + slot * S::CELLS, map, bar(slot), i0 - 2 + g.halo, j0 - 2 + g.halo, q + g.halo, 0);
                 }
             } else {
+                // Cell by cell, NC apart: the row and component steps are taken as they come (a division
+                // per cell and 64-bit offsets of all of them at once ran the whole march 1.6 times longer).
                 const double* base = U + (i64)(q + g.halo) * g.isz + (i64)(j0 - 2 + g.halo) * g.isy + (i0 - 2 + g.halo);
-                const u32 m = keep(q);
-#pragma unroll
-                for (int n = 0; n < NE; ++n) {
-                    const int e = tid + n * NT;
-                    if (e >= S::CELLS) break;
-                    const int c = e / PLANE, r = e % PLANE;
-                    const bool in = (m >> n) & 1u;
-                    cp_async8_or_zero(smem + slot * S::CELLS + e, base + (in ? c * g.isc + (r / PX) * g.isy + r % PX : 0), in);
+                u32 m = keep(q), dst = rs + (slot * S::CELLS + cell) * 8;
+                int xx = cell % PX, yy = cell / PX;
+                const double* at = base + yy * g.isy + xx;
+#pragma unroll 1
+                for (int e = cell; e >= 0 && e < S::CELLS; e += NC) {
+                    cp_async8_or_zero(dst, (m & 1u) ? at : base, m & 1u);
+                    m >>= 1;
+                    dst += NC * 8;
+                    at += (NC / PX) * g.isy + NC % PX;
+                    xx += NC % PX;
+                    yy += NC / PX;
+                    if (xx >= PX) {
+                        xx -= PX;
+                        ++yy;
+                        at += g.isy - PX;
+                    }
+                    if (yy >= S::PY) {
+                        yy -= S::PY;
+                        at += g.isc - S::PY * g.isy;
+                    }
                 }
                 cp_async_commit();
             }
@@ -180,8 +195,8 @@ struct RhsFixMarch {
         };
         // f(n, cell, kind) over this thread's cells of a slot; kind 0 rho, 1 momentum, 2 E
         auto kind_of = [&](int n) {
-            const int e = tid + n * NT;
-            return (n + 1) * NT <= PLANE ? 0 : n * NT >= PLANE && (n + 1) * NT <= 4 * PLANE ? 1 : n * NT >= 4 * PLANE ? 2
+            const int e = cell + n * NC;
+            return (n + 1) * NC <= PLANE ? 0 : n * NC >= PLANE && (n + 1) * NC <= 4 * PLANE ? 1 : n * NC >= 4 * PLANE ? 2
                    : e < PLANE ? 0 : e < 4 * PLANE ? 1 : 2;
         };
 
@@ -199,8 +214,8 @@ struct RhsFixMarch {
             const u32 m = keep(k0 - 2 + p);
 #pragma unroll
             for (int n = 0; n < NE; ++n) {
-                if (!((m >> n) & 1u) || tid + n * NT >= S::CELLS) continue;
-                const u64 v = lds1(rs + (p * S::CELLS + tid + n * NT) * 8);
+                if (cell < 0 || !((m >> n) & 1u) || cell + n * NC >= S::CELLS) continue;
+                const u64 v = lds1(rs + (p * S::CELLS + cell + n * NC) * 8);
                 const int e = (int)((hi32(v) << 1) >> 21), kd = kind_of(n);
                 if (kd == 0) {
                     rng[0] = max(rng[0], e);
@@ -311,19 +326,23 @@ struct RhsFixMarch {
                 rfrom = ((ry + 2) * PX + rx + 2) * 8;
             }
         }
-        // Fluxes of the plane at sn. The ring's and the own one stand in one stretch of code, so that
-        // their chains of FP64 operations overlap: the ring's warps are the ones every step waits for.
-        auto fluxes = [&](u32 sn, auto kind) {
-            constexpr int RING = decltype(kind)::value;
-            double a[4], b[4], c[4], d[4], e[4], f[4];
-            if (RING) flux(sn + rfrom, d, e, f);
+        auto ring_flux = [&](u32 sn) {   // of the plane at sn
+            double a[4], b[4], c[4];
+            flux(sn + rfrom, a, b, c);
+            if (ring == 1) {
+#pragma unroll
+                for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(b[n]) : fixe(b[n]);
+            } else {
+#pragma unroll
+                for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(a[n]) : fixe(a[n]);
+            }
+        };
+        auto own_flux = [&](u32 sn) {
+            double a[4], b[4], c[4];
             flux(sn + mine, a, b, c);
             ix[0] = fixm(a[0]), ix[1] = fixm(a[1]), ix[2] = fixm(a[2]), ix[3] = fixe(a[3]);
             iy[0] = ISO ? ix[1] : fixm(b[0]), iy[1] = fixm(b[1]), iy[2] = fixm(b[2]), iy[3] = fixe(b[3]);
             iz[0] = ISO ? ix[2] : fixm(c[0]), iz[1] = ISO ? iy[2] : fixm(c[1]), iz[2] = fixm(c[2]), iz[3] = fixe(c[3]);
-            if (RING)
-#pragma unroll
-                for (int n = 0; n < 4; ++n) rg[n] = n < 3 ? fixm(RING == 1 ? e[n] : d[n]) : fixe(RING == 1 ? e[n] : d[n]);
         };
         // x and y flux differences of plane q; the flux sums move on by one plane.
         u64 po[4];   // the complete flux sums of plane q-2
@@ -341,20 +360,22 @@ struct RhsFixMarch {
                 if (zflux) fzp[n] = iz[n];
             }
         };
+        u64 old[5];   // the thread's own values at plane q-4: its slot is being filled again
         auto emit = [&]() {   // the result at plane q-2
             const int kk = q - 2;
-            const u32 s0 = back(2) + own, sm1 = back(3) + own, sm2 = back(4) + own, sp1 = back(1) + own, sp2 = back(0) + own;
+            const u32 s0 = back(2) + own, sm1 = back(3) + own, sp1 = back(1) + own, sp2 = back(0) + own;
             double* Rp = R + (i64)kk * g.osz + (i64)(j0 + ty) * g.osy + (i0 + tx);
             i64 z[5];
             int ze[5];
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
                 constexpr int C = PLANE * 8;
-                const u64 mid = lds1(s0 + c * C);
+                const u64 mid = lds1(s0 + c * C), below = lds1(sm1 + c * C);
                 const u64 s2 = (lds1(s0 + c * C - 16) + lds1(s0 + c * C + 16) + lds1(s0 + c * C - 16 * PX)) +
-                               (lds1(s0 + c * C + 16 * PX) + lds1(sm2 + c * C) + lds1(sp2 + c * C));
+                               (lds1(s0 + c * C + 16 * PX) + old[c] + lds1(sp2 + c * C));
                 const u64 s1 = (lds1(s0 + c * C - 8) + lds1(s0 + c * C + 8) + lds1(s0 + c * C - 8 * PX)) +
-                               (lds1(s0 + c * C + 8 * PX) + lds1(sm1 + c * C) + lds1(sp1 + c * C));
+                               (lds1(s0 + c * C + 8 * PX) + below + lds1(sp1 + c * C));
+                old[c] = below;
                 const u64 d4 = (u64)((i64)s2 >> 2) - s1 + (mid << 2) + (u64)((i64)mid >> 1);
                 const i64 ds = mul63((i64)d4, fx.eh, fx.el);
                 i64 a;
@@ -377,21 +398,16 @@ struct RhsFixMarch {
 #pragma unroll
             for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
         };
-        auto arrive = [&](int p, int slot) {   // plane p's raw values are in its slot
-            if (p >= k0 + 3) {
-                if (!TMA) cp_async_wait_all();
-                landed(slot);
-            }
-            if (!TMA) __syncthreads();   // other threads' element copies are visible after a barrier only
-        };
         const bool whole = w == BX && h == BY;
-        arrive(q, cur);
 #pragma unroll 1
         for (; q < k1 + 2; ++q) {
             const u32 sq = rs + cur * (S::CELLS * 8);
+            const int nslot = cur + 1 == NSLOT ? 0 : cur + 1;
+            const u32 sn = rs + nslot * (S::CELLS * 8);
             const bool zflux = z_plane(q), xy = xy_plane(q);
-            __syncthreads();   // plane q's raw values, plane q-1's fluxes and plane q-5 have been read
-            if (next < k1 + 2 && next <= q + 1) stage(next++);
+            if (!TMA) cp_async_wait_all();   // this thread's copies up to plane q+1, visible after the barrier
+            __syncthreads();   // plane q's raw values, plane q-1's fluxes and plane q-4 have been read
+            if (next < k1 + 2 && next <= q + 2) stage(next++);
             if (xy) {
                 if (fluxer) {
 #pragma unroll
@@ -406,12 +422,16 @@ struct RhsFixMarch {
                         sts1(ring == 1 ? fys + (n * (BY + 2) * BX + rat) * 8 : fxs + (n * BY * (BX + 2) + rat) * 8, rg[n]);
                 }
             }
-            {   // plane q to fixed point, in place
+            if (q + 1 < k1 + 2 && q + 1 >= k0 + 3) landed(nslot);
+            // The ring's fluxes of plane q+1 in FP64, beside the other threads' conversion of plane q.
+            if (ring) {
+                if (xy_plane(q + 1)) ring_flux(sn);
+            } else {   // plane q to fixed point, in place
                 const u32 m = rim || !TMA || !xy ? keep(q) : ~0u;
                 u64 v[NE];
 #pragma unroll
                 for (int n = 0; n < NE; ++n)
-                    v[n] = (n + 1) * NT <= S::CELLS || tid + n * NT < S::CELLS ? lds1(sq + (tid + n * NT) * 8) : 0ull;
+                    v[n] = (n + 1) * NC <= S::CELLS || cell + n * NC < S::CELLS ? lds1(sq + (cell + n * NC) * 8) : 0ull;
                 if (m != ~0u) {
 #pragma unroll
                     for (int n = 0; n < NE; ++n) {   // cells no point reads: a value in range
@@ -423,10 +443,10 @@ struct RhsFixMarch {
                 for (int n = 0; n < NE; ++n) {
                     const int kd = kind_of(n);
                     const int cu = lds_int(sc + 48 + 4 * kd);
-                    if ((n + 1) * NT <= S::CELLS || tid + n * NT < S::CELLS) {
-                        if ((n + 1) * NT > 4 * PLANE || n * NT < PLANE)
+                    if ((n + 1) * NC <= S::CELLS || cell + n * NC < S::CELLS) {
+                        if ((n + 1) * NC > 4 * PLANE || n * NC < PLANE)
                             bad |= (int)((hi32(v[n]) << 1) >> 21) - lds_int(sc + 60 + 4 * kd);
-                        sts1(sq + (tid + n * NT) * 8, to_fixed(v[n], cu, 0, bad));
+                        sts1(sq + (cell + n * NC) * 8, to_fixed(v[n], cu, 0, bad));
                     }
                 }
                 if (TMA) fence_proxy_async();
@@ -437,45 +457,26 @@ struct RhsFixMarch {
             bad = 0;
             // Then plane q-2's result from integers and plane q+1's fluxes in FP64: independent, and in one
             // stretch of code where the whole tile takes part, so that the two pipes work at once.
-            const int nslot = cur + 1 == NSLOT ? 0 : cur + 1;
-            const u32 sn = rs + nslot * (S::CELLS * 8);
-            using I0 = std::integral_constant<int, 0>;
-            using I1 = std::integral_constant<int, 1>;
-            using I2 = std::integral_constant<int, 2>;
-            if (TMA && whole && q - 2 >= k0 && q + 1 < k1) {
+            if (whole && q - 2 >= k0 && q + 1 < k1) {
                 gather(true, true);
-                arrive(q + 1, nslot);
-                if (ring == 1) {
-                    fluxes(sn, I1{});
-                    emit();
-                } else if (ring == 2) {
-                    fluxes(sn, I2{});
-                    emit();
-                } else {
-                    fluxes(sn, I0{});
-                    emit();
-                }
+                own_flux(sn);
+                emit();
             } else {
                 if (active) {
                     gather(xy, zflux);
-                    if (q - 2 >= k0) emit();
-                }
-                if (q + 1 < k1 + 2) {
-                    arrive(q + 1, nslot);
-                    if (z_plane(q + 1)) {
-                        if (xy_plane(q + 1) && ring == 1)
-                            fluxes(sn, I1{});
-                        else if (xy_plane(q + 1) && ring == 2)
-                            fluxes(sn, I2{});
-                        else if (fluxer)
-                            fluxes(sn, I0{});
+                    if (q - 2 >= k0) {
+                        emit();
+                    } else if (q == k0 + 1) {
+#pragma unroll
+                        for (int c = 0; c < 5; ++c) old[c] = lds1(back(3) + own + c * PLANE * 8);
                     }
                 }
+                if (fluxer && z_plane(q + 1)) own_flux(sn);
             }
             cur = nslot;
         }
-        // Copies not waited for yet: planes after q that a segment cut short had under way.
-        for (int p = max(q + 1, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
+        // Copies not waited for yet: planes after q + 1 that a segment cut short had under way.
+        for (int p = max(q + 2, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
         if (!TMA) cp_async_wait_all();
         return min(max(q - 2, k0), k1);
     }

@@ -107,7 +107,7 @@ struct StarFixMarch {
 #pragma unroll
             for (int n = 0; n < NE; ++n)
                 if (NE * NT == PLANE || n + 1 < NE || tid + n * NT < PLANE)
-                    cp_async8_or_zero(dst + tid + n * NT, base + off[n], (keep >> n) & 1u);
+                    cp_async8_or_zero(smem_addr(dst + tid + n * NT), base + off[n], (keep >> n) & 1u);
             cp_async_commit();
         }
     }
