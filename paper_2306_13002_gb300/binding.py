@@ -91,6 +91,8 @@ EXPORTS = ("acs_rhs_plain", "acs_rhs_saturated", "acs_rhs_form", "acs_stencil_pl
 def lib() -> ctypes.CDLL:
     """Load libacs.so (built by `build.build()` / `__graft_entry__.build()`)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -179,13 +181,28 @@ def _check(status: int, func: str) -> None:
         raise AcsError(status, func, lib().acs_last_error().decode())
 
 
+_raw_stream = None   # device index -> the current stream's handle, where this torch has the direct query
+
+
+def _current_stream() -> int | None:
+    """Handle of the current stream of the current device (0.3 us by torch's direct query, 2 us through a
+    Stream object: a small grid's whole call is 10 us)."""
+    global _raw_stream
+    try:
+        if _raw_stream is None:
+            import torch
+            raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+            if raw is None or dev is None or not torch.cuda.is_initialized():
+                return torch.cuda.current_stream().cuda_stream or None
+            _raw_stream = lambda: raw(dev())  # noqa: E731
+        return _raw_stream() or None
+    except Exception:  # pragma: no cover
+        return None
+
+
 def _stream_ptr(stream) -> int | None:
     if stream is None:
-        try:
-            import torch
-            return torch.cuda.current_stream().cuda_stream or None
-        except Exception:  # pragma: no cover
-            return None
+        return _current_stream()
     if isinstance(stream, int):
         return stream or None
     return getattr(stream, "cuda_stream", None) or None
@@ -234,8 +251,11 @@ def grid_for(inp, out, halo: int, ncomp: int, host: bool = False) -> Grid:
     return Grid(nx, ny, nz, halo, isy, isz, isc, osy, osz, osc)
 
 
+_Triple = ctypes.c_double * 3
+
+
 def _params(gamma, eps, h) -> RhsParams:
-    return RhsParams(float(gamma), float(eps), (ctypes.c_double * 3)(*[float(v) for v in h]))
+    return RhsParams(float(gamma), float(eps), _Triple(*[float(v) for v in h]))
 
 
 def acs_rhs_plain(U, R, gamma: float = 1.4, eps: float = 0.25, h=(1.0, 1.0, 1.0), halo: int = 2,
@@ -268,14 +288,17 @@ def acs_rhs_form(U, R, form, gamma: float = 1.4, eps: float = 0.25, h=(1.0, 1.0,
                               _stream_ptr(stream)), "acs_rhs_form")
 
 
+_Coef = ctypes.c_double * 12
+_TAYLOR8_COEF = _Coef(*(TAYLOR8 * 3))   # read by the library only
+
+
 def _coef(c) -> ctypes.Array:
     if c is None:
-        vals = list(TAYLOR8) * 3
-    else:
-        vals = [float(v) for row in c for v in (row if hasattr(row, "__len__") else [row])]
+        return _TAYLOR8_COEF
+    vals = [float(v) for row in c for v in (row if hasattr(row, "__len__") else [row])]
     if len(vals) != 12:
         raise ValueError("stencil coefficients must be 3 x 4")
-    return (ctypes.c_double * 12)(*vals)
+    return _Coef(*vals)
 
 
 def acs_stencil_plain(u, a, out, c=None, halo: int = 4, stream=None) -> None:
