@@ -131,8 +131,8 @@ typedef struct acs_tile {
  * Accepted by the single-grid saturated calls, their autotuners and star-stencil batches
  * (acs_batch_prepare, acs_autotune_batch: per grid; RHS batches and acs_batch_run_static reject
  * it). Used where the layout allows it (16-byte aligned input, row, plane and component strides
- * that are multiples of 2 elements, even halo); other layouts, or other grids of a batch, are
- * staged element-wise, with the same results. Waits on the mbarriers are bounded (about one
+ * that are multiples of 2 elements, even halo); other layouts, and batches with such a
+ * grid, are staged element-wise, with the same results. Waits on the mbarriers are bounded (about one
  * second); one that runs out is counted (acs_wait_timeouts) and the call's results are then
  * wrong, but the kernel ends. */
 #define ACS_TILE_TMA 2
@@ -265,8 +265,9 @@ size_t acs_batch_workspace_bytes(int n);
  * ACS_ERR_ALIGN / ACS_ERR_WORKSPACE otherwise). `tile` NULL = 16 x 8 with z-chunks of 32
  * planes and ACS_TILE_TMA (star stencil) or 16 x 16 with z-chunks of 24 (RHS; the columns of an RHS
  * batch are 16 x 16 whatever the tile); tile->flags may be ACS_TILE_TMA for a star-stencil batch,
- * which encodes a tensor map per grid into the workspace (grids of even row and plane pitch are then staged by tensor
- * copies, the others element-wise). On success fills `plan`.
+ * which encodes a tensor map per grid into the workspace if every grid of the batch can be staged so
+ * (even row and plane pitch, 16-byte aligned; otherwise all are staged element-wise). Long z-chunks
+ * are shortened for batches with little work per resident block. On success fills `plan`.
  */
 acs_status acs_batch_prepare(const acs_batch_item *items, int n, int kind, const acs_tile *tile, void *ws,
                              size_t ws_bytes, acs_batch_plan *plan, acs_stream stream);

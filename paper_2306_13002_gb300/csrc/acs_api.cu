@@ -376,8 +376,8 @@ acs_status batch_params(int kind, const void* params, RhsConst& rk, StarCoef& sc
 const acs_tile kDefaultRhsTile = {16, 16, 0, ACS_TILE_BALANCED | ACS_TILE_TMA};
 const acs_tile kDefaultStarTile = {32, 8, 0, ACS_TILE_TMA};
 // Batches: the marches start a few planes before their first result, so chunks are long (64 star grids:
-// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 680 us with chunks of
-// 24, 691 with 16, 761 with 32, whose last units run alone).
+// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 607 us with chunks of
+// 24, 605 with 16, 672 with 8); batches with less work take shorter ones (batch_pack).
 acs_tile default_batch_tile(int kind, int staging) {
     return kind == ACS_KIND_STENCIL ? acs_tile{16, 8, 32, staging} : acs_tile{16, 16, 24, 0};
 }

@@ -59,6 +59,7 @@ acs_status launch_stencil_saturated(const double* u, const double* a, double* ou
                                     const StarCoef& c, const acs_tile& t, cudaStream_t s);
 
 // Host view of a prepared batch (mirrors acs_batch_plan).
+constexpr int kBatchPlain = 0x100;   // in a plan's tile.flags: too little work for the fixed-point RHS march
 struct BatchPlanHost {
     unsigned char* ws;
     size_t ws_bytes;

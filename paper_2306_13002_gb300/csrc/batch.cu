@@ -12,10 +12,9 @@
 //   [0, 64)                BatchHeader (the work counter, the unit total, the shape)
 //   [64, 64 + n*D)         BatchDesc per grid, in processing order
 //   [.., + 8 (n+1))        prefix sums of the grids' unit counts
-//   [maps, + 128 n)        star-stencil batches with ACS_TILE_TMA: a tensor map per grid, in
-//                          processing order, at the first 128-byte aligned address after the
-//                          prefix sums (the header records the offset); grids whose layout TMA
-//                          cannot copy are staged element-wise.
+//   [maps, + 128 n)        star-stencil batches with ACS_TILE_TMA all of whose grids TMA can copy: a
+//                          tensor map per grid, in processing order, at the first 128-byte aligned
+//                          address after the prefix sums (the header records the offset).
 // acs_batch_prepare uploads everything but the counter; acs_batch_launch zeroes the
 // counter with a memset on the stream and launches, so a prepared batch can be launched
 // repeatedly and captured in a CUDA graph (a memset node plus a kernel node).
@@ -159,18 +158,29 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     std::iota(order.begin(), order.end(), 0);
     auto points = [&](int q) { return (long long)geo[q].nx * geo[q].ny * geo[q].nz; };
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return points(x) > points(y); });
-    // Guided z-chunks: the grids at the end of the order, whose units make up the last two
-    // waves of the queue (two units per resident block), take z-chunks a quarter as long, so
-    // the blocks run out of work closer together.
-    const long long waves = 2LL * resident_batch_blocks(kind, tile);
-    const int tail_kchunk = std::max(1, tile.kchunk / 4);
-    std::vector<int> kchunk(n, tile.kchunk);
-    std::vector<long long> units(n);
+    // z-chunks of a batch with little work are shortened, so that the queue still holds a few units per
+    // resident block (RHS: two; star stencil, whose blocks are smaller: one) but no shorter than what a
+    // unit's start is worth. 8 RHS grids with sides of 16 to 96: chunks of 24 / 16 / 8 / 6 ran 404 / 297 /
+    // 206 / 205 us, 16 grids 410 / 302 / 311 / 328; 8 star grids 32 / 16 / 8: 72 / 57 / 62 us.
+    const long long resident = resident_batch_blocks(kind, tile);
     auto unit_count = [&](int q, int kc) {
         const Geom& g = geo[q];
         const long long ntx = (g.nx + tile.bx - 1) / tile.bx, nty = (g.ny + tile.by - 1) / tile.by;
         return ntx * nty * ((g.nz + kc - 1) / kc);
     };
+    long long planes = 0;
+    for (int q = 0; q < n; ++q) planes += unit_count(q, 1);
+    const bool rhs = kind == ACS_KIND_RHS;
+    const bool plain = (tile.flags & kBatchPlain) != 0;   // the FP64 march, which starts at once
+    const int kc = plain ? std::min(tile.kchunk, 16)
+                         : (int)std::min<long long>(tile.kchunk, std::max<long long>(rhs ? 8 : 16, planes / (resident * (rhs ? 2 : 1))));
+    // Guided z-chunks: the grids at the end of the order, whose units make up the last two
+    // waves of the queue (two units per resident block), take z-chunks a quarter as long, so
+    // the blocks run out of work closer together.
+    const long long waves = 2LL * resident;
+    const int tail_kchunk = std::min(kc, std::max(plain ? 1 : 4, kc / 4));
+    std::vector<int> kchunk(n, kc);
+    std::vector<long long> units(n);
     long long tail = 0;
     for (int r = n - 1; r >= 0; --r) {
         const int q = order[r];
@@ -191,7 +201,17 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     long long* prefix = reinterpret_cast<long long*>(image.data() + kHeader + desc_bytes(n));
     // Tensor maps of a star-stencil batch staged by TMA: at the first 128-byte aligned device
     // address after the table.
-    const bool tma = (tile.flags & ACS_TILE_TMA) && kind == ACS_KIND_STENCIL;
+    // All grids or none: blocks that run both stagings by turns crowd the instruction cache (64 grids, half
+    // of them of even pitch: 293 us mixed, 257 us element-wise, 245 us if all can be copied).
+    bool tma = (tile.flags & ACS_TILE_TMA) && kind == ACS_KIND_STENCIL;
+    std::vector<CUtensorMap> map(tma ? n : 0);
+    for (int q = 0; q < n && tma; ++q) {
+        std::memset(&map[q], 0, sizeof(CUtensorMap));
+        if (encode_plane_map(items[q].in0, geo[q], 1, tile.bx + 8, tile.by + 8, &map[q]) != ACS_OK) {
+            tma = false;   // an odd pitch or a misaligned base
+            set_error("%s", "");
+        }
+    }
     if (tma) {
         const uintptr_t first = (ws_addr + batch_table_bytes(n) + 127) & ~(uintptr_t)127;
         h.maps_off = (int)(first - ws_addr);
@@ -210,15 +230,9 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
         e.nty = (g.ny + tile.by - 1) / tile.by;
         e.nkc = (g.nz + kchunk[q] - 1) / kchunk[q];
         e.kchunk = kchunk[q];
-        if (tma) {   // a layout TMA cannot copy (odd pitch, misaligned base) is staged element-wise
-            CUtensorMap map;
-            std::memset(&map, 0, sizeof(map));
-            if (encode_plane_map(items[q].in0, g, 1, tile.bx + 8, tile.by + 8, &map) == ACS_OK) {
-                e.tma = 1;
-                std::memcpy(image.data() + h.maps_off + (size_t)r * sizeof(CUtensorMap), &map, sizeof(map));
-            } else {
-                set_error("%s", "");
-            }
+        if (tma) {
+            e.tma = 1;
+            std::memcpy(image.data() + h.maps_off + (size_t)r * sizeof(CUtensorMap), &map[q], sizeof(CUtensorMap));
         }
         d[r] = e;
         prefix[r] = acc;
@@ -236,7 +250,14 @@ acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int 
     // Columns of an RHS batch are 16 x 16, the shape the fixed-point march is built for (whether the
     // parameters suit it is known at the launch only).
     acs_tile tile = asked;
-    if (kind == ACS_KIND_RHS) tile.bx = tile.by = 16;
+    if (kind == ACS_KIND_RHS) {
+        tile.bx = tile.by = 16;
+        // Few planes per resident block: the FP64 march (4 grids with sides of 16 to 60, 3.2 planes: 87 us
+        // against 95 to 105; 12 grids, 8.9 planes: 223 against 165).
+        long long planes = 0;
+        for (int q = 0; q < n; ++q) planes += (i64)((geo[q].nx + 15) / 16) * ((geo[q].ny + 15) / 16) * geo[q].nz;
+        if (planes < 5 * resident_batch_blocks(kind, tile)) tile.flags |= kBatchPlain;
+    }
     std::vector<unsigned char> image;
     long long total = 0;
     acs_status st = batch_pack(items, geo, n, kind, tile, (uintptr_t)ws, image, total);

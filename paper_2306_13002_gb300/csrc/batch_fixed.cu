@@ -107,7 +107,7 @@ bool batch_fixed_launch(const BatchPlanHost& p, unsigned long long* counter, con
     RhsConst kc;
     rhs_fix(rk, fx, kc);
     if (!fx.ok) return false;
-    if (bx != 16 || by != 16) return false;
+    if (bx != 16 || by != 16 || (p.tile.flags & kBatchPlain)) return false;
     st = launch_rhs_t<16, 16>(p, counter, rk, kc, fx, s);
     return true;
 }
