@@ -34,16 +34,14 @@ UNIT = "Gpoint-updates/s"
 N_RHS = 256
 N_STAR = 384
 
-# FP64-pipe operations per interior point of the saturated RHS, from its expression DAG
-# (FMA, add, mul each one pipe operation). With three spacings: per point 21 for the fluxes
-# (3 Newton FMAs of the reciprocal, 3 velocities, 2 for |m.v|, 2 for P, E+P, 3 diagonal,
-# 3 off-diagonal, 3 energy) + 5 components x 19 (3 differences, 3 for the scaled flux sum,
-# 10 for S2 and S1, 2 for S2 - 4 S1 + 18 U, 1 final FMA) = 116; the rewriter's march variants
-# compute this form. With equal spacing (the benchmark grids) the built-in kernel folds
-# -1/(2h) into the fluxes: 23 for the fluxes (+ the scaled reciprocal and pressure) + 19 for
-# the mass component + 4 x 18 (2 adds in place of 3 scaled terms) = 114.
-# The star stencil: 1 + 12 x 2 + 1 = 26.
-DP_OPS_PER_POINT = {"rhs_saturated": 114, "rhs_saturated_anisotropic": 116, "star_saturated": 26}
+# FP64-pipe operations per interior point. The built-in saturated kernels add neighbours on the
+# integer pipes and keep FP64 for the fluxes (equal spacing: 3 Newton FMAs of the reciprocal and its
+# scale, 3 velocities, 3 for |m.v|, 2 for P and 1 for its scale, E+P, 3 diagonal, 3 off-diagonal, 3 energy
+# = 23) and, in the star stencil, for the conversion of the sum (2) and the product with a(p) (1). The
+# rewriter's march variants compute all of the RHS in FP64 with three spacings: 21 for the fluxes +
+# 5 components x 19 (3 differences, 3 for the scaled flux sum, 10 for S2 and S1, 2 for
+# S2 - 4 S1 + 18 U, 1 final FMA) = 116.
+DP_OPS_PER_POINT = {"rhs_saturated": 23, "rhs_variant": 116, "star_saturated": 3}
 # The FP64 pipe's nominal issue rate: 2 operations / clock / SM (nominal 1.25 TFLOP/s of FMA
 # at 2070 MHz on 152 SMs: 1.25e12 / 2 / 152 / 2.07e9 = 1.99). The roofline's peak is the rate
 # the FP64 probe measures in the same run; 2 x SMs x max SM clock (both queried from the device)
@@ -65,12 +63,13 @@ NCU_TRAFFIC = {
 
 def kernel_source_hash() -> str:
     """Hash of the code (comments and whitespace removed) the saturated RHS kernel is compiled
-    from: rhs_saturated.cu, device_ops.cuh, tma.cuh and the RHS part of march.cuh (everything
-    before the star stencil's StarShape). A comment edit, or an edit of the star stencil's
-    march, keeps the recorded ncu traffic; a code edit of the RHS kernel drops it."""
+    from: the rhs_fixed files, fixed.cuh, rhs_saturated.cu, device_ops.cuh, tma.cuh and the RHS part
+    of march.cuh (everything before the star stencil's StarShape). A comment edit, or an edit of the
+    star stencil's march, keeps the recorded ncu traffic; a code edit of the RHS kernel drops it."""
     import re
     h = hashlib.sha256()
-    for f in ("march.cuh", "rhs_saturated.cu", "device_ops.cuh", "tma.cuh"):
+    for f in ("march.cuh", "rhs_saturated.cu", "device_ops.cuh", "tma.cuh", "fixed.cuh", "rhs_fixed.cuh",
+              "rhs_fixed_launch.cuh", "rhs_fixed_iso.cu"):
         with open(os.path.join(ROOT, "paper_2306_13002_gb300", "csrc", f)) as fh:
             text = fh.read()
         if f == "march.cuh":
@@ -635,7 +634,7 @@ def bench_large(torch, binding, inputs, stream, peak_gops: float, pick_index: in
         rhs[form] = {"ms": ms, "gpts": pts / (ms * 1e-3) / 1e9}
     if pick is not None:
         rhs["ranker_pick_variant"].update({"index": pick_index, "shape": [*pick.block, pick.flags],
-                                           "fp64_frac_at_116_ops": DP_OPS_PER_POINT["rhs_saturated_anisotropic"] * pts /
+                                           "fp64_frac_at_116_ops": DP_OPS_PER_POINT["rhs_variant"] * pts /
                                            (rhs["ranker_pick_variant"]["ms"] * 1e-3) / 1e9 / peak_gops})
         pick.close()
     sat = rhs["saturated_autotuned"]["ms"]

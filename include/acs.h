@@ -43,6 +43,9 @@
  *    returns a status. Launch failures return ACS_ERR_CUDA. `acs_last_error()` gives a
  *    human-readable reason for the last failure of the calling thread.
  *  - Inputs and outputs must not overlap in memory (ACS_ERR_ALIAS).
+ *  - The saturated kernels add neighbours in 64-bit fixed point, with one exponent per block of
+ *    planes, where the values' ranges allow it, and in FP64 elsewhere. Results are as near to the
+ *    exact value as FP64's or nearer; their last bits may depend on the launch shape.
  *  - The saturated RHS computes 1/rho with a refined hardware reciprocal estimate for
  *    normal |rho| in [2^-1000, 2^1001), faithful (within 1 ulp of the correctly rounded 1/rho),
  *    and falls back to an IEEE division otherwise.
@@ -151,15 +154,18 @@ acs_status acs_rhs_plain(const double *U, double *R, const acs_grid *g, const ac
 /*
  * acs_rhs_saturated - the saturated RHS: per-point fluxes computed once and shared with
  * the six neighbours, one reciprocal per point, dissipation reassociated as
- * sum(U at +-2) - 4 sum(U at +-1) + 18 U, FMA throughout, and every plane of U staged in
- * shared memory ahead of the arithmetic (bulk load). With equal spacing on the three axes
- * (h within 2^-65 .. 2^63) the library's kernel folds -1/(2h) into the fluxes where they are
- * formed (114 FP64 operations per point instead of 116); both forms equal the as-written
- * definition over the reals and differ from it only by rounding. Same arguments as
- * acs_rhs_plain plus
+ * sum(U at +-2) - 4 sum(U at +-1) + 18 U, and every plane of U staged in shared memory ahead of
+ * the arithmetic (bulk load). Grids of more than two planes per resident block with positive spacing
+ * and dissipation form the fluxes in FP64 (23 operations per point with equal spacing, 30 without)
+ * and the differences and the dissipation in fixed point, in blocks whose values' ranges suit it; the
+ * others run in FP64 throughout (114 operations with equal spacing within 2^-65 .. 2^63, where -1/(2h)
+ * is folded into the fluxes, else 116). All forms equal the as-written definition over the reals
+ * and differ from it only by rounding. Same arguments as acs_rhs_plain plus
  *   tile     launch shape or NULL (the autotuned shape for this grid size if acs_autotune_rhs
  *            recorded one, else 16 x 16 with the balanced schedule and TMA plane staging where
- *            the layout allows it).
+ *            the layout allows it). The fixed-point kernel is built for 16 x 16 columns and takes the
+ *            schedule and the staging of any tile, but on grids that fill such columns much worse
+ *            than the tile's.
  *   variant  NULL for the library's own saturated kernel, or a march-scope rewriter variant
  *            (acs_variant_generate with ACS_SCOPE_MARCH, acs_variant_build), for instance the
  *            one the learned ranker put first (acs_variant_rank). A variant is compiled for its
@@ -213,11 +219,13 @@ acs_status acs_stencil_plain(const double *u, const double *a, double *out, cons
 /*
  * acs_stencil_saturated - the saturated star stencil:
  *   out = a(p) * (C0 u(p) + sum_d sum_o c[d][o] (u(p+o e_d) + u(p-o e_d))),
- *   C0 = -2 sum c (folded on the host), FMA throughout, u planes staged in shared memory
- *   and reused by the 9 z-offsets as the block marches along z.
+ *   C0 = -2 sum c (folded on the host), u planes staged in shared memory and reused by the 9
+ *   z-offsets as the block marches along z. Weights of alternating sign (second-derivative weights
+ *   of every order) are summed exactly in block-scaled 64-bit fixed point and rounded once, others in
+ *   FP64 with FMA throughout; points and blocks whose values do not fit the scale fall back to FP64.
  *   tile   launch shape or NULL (the autotuned shape for this grid size if
- *          acs_autotune_stencil recorded one, else 32 x 8, z-chunks from the grid size, TMA
- *          plane staging where the layout allows it).
+ *          acs_autotune_stencil recorded one, else a shape by weights and layout, z-chunks from the
+ *          grid size, TMA plane staging where the layout allows it).
  */
 acs_status acs_stencil_saturated(const double *u, const double *a, double *out, const acs_grid *g,
                                  const double *c, const acs_tile *tile, acs_stream stream);

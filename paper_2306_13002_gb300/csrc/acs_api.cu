@@ -375,6 +375,17 @@ acs_status batch_params(int kind, const void* params, RhsConst& rk, StarCoef& sc
 
 const acs_tile kDefaultRhsTile = {16, 16, 0, ACS_TILE_BALANCED | ACS_TILE_TMA};
 const acs_tile kDefaultStarTile = {32, 8, 0, ACS_TILE_TMA};
+// The star stencil's tile without one asked for. Fixed-point march, 32 x 8 / 16 x 8 / 16 x 16: same weights
+// on every axis and tensor copies 605 / 591 / 601 us at 384^3 (4.49 / 4.38 / 4.47 ms at 768^3), element-wise
+// 660 / 699 / 679; weights of its own per axis 876 / 902 / 860 (6.57 / 6.73 / 6.45 ms).
+acs_tile default_star_tile(const Geom& g, const StarCoef& cf, const double* u) {
+    StarFix fx;
+    star_fix(cf, fx);
+    const bool copies = ((g.isy | g.isz | g.halo) & 1) == 0 && (uintptr_t)u % 16 == 0;
+    if (fx.kind == 2) return acs_tile{16, 16, 0, ACS_TILE_TMA};
+    if (fx.kind == 1 && copies) return acs_tile{16, 8, 0, ACS_TILE_TMA};
+    return kDefaultStarTile;
+}
 // Batches: the marches start a few planes before their first result, so chunks are long (64 star grids:
 // 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 607 us with chunks of
 // 24, 605 with 16, 672 with 8); batches with less work take shorter ones (batch_pack).
@@ -500,7 +511,7 @@ acs_status acs_stencil_saturated(const double* u, const double* a, double* out, 
     acs_status st = check_star(u, a, out, g, c, geo, cf);
     if (st != ACS_OK) return st;
     acs_tile t;
-    st = check_tile(tile, kDefaultStarTile, star_tile_supported, t, ACS_KIND_STENCIL, &geo);
+    st = check_tile(tile, default_star_tile(geo, cf, u), star_tile_supported, t, ACS_KIND_STENCIL, &geo);
     if (st != ACS_OK) return st;
     return launch_stencil_saturated(u, a, out, geo, cf, t, (cudaStream_t)stream);
 }

@@ -1,4 +1,6 @@
-// Saturated RHS of the compressible Euler equations with 4th-order dissipation.
+// Saturated RHS of the compressible Euler equations with 4th-order dissipation: the FP64 march, which
+// small grids and unusual parameters take, and the choice between it and the fixed-point one
+// (rhs_fixed.cuh), which runs it where a block's values do not fit.
 //
 // Same value as the as-written loop body (rhs_plain.cu) up to rounding; the arithmetic is
 // the result of the paper's rewrites (Sec. V-A, Table I) and extraction with shared

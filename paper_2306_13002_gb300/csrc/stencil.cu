@@ -5,7 +5,8 @@
 // As-written: one thread per point, the twelve terms in statement order, each reloading
 // a(p) and u(p) and multiplying by a(p) separately.
 //
-// Saturated (Table I rules plus bulk load, Sec. VI-B):
+// Saturated (Table I rules plus bulk load, Sec. VI-B; FP64, for weights the fixed-point march of
+// star_fixed.cuh does not take):
 //   out(p) = a(p) * (C0 u(p) + sum_d sum_o c[d][o] (u(p+o e_d) + u(p-o e_d))),
 //   C0 = -2 sum c  (folded on the host: constant folding),
 // i.e. the common factor a(p) is pulled out of the twelve terms (distributivity expressed
