@@ -83,7 +83,7 @@ struct RhsFixShape {
     static constexpr int FX = 4 * BY * (BX + 2), FY = 4 * (BY + 2) * BX;
     static constexpr int CONST_ELEMS = 16;
     // ... constants of the launch, mbarriers, the scan's results, constants of the segment
-    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * CELLS + FX + FY + CONST_ELEMS + NSLOT + 4 + 10);
+    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * CELLS + FX + FY + CONST_ELEMS + NSLOT + 4 + 10 + 3);
     static constexpr int MINB = NT <= 128 ? 4 : 2;
     static_assert((CELLS * sizeof(u64)) % 128 == 0, "every ring slot 128-byte aligned");
     static_assert(NT >= 2 * (BX + BY) && (2 * BX) % 32 == 0, "flux ring needs 2(BX+BY) threads, y-ring whole warps");
@@ -96,8 +96,9 @@ struct RhsScale {
     int join[3][4];               // rho, momenta, E: RhsJoin
     int cu[3], lo[3];             // conversion exponents of U, least exponents (none for the momenta)
     int cf[2];                    // conversion exponents of the momentum and energy fluxes
+    int seen[6];                  // exponent ranges of the planes marched so far (as the scan's; one spare)
 };
-static_assert(sizeof(RhsScale) == 80, "RhsFixShape reserves ten words");
+static_assert(sizeof(RhsScale) == 104, "RhsFixShape reserves thirteen words");
 
 // Shifts and exponent that join a component's flux sum a and dissipation d: z = (a >> sa) + (d >> sd),
 // in units of 2^e.
@@ -128,9 +129,11 @@ struct RhsFixMarch {
         return reinterpret_cast<uint64_t*>(smem + NSLOT * S::CELLS + S::FX + S::FY + S::CONST_ELEMS) + slot;
     }
 
+    __device__ __forceinline__ RhsScale* scales() const { return reinterpret_cast<RhsScale*>(bar(NSLOT) + 4); }
+
     // Marches from plane k0; returns the first plane not finished. `phase`, `flying`, `ok`: as
-    // StarFixMarch::segment. `room`: bits of headroom for the scales.
-    __device__ __forceinline__ int segment(int k0, int room, u32& phase, u32& flying, bool& ok) const {
+    // StarFixMarch::segment.
+    __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
         const int tid = threadIdx.y * BX + threadIdx.x;
         const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX * 8;
         int* note = reinterpret_cast<int*>(bar(NSLOT));   // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E
@@ -248,14 +251,30 @@ struct RhsFixMarch {
             }
         }
         if (!ok) note[0] = 0x7ff;
+        // The exponent ranges of the planes marched before, widened by this segment's: a flow that swings
+        // over a power of two then ends one segment by it, not one per swing.
+        RhsScale* const scale = scales();
+        int seen[5];
+#pragma unroll
+        for (int n = 0; n < 5; ++n) seen[n] = scale->seen[n];
         __syncthreads();
-        // Exponents: |rho| in [2^rlo, 2^rhi), |m| < 2^mhi, |E| in [2^elo, 2^ehi).
-        const int rhi = note[0] - 1022 + room, rlo = note[1] - 1023 - 1 - room, mhi = max(note[2], 1023 + rlo - 60) - 1022 + room,
-                  ehi = note[3] - 1022 + room, elo = note[4] - 1023 - 1 - room;
-        bool fits = note[0] < 0x7ff && note[2] < 0x7ff && note[3] < 0x7ff && abs(rhi) < 200 && abs(ehi) < 200 &&
-                    abs(mhi) < 200 && rhi - rlo <= 8 + 2 * room && ehi - elo <= 8 + 2 * room;
-        int efm = 0, efe = 0;
-        if (fits) {
+        // Exponents: |rho| in [2^rlo, 2^rhi), |m| < 2^mhi, |E| in [2^elo, 2^ehi), of all planes so far or,
+        // where these range too far, of the scanned ones.
+        int rhi = 0, rlo = 0, mhi = 0, ehi = 0, elo = 0, efm = 0, efe = 0;
+        bool fits = false;
+#pragma unroll 1
+        for (int t = 0; t < 2 && !fits; ++t) {
+#pragma unroll
+            for (int n = 0; n < 5; ++n)
+                seen[n] = t ? note[n] : n == 1 || n == 4 ? min(seen[n], note[n]) : max(seen[n], note[n]);
+            rhi = seen[0] - 1022;
+            rlo = seen[1] - 1023 - 1;
+            mhi = max(seen[2], 1023 + rlo - 60) - 1022;
+            ehi = seen[3] - 1022;
+            elo = seen[4] - 1023 - 1;
+            fits = seen[0] < 0x7ff && seen[2] < 0x7ff && seen[3] < 0x7ff && abs(rhi) < 200 && abs(ehi) < 200 &&
+                   abs(mhi) < 200 && rhi - rlo <= 8 && ehi - elo <= 8;
+            if (!fits) continue;
             // Bounds of the fluxes, and whether quantising against them stays below what FP64 rounds
             // anyway at the least rho and E: the dissipation (eps 18 U 2^-53) for the mass and energy
             // components, the pressure ((gamma - 1) E 2^-53) for the momenta.
@@ -278,7 +297,6 @@ struct RhsFixMarch {
         const int ur = rhi - 59, um = mhi - 59, ue = ehi - 59;
         const int dx = 2 + 1 + fx.ex_eps;   // dissipation / 4, mul63
         const int es = max(max(fx.ex_s[0], fx.ex_s[1]), fx.ex_s[2]);
-        RhsScale* const scale = reinterpret_cast<RhsScale*>(note + 8);
         const u32 sc = smem_addr(scale);
         if (tid == 0) {
             const RhsJoin j[3] = {rhs_join(um + 1 + es + (ISO ? 0 : 2), ur + dx), rhs_join(efm - 60, um + dx),
@@ -292,6 +310,7 @@ struct RhsFixMarch {
             }
             scale->cf[0] = cfm;
             scale->cf[1] = cfe;
+            for (int n = 0; n < 5; ++n) scale->seen[n] = seen[n];
         }
         __syncthreads();
 
@@ -501,6 +520,7 @@ __device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, do
     const int tid = threadIdx.y * BX + threadIdx.x;
     const RhsFixMarch<BX, BY, TMA, ISO> m{U, R, g, kc, fx, i0, j0, k1, smem, map, tmo};
     stage_consts_write(smem + S::NSLOT * S::CELLS + S::FX + S::FY, kc, tid);
+    if (tid < 5) m.scales()->seen[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
     if (TMA && tid == 0) {
         for (int s = 0; s < S::NSLOT; ++s) mbar_init(m.bar(s), 1);
         fence_mbar_init();
@@ -509,8 +529,8 @@ __device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, do
     u32 phase = 0, flying = 0;
     bool ok = !TMA || (smem_addr(smem) & 127u) == 0;
     int kk = k0;
-    for (int left = 4, room = 0; kk < k1 && ok; --left, room = 1) {
-        const int done = m.segment(kk, room, phase, flying, ok);
+    for (int left = 4; kk < k1 && ok; --left) {
+        const int done = m.segment(kk, phase, flying, ok);
         __syncthreads();   // shared memory is free again
         left += (done - kk) / 16;
         const bool stop = done == kk || left <= 0;
