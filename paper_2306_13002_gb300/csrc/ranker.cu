@@ -222,11 +222,17 @@ __global__ void __launch_bounds__(kTrainThreads)
         xs[e] = (X[e] - prm[L.mu + f]) / prm[L.sd + f];
     }
     auto load_model = [&]() {
+        // (unrolled, here and below, so that the trips to the L2 overlap)
+        float w2[H * H / kTrainThreads];
+#pragma unroll
+        for (int r = 0; r < H * H / kTrainThreads; ++r) w2[r] = __ldcg(prm + L.W2 + tid + r * kTrainThreads);
+#pragma unroll 4
         for (int e = tid; e < H * F; e += kTrainThreads) W1T[(e % F) * H + e / F] = __ldcg(prm + L.W1 + e);
-        for (int e = tid; e < H * H; e += kTrainThreads) {
-            const float w = __ldcg(prm + L.W2 + e);
-            W2[e] = w;
-            W2T[(e % H) * kTrainPad + e / H] = w;
+#pragma unroll
+        for (int r = 0; r < H * H / kTrainThreads; ++r) {
+            const int e = tid + r * kTrainThreads;
+            W2[e] = w2[r];
+            W2T[(e % H) * kTrainPad + e / H] = w2[r];
         }
         if (tid < H) {
             b1[tid] = __ldcg(prm + L.b1 + tid);
@@ -362,7 +368,9 @@ __global__ void __launch_bounds__(kTrainThreads)
         {
             float4* d = reinterpret_cast<float4*>(h1a);
             const float4* src = reinterpret_cast<const float4*>(H1);
+#pragma unroll 8
             for (int e = tid; e < n * H / 4; e += kTrainThreads) d[e] = __ldcg(src + e);
+#pragma unroll 4
             for (int e = tid; e < n * kTrainRows; e += kTrainThreads) {
                 const size_t at = (size_t)(e / kTrainRows) * H + j0 + e % kTrainRows;
                 c2[e] = __ldcg(DH2 + at);
