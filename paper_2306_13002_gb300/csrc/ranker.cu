@@ -166,9 +166,10 @@ __global__ void mlp_grad_adam(const float* __restrict__ X, const float* __restri
 //
 // The three launches per epoch took 100 us for 400 samples of 20 features (400 x 64 threads that wait on
 // L2 for every weight, then one thread per parameter over 400 samples): 203 ms for 2000 epochs, now
-// 46 ms. What bounds it now is latency: the sums' chains of 64 and 400 dependent additions, whose order
+// 40 ms. What bounds it now is latency: the sums' chains of 64 and 400 dependent additions, whose order
 // is kept, and two cluster barriers with a trip through the L2 per epoch.
 constexpr int kTrainBlocks = 8, kTrainThreads = 512, kTrainH = 64, kTrainRows = kTrainH / kTrainBlocks;
+constexpr int kSamples = 4;               // samples a thread works on at once
 constexpr int kTrainPad = kTrainH + 1;   // row pitch of the activations a thread reads along
 
 struct TrainShape {
@@ -181,11 +182,11 @@ struct TrainShape {
         cols = all + ((size_t)n * kTrainH > own ? (size_t)n * kTrainH : own);   // own columns of DH2, DH1, H2
         cols = (cols + 3) & ~(size_t)3;
         dy = cols + (size_t)n * 3 * kTrainRows;
-        w1t = dy + n;                            // W1 transposed, W2, W2 transposed, b1 b2 w3 b3
+        w1t = dy + n;                            // W1 transposed, W2, W2 transposed, b1 b2 w3 b3 and a one
         w2 = w1t + (size_t)F * kTrainH;
         w2t = w2 + kTrainH * kTrainH;
         vec = w2t + kTrainH * kTrainPad;
-        floats = vec + 3 * kTrainH + 1;
+        floats = vec + 3 * kTrainH + 2;
     }
 };
 
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(kTrainThreads)
         }
         if (tid == 0) b3[0] = __ldcg(prm + L.b3);
     };
+    if (tid == 0) b3[1] = 1.f;
     load_model();
 
     // The parameters of this block: rows [j0, j0 + 8) of W1, W2, b1, b2 and of w3 (block 0 also b3).
@@ -268,74 +270,109 @@ __global__ void __launch_bounds__(kTrainThreads)
     __syncthreads();
     cluster.sync();   // nobody updates a parameter before all blocks have read the model
 
-    const int j = tid % H, grp = tid / H;
-    constexpr int G = kTrainThreads / H;   // samples worked on at once
-    // a[i] += sum_k w[k][j] v[s_i][k], k in order; four of v at a time (one value serves a whole warp)
-    auto along = [&](const float* w, int pitch, const float* v, float (&a)[8], int base) {
+    // A thread works on hidden units j and j + 32 of four samples: a sample's value serves a whole warp but
+    // takes as long to fetch as 32 different ones, so it is used twice (eight samples of one unit: 6100
+    // cycles a layer).
+    const int j = tid % 32, grp = tid / 32;
+    constexpr int G = kTrainThreads / 32;   // samples worked on at once
+    // a[u][i] += sum_k w[k][j + 32 u] v[s_i][k], k in order; four of v at a time
+    auto along = [&](const float* w, int pitch, const float* v, float (&a)[2][kSamples], int base) {
 #pragma unroll 4
         for (int k = 0; k < H; k += 4) {
-            const float w0 = w[k * pitch + j], w1 = w[(k + 1) * pitch + j], w2 = w[(k + 2) * pitch + j], w3k = w[(k + 3) * pitch + j];
+            float wk[2][4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int q = 0; q < 4; ++q) {
+                wk[0][q] = w[(k + q) * pitch + j];
+                wk[1][q] = w[(k + q) * pitch + j + 32];
+            }
+#pragma unroll
+            for (int i = 0; i < kSamples; ++i) {
                 const float4 x = *reinterpret_cast<const float4*>(v + min(base + grp + i * G, ns - 1) * H + k);
-                a[i] += w0 * x.x;
-                a[i] += w1 * x.y;
-                a[i] += w2 * x.z;
-                a[i] += w3k * x.w;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    a[u][i] += wk[u][0] * x.x;
+                    a[u][i] += wk[u][1] * x.y;
+                    a[u][i] += wk[u][2] * x.z;
+                    a[u][i] += wk[u][3] * x.w;
+                }
             }
         }
     };
     for (int ep = 1; ep <= epochs; ++ep) {
-        // Forward and backward passes of the block's samples, a thread per hidden unit.
-        for (int base = 0; base < ns; base += 8 * G) {   // (up to eight samples per thread at a time)
-            float a[8], r1[8], r2[8];
+        // Forward and backward passes of the block's samples.
+        for (int base = 0; base < ns; base += kSamples * G) {
+            float a[2][kSamples], r1[2][kSamples], r2[2][kSamples];
+            int at[kSamples];   // (rows of samples past the block's own are read as its last and not used)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) a[i] = b1[j];
-            // (rows of samples past the block's own are read, inside shared memory, and not used)
+            for (int i = 0; i < kSamples; ++i) {
+                at[i] = (s_lo + min(base + grp + i * G, ns - 1)) * F;
+                a[0][i] = b1[j];
+                a[1][i] = b1[j + 32];
+            }
             int f = 0;
             if (F % 4 == 0) {
+#pragma unroll 5
                 for (; f < F; f += 4) {
-                    const float w0 = W1T[f * H + j], w1 = W1T[(f + 1) * H + j], w2 = W1T[(f + 2) * H + j], w3f = W1T[(f + 3) * H + j];
+                    float wf[2][4];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int s = min(base + grp + i * G, ns - 1);
-                        const float4 x = *reinterpret_cast<const float4*>(xs + (size_t)(s_lo + s) * F + f);
-                        a[i] += w0 * x.x;
-                        a[i] += w1 * x.y;
-                        a[i] += w2 * x.z;
-                        a[i] += w3f * x.w;
+                    for (int q = 0; q < 4; ++q) {
+                        wf[0][q] = W1T[(f + q) * H + j];
+                        wf[1][q] = W1T[(f + q) * H + j + 32];
+                    }
+#pragma unroll
+                    for (int i = 0; i < kSamples; ++i) {
+                        const float4 x = *reinterpret_cast<const float4*>(xs + at[i] + f);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            a[u][i] += wf[u][0] * x.x;
+                            a[u][i] += wf[u][1] * x.y;
+                            a[u][i] += wf[u][2] * x.z;
+                            a[u][i] += wf[u][3] * x.w;
+                        }
                     }
                 }
             }
             for (; f < F; ++f) {
-                const float w = W1T[f * H + j];
+                const float w0 = W1T[f * H + j], w1 = W1T[f * H + j + 32];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] += w * xs[(size_t)(s_lo + min(base + grp + i * G, ns - 1)) * F + f];
+                for (int i = 0; i < kSamples; ++i) {
+                    const float x = xs[at[i] + f];
+                    a[0][i] += w0 * x;
+                    a[1][i] += w1 * x;
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < kSamples; ++i) {
                 const int s = base + grp + i * G;
-                r1[i] = a[i] > 0.f ? a[i] : 0.f;
-                if (s < ns) {
-                    h1o[s * H + j] = r1[i];
-                    H1[(size_t)(s_lo + s) * H + j] = r1[i];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int ju = j + 32 * u;
+                    r1[u][i] = a[u][i] > 0.f ? a[u][i] : 0.f;
+                    if (s < ns) {
+                        h1o[s * H + ju] = r1[u][i];
+                        H1[(size_t)(s_lo + s) * H + ju] = r1[u][i];
+                    }
+                    a[u][i] = b2[ju];
                 }
-                a[i] = b2[j];
             }
             __syncthreads();
             along(W2T, kTrainPad, h1o, a, base);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < kSamples; ++i) {
                 const int s = base + grp + i * G;
-                r2[i] = a[i] > 0.f ? a[i] : 0.f;
-                if (s < ns) {
-                    h2o[s * kTrainPad + j] = r2[i];
-                    H2[(size_t)(s_lo + s) * H + j] = r2[i];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int ju = j + 32 * u;
+                    r2[u][i] = a[u][i] > 0.f ? a[u][i] : 0.f;
+                    if (s < ns) {
+                        h2o[s * kTrainPad + ju] = r2[u][i];
+                        H2[(size_t)(s_lo + s) * H + ju] = r2[u][i];
+                    }
                 }
             }
             __syncthreads();
             const int sy = base + tid;
-            if (tid < 8 * G && sy < ns) {
+            if (tid < kSamples * G && sy < ns) {
                 float y = b3[0];
 #pragma unroll 8
                 for (int k = 0; k < H; ++k) y += w3[k] * h2o[sy * kTrainPad + k];
@@ -345,37 +382,43 @@ __global__ void __launch_bounds__(kTrainThreads)
             }
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < kSamples; ++i) {
                 const int s = base + grp + i * G;
-                if (s < ns) {
-                    const float gq = r2[i] > 0.f ? dyo[s] * w3[j] : 0.f;
-                    d2o[s * H + j] = gq;
-                    DH2[(size_t)(s_lo + s) * H + j] = gq;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int ju = j + 32 * u;
+                    if (s < ns) {
+                        const float gq = r2[u][i] > 0.f ? dyo[s] * w3[ju] : 0.f;
+                        d2o[s * H + ju] = gq;
+                        DH2[(size_t)(s_lo + s) * H + ju] = gq;
+                    }
+                    a[u][i] = 0.f;
                 }
-                a[i] = 0.f;
             }
             __syncthreads();
             along(W2, H, d2o, a, base);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < kSamples; ++i) {
                 const int s = base + grp + i * G;
-                if (s < ns) DH1[(size_t)(s_lo + s) * H + j] = r1[i] > 0.f ? a[i] : 0.f;
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (s < ns) DH1[(size_t)(s_lo + s) * H + j + 32 * u] = r1[u][i] > 0.f ? a[u][i] : 0.f;
             }
             __syncthreads();
         }
         cluster.sync();
-        // Activations of all samples: H1 whole, the block's columns of the others.
+        // Activations of all samples: H1 whole, the block's columns of the others (their copies follow each
+        // other in shared memory), as one list of 16-byte pieces, so that the trips to the L2 overlap.
         {
-            float4* d = reinterpret_cast<float4*>(h1a);
-            const float4* src = reinterpret_cast<const float4*>(H1);
-#pragma unroll 8
-            for (int e = tid; e < n * H / 4; e += kTrainThreads) d[e] = __ldcg(src + e);
-#pragma unroll 4
-            for (int e = tid; e < n * kTrainRows; e += kTrainThreads) {
-                const size_t at = (size_t)(e / kTrainRows) * H + j0 + e % kTrainRows;
-                c2[e] = __ldcg(DH2 + at);
-                c1[e] = __ldcg(DH1 + at);
-                ch[e] = __ldcg(H2 + at);
+            constexpr int CQ = kTrainRows / 4;
+            const int nh = n * (H / 4), nc = n * CQ, total = nh + 3 * nc;
+#pragma unroll 9
+            for (int e = tid; e < total; e += kTrainThreads) {
+                const int r = e - nh, q = (r >= nc) + (r >= 2 * nc), p = r - q * nc;
+                const float* src = r < 0 ? H1 + 4 * (size_t)e
+                                         : (q == 0 ? DH2 : q == 1 ? DH1 : H2) + (size_t)(p / CQ) * H + j0 + 4 * (p % CQ);
+                *reinterpret_cast<float4*>(r < 0 ? h1a + 4 * (size_t)e : c2 + 4 * (size_t)r) =
+                    __ldcg(reinterpret_cast<const float4*>(src));
             }
             for (int e = tid; e < n; e += kTrainThreads) dyv[e] = __ldcg(DY + e);
         }
@@ -401,22 +444,27 @@ __global__ void __launch_bounds__(kTrainThreads)
             for (int r = 0; r < kMost; ++r) {
                 const int o = tid - 128 + r * kOther, q = o - kTrainRows * F;
                 if (o >= others) continue;
-                float g = 0.f;
+                // g = sum_s x y over the samples; y is 1 for the biases (the same bits as adding x). One loop
+                // for all of them: a warp that took the four kinds by turns was the last by 5000 cycles.
+                const float *x, *y = b3 + 1;
+                int ix = kTrainRows, iy = 0;
                 if (q < 0) {
-                    const int f = o % F, jl = o / F;
-#pragma unroll 8
-                    for (int s = 0; s < n; ++s) g += c1[s * kTrainRows + jl] * xs[s * F + f];
+                    x = c1 + o / F;
+                    y = xs + o % F;
+                    iy = F;
                 } else if (q < 2 * kTrainRows) {
-                    const float* c = q < kTrainRows ? c1 + q : c2 + q - kTrainRows;
-#pragma unroll 8
-                    for (int s = 0; s < n; ++s) g += c[s * kTrainRows];
-                } else if (q < 3 * kTrainRows) {
-#pragma unroll 8
-                    for (int s = 0; s < n; ++s) g += dyv[s] * ch[s * kTrainRows + q - 2 * kTrainRows];
+                    x = q < kTrainRows ? c1 + q : c2 + q - kTrainRows;
                 } else {
-#pragma unroll 8
-                    for (int s = 0; s < n; ++s) g += dyv[s];
+                    x = dyv;
+                    ix = 1;
+                    if (q < 3 * kTrainRows) {
+                        y = ch + q - 2 * kTrainRows;
+                        iy = kTrainRows;
+                    }
                 }
+                float g = 0.f;
+#pragma unroll 8
+                for (int s = 0; s < n; ++s) g += x[s * ix] * y[s * iy];
                 pv[r] = adam_step(pv[r], mv[r], vv[r], g, ep, lr);
                 prm[po[r]] = pv[r];
             }
