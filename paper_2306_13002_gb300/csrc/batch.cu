@@ -179,14 +179,22 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     // the blocks run out of work closer together.
     const long long waves = 2LL * resident;
     const int tail_kchunk = std::min(kc, std::max(plain ? 1 : 4, kc / 4));
-    std::vector<int> kchunk(n, kc);
+    // The fixed-point RHS march starts four planes early, so a grid's planes are split evenly instead of
+    // leaving a last chunk of a few planes: 32 grids with sides of 16 to 96 611 -> 592 us, 20 of 60 to 96
+    // 1283 -> 1234 us, smaller batches and the star stencil within 1 % either way.
+    auto split = [&](int q, int c) {
+        const int m = (geo[q].nz + c - 1) / c;
+        return rhs && !plain ? (geo[q].nz + m - 1) / m : c;
+    };
+    std::vector<int> kchunk(n);
+    for (int q = 0; q < n; ++q) kchunk[q] = split(q, kc);
     std::vector<long long> units(n);
     long long tail = 0;
     for (int r = n - 1; r >= 0; --r) {
         const int q = order[r];
-        tail += unit_count(q, tail_kchunk);
+        tail += unit_count(q, split(q, tail_kchunk));
         if (tail > waves) break;
-        kchunk[q] = tail_kchunk;
+        kchunk[q] = split(q, tail_kchunk);
     }
     for (int q = 0; q < n; ++q) units[q] = unit_count(q, kchunk[q]);
     image.assign(batch_ws_bytes(n), 0);
