@@ -132,7 +132,7 @@ __device__ __forceinline__ double twice(double v) {
 // four FP64 operations per entry (the doubling is exact and integer) against six with a thread per
 // output point. The loop-invariant products are folded once and held in registers like the Pipe
 // constants, and every add, subtract and multiply is issued as an FMA (Pipe).
-// FP64-bound before and after: 128^3, 167 -> 119.5 operations per point, 584 -> 440 us (96 % of the pipe),
+// FP64-bound before and after: 128^3, 167 -> 119.5 operations per point, 584 -> 440 us (90 % of the pipe),
 // 64^3 84 -> 66 us. The register bound (four 256-thread blocks per SM, 64 registers) is tuned:
 // 2 / 3 / 4 / 5 / 6 / 8 blocks ran 641 / 495 / 440 / 450 / 494 / 496 us.
 __global__ void __launch_bounds__(256, 4) block_saturated_kernel(const double* __restrict__ A,

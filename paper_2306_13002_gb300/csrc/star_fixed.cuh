@@ -10,7 +10,7 @@
 // Measured on GB300, tensor copies: 384^3 with 16 x 8 tiles 2388 us in FP64 (26 operations per point, 98 %
 // of the FP64 pipe) -> 591 us; 768^3 with distinct weights per axis 19.0 -> 6.45 ms. Error against
 // 64 bits (2-norm): uniform values 3.1e-16 -> 8.1e-17, a smooth wave 5.8e-15 -> 9.6e-17. What bounds it
-// now: about 230 instructions per point (124 on the ALU pipe, 57 on the FMA pipe) issued at half of
+// now: about 240 instructions per point (130 on the ALU pipe, 63 on the FMA pipe) issued at 55 % of
 // the peak rate, 16 warps per SM at 128 registers waiting on each other's results; launch bounds for
 // more warps spill and run 1.1 to 2 times longer. The 2 FP64 additions and one multiplication left
 // per point take 40 % of the FP64 pipe, memory 1.4 GB at a third of its rate.
