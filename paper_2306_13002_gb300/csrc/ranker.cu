@@ -166,7 +166,7 @@ __global__ void mlp_grad_adam(const float* __restrict__ X, const float* __restri
 //
 // The three launches per epoch took 100 us for 400 samples of 20 features (400 x 64 threads that wait on
 // L2 for every weight, then one thread per parameter over 400 samples): 203 ms for 2000 epochs, now
-// 40 ms. What bounds it now is latency: the sums' chains of 64 and 400 dependent additions, whose order
+// 38 ms. What bounds it now is latency: the sums' chains of 64 and 400 dependent additions, whose order
 // is kept, and two cluster barriers with a trip through the L2 per epoch.
 constexpr int kTrainBlocks = 8, kTrainThreads = 512, kTrainH = 64, kTrainRows = kTrainH / kTrainBlocks;
 constexpr int kSamples = 4;               // samples a thread works on at once
@@ -412,13 +412,22 @@ __global__ void __launch_bounds__(kTrainThreads)
         {
             constexpr int CQ = kTrainRows / 4;
             const int nh = n * (H / 4), nc = n * CQ, total = nh + 3 * nc;
-#pragma unroll 9
-            for (int e = tid; e < total; e += kTrainThreads) {
-                const int r = e - nh, q = (r >= nc) + (r >= 2 * nc), p = r - q * nc;
-                const float* src = r < 0 ? H1 + 4 * (size_t)e
-                                         : (q == 0 ? DH2 : q == 1 ? DH1 : H2) + (size_t)(p / CQ) * H + j0 + 4 * (p % CQ);
-                *reinterpret_cast<float4*>(r < 0 ? h1a + 4 * (size_t)e : c2 + 4 * (size_t)r) =
-                    __ldcg(reinterpret_cast<const float4*>(src));
+            constexpr int NB = 6;
+            for (int e0 = tid; e0 < total; e0 += NB * kTrainThreads) {
+                float4 x[NB];
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    const int e = e0 + i * kTrainThreads;
+                    const int r = e - nh, q = (r >= nc) + (r >= 2 * nc), p = r - q * nc;
+                    const float* src = r < 0 ? H1 + 4 * (size_t)e
+                                             : (q == 0 ? DH2 : q == 1 ? DH1 : H2) + (size_t)(p / CQ) * H + j0 + 4 * (p % CQ);
+                    if (e < total) x[i] = __ldcg(reinterpret_cast<const float4*>(src));
+                }
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    const int e = e0 + i * kTrainThreads;
+                    if (e < total) *reinterpret_cast<float4*>(e < nh ? h1a + 4 * (size_t)e : c2 + 4 * (size_t)(e - nh)) = x[i];
+                }
             }
             for (int e = tid; e < n; e += kTrainThreads) dyv[e] = __ldcg(DY + e);
         }
