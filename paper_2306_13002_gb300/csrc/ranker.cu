@@ -271,8 +271,8 @@ __global__ void __launch_bounds__(kTrainThreads)
     cluster.sync();   // nobody updates a parameter before all blocks have read the model
 
     // A thread works on hidden units j and j + 32 of four samples: a sample's value serves a whole warp but
-    // takes as long to fetch as 32 different ones, so it is used twice (eight samples of one unit: 6100
-    // cycles a layer).
+    // takes as long to fetch as 32 different ones, so it is used twice (5000 cycles a layer; eight samples of
+    // one unit: 6100).
     const int j = tid % 32, grp = tid / 32;
     constexpr int G = kTrainThreads / 32;   // samples worked on at once
     // a[u][i] += sum_k w[k][j + 32 u] v[s_i][k], k in order; four of v at a time
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kTrainThreads)
                 const int o = tid - 128 + r * kOther, q = o - kTrainRows * F;
                 if (o >= others) continue;
                 // g = sum_s x y over the samples; y is 1 for the biases (the same bits as adding x). One loop
-                // for all of them: a warp that took the four kinds by turns was the last by 5000 cycles.
+                // for all of them: a warp that holds several kinds would run them by turns.
                 const float *x, *y = b3 + 1;
                 int ix = kTrainRows, iy = 0;
                 if (q < 0) {

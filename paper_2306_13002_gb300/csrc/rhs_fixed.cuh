@@ -499,7 +499,9 @@ struct RhsFixMarch {
                         for (int c = 0; c < 5; ++c) old[c] = lds1(back(3) + own + c * PLANE * 8);
                     }
                 }
-                if (fluxer && z_plane(q + 1)) own_flux(sn);
+                // (Of the planes before and after the segment only points of the tile: their edges are not
+                // staged, and an empty cell's flux would end the segment.)
+                if (xy_plane(q + 1) ? fluxer : active && z_plane(q + 1)) own_flux(sn);
             }
             cur = nslot;
         }
