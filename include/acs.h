@@ -271,7 +271,7 @@ size_t acs_batch_workspace_bytes(int n);
  * would, including the alias check), order them largest first, and upload the unit table
  * into `ws` (16-byte aligned device memory of at least acs_batch_workspace_bytes(n) bytes:
  * ACS_ERR_ALIGN / ACS_ERR_WORKSPACE otherwise). `tile` NULL = 16 x 8 with z-chunks of 32
- * planes and ACS_TILE_TMA (star stencil) or 16 x 16 with z-chunks of 24 (RHS; the columns of an RHS
+ * planes and ACS_TILE_TMA (star stencil) or 16 x 16 with z-chunks of 32 (RHS; the columns of an RHS
  * batch are 16 x 16 whatever the tile); tile->flags may be ACS_TILE_TMA for a star-stencil batch,
  * which encodes a tensor map per grid into the workspace if every grid of the batch can be staged so
  * (even row and plane pitch, 16-byte aligned; otherwise all are staged element-wise). Long z-chunks

@@ -387,10 +387,10 @@ acs_tile default_star_tile(const Geom& g, const StarCoef& cf, const double* u) {
     return kDefaultStarTile;
 }
 // Batches: the marches start a few planes before their first result, so chunks are long (64 star grids:
-// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 607 us with chunks of
-// 24, 605 with 16, 672 with 8); batches with less work take shorter ones (batch_pack).
+// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 397 us with chunks of
+// 32, 412 with 24, 434 with 16, 496 with 8); batches with less work take shorter ones (batch_pack).
 acs_tile default_batch_tile(int kind, int staging) {
-    return kind == ACS_KIND_STENCIL ? acs_tile{16, 8, 32, staging} : acs_tile{16, 16, 24, 0};
+    return kind == ACS_KIND_STENCIL ? acs_tile{16, 8, 32, staging} : acs_tile{16, 16, 32, 0};
 }
 
 acs_status check_tile(const acs_tile* t, const acs_tile& def, bool (*supported)(int, int), acs_tile& out,

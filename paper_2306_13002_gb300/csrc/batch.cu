@@ -161,7 +161,7 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     // z-chunks of a batch with little work are shortened, so that the queue still holds a few units per
     // resident block (RHS: two; star stencil, whose blocks are smaller: one) but no shorter than what a
     // unit's start is worth. 8 RHS grids with sides of 16 to 96: chunks of 24 / 16 / 8 / 6 ran 404 / 297 /
-    // 206 / 205 us, 16 grids 410 / 302 / 311 / 328; 8 star grids 32 / 16 / 8: 72 / 57 / 62 us.
+    // 206 / 205 us, 16 grids 410 / 302 / 311 / 328 (by this rule and with the march as it is now 149 and 223); 8 star grids 32 / 16 / 8: 72 / 57 / 62 us.
     const long long resident = resident_batch_blocks(kind, tile);
     auto unit_count = [&](int q, int kc) {
         const Geom& g = geo[q];
@@ -181,7 +181,8 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     const int tail_kchunk = std::min(kc, std::max(plain ? 1 : 4, kc / 4));
     // The fixed-point RHS march starts four planes early, so a grid's planes are split evenly instead of
     // leaving a last chunk of a few planes: 32 grids with sides of 16 to 96 611 -> 592 us, 20 of 60 to 96
-    // 1283 -> 1234 us, smaller batches and the star stencil within 1 % either way.
+    // 1283 -> 1234 us (with cut tiles still in the FP64 march, 398 and 881 us now), smaller batches and the
+    // star stencil within 1 % either way.
     auto split = [&](int q, int c) {
         const int m = (geo[q].nz + c - 1) / c;
         return rhs && !plain ? (geo[q].nz + m - 1) / m : c;

@@ -13,8 +13,8 @@
 // must not lose their low bits); the fluxes' scales follow from these bounds. A plane that leaves
 // the ranges ends the segment.
 //
-// Measured on GB300: 256^3 3237 us in FP64 (114 operations per point, 94 % of the FP64 pipe) -> 1151 us
-// (element-wise staging 1268), three spacings 3270 -> 1384, 162^3 with three spacings 999 -> 439, 512^3 of a
+// Measured on GB300: 256^3 3237 us in FP64 (114 operations per point, 94 % of the FP64 pipe) -> 1160 us
+// (element-wise staging 1268), three spacings 3270 -> 1384, 162^3 with three spacings 999 -> 441, 512^3 of a
 // smooth flow 25.7 -> 8.5 ms, 128^3 420 -> 178. Error against 64 bits (2-norm): uniform state 2.2e-16 ->
 // 4.9e-17, smooth flow 2.4e-15 -> 5.7e-16. What bounds it now: a warp's own chains. About 1200
 // instructions per point (29 of them FP64, ring included: 67 % of that pipe's time) issue at 44 % of
