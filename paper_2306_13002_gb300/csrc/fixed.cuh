@@ -66,17 +66,23 @@ __device__ __forceinline__ u32 hi32(u64 v) { return (u32)(v >> 32); }
 __device__ __forceinline__ u32 lo32(u64 v) { return (u32)v; }
 
 // The bits v of a double as fixed point: floor(v / d) + (bias_hi << 32), its leading bit at 59 for the
-// exponent E0 (an exact negative multiple of d comes out one lower). `bad` turns negative if v's
-// exponent exceeds E0 (infinities and NaN do). Zeros and values too small for the scale give 0 or -1.
-// E0 >= kFixMinExp.
-__device__ __forceinline__ u64 to_fixed(u64 v, int E0, u32 bias_hi, int& bad) {
+// exponent E0 (an exact negative multiple of d comes out one lower). s: the bits between v's exponent
+// and E0, negative if it exceeds E0 (infinities and NaN do). Zeros and values too small for the scale
+// give 0 or -1. E0 >= kFixMinExp.
+__device__ __forceinline__ u64 to_fixed_by(u64 v, int E0, u32 bias_hi, int& s) {
     const u32 hi = hi32(v), lo = lo32(v);
-    const int s = E0 - (int)((hi << 1) >> 21);
-    bad |= s;
+    s = E0 - (int)((hi << 1) >> 21);
     const u32 mh = (__funnelshift_l(lo, hi, 7) & 0x07ffffffu) | 0x08000000u;
     const u64 m = shr64(pack64(mh, lo << 7), s);
     const u32 sg = (u32)((int)hi >> 31);
     return pack64((hi32(m) ^ sg) + bias_hi, lo32(m) ^ sg);
+}
+// The same; `bad` turns negative if v's exponent exceeds E0.
+__device__ __forceinline__ u64 to_fixed(u64 v, int E0, u32 bias_hi, int& bad) {
+    int s;
+    const u64 r = to_fixed_by(v, E0, bias_hi, s);
+    bad |= s;
+    return r;
 }
 
 // Constants that turn a 64-bit integer t into the double t * 2^e2 (times -1 if `neg`): the two

@@ -137,7 +137,8 @@ struct RhsFixMarch {
     __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
         const int tid = threadIdx.y * BX + threadIdx.x;
         const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX * 8;
-        int* note = reinterpret_cast<int*>(bar(NSLOT));   // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E
+        // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E, [5] 1: a point's dissipation may not fit
+        int* note = reinterpret_cast<int*>(bar(NSLOT));
         // Tiles cut by the grid's edges: points packed as in rhs_march, one halo column more than the
         // valid ones; rows up to the one past the last valid row.
         const int w = min(BX, g.nx - i0), h = min(BY, g.ny - j0);
@@ -215,7 +216,7 @@ struct RhsFixMarch {
         // Prologue: the first six planes under way; exponent ranges of the first five.
         int next = k0 - 2;
         for (; next < k0 + 4 && next < k1 + 2; ++next) stage(next);
-        if (tid < 5) note[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
+        if (tid < 6) note[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
         __syncthreads();
         int rng[5] = {0, 0x7ff, 0, 0, 0x7ff};
         if (!TMA) cp_async_wait_all();
@@ -292,8 +293,10 @@ struct RhsFixMarch {
             for (int p = scanned; p < next - k0 + 2; ++p) landed(p);
             return k0;
         }
-        // Conversion exponents (leading bit at 59; one more bit of room for U, whose dissipation sums
-        // to 12 times its largest value) and the units of the sums.
+        // Conversion exponents (leading bit at 59) and the units of the sums. U has one more bit of room, so
+        // that a flow may double on the way: the dissipation, 6/4 + 6 + 4.5 times the largest value, is
+        // below 12 2^59 for values as scanned and for values of one sign (a negative rho or E ends the
+        // segment), and may need more than 63 bits for larger momenta of both (see roomy).
         const int cr = rhi + 1023, cm = mhi + 1023, ce = ehi + 1023, cfm = efm + 1022, cfe = efe + 1022;
         const int ur = rhi - 59, um = mhi - 59, ue = ehi - 59;
         const int dx = 2 + 1 + fx.ex_eps;   // dissipation / 4, mul63
@@ -426,6 +429,22 @@ struct RhsFixMarch {
 #pragma unroll
             for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
         };
+        // Whether the dissipation of this thread's momenta in plane q-2 has room for certain, from the upper
+        // halves of its values: 4.5 of the point's own and a quarter of the six at distance 2 are at most
+        // 12 2^59, so it takes six nearest values of the other sign that sum to 4 2^59 to exceed 2^63.
+        auto roomy = [&]() {
+            const u32 s0 = back(2) + own + 4, sm1 = back(3) + own + 4, sp1 = back(1) + own + 4;
+            bool all = true;
+#pragma unroll
+            for (int c = 1; c < 4; ++c) {
+                constexpr int C = PLANE * 8;
+                auto hi = [&](u32 a) { return lds_int(a + c * C); };
+                const int h1 = (hi(s0 - 8) + hi(s0 + 8) + hi(s0 - 8 * PX)) + (hi(s0 + 8 * PX) + hi(sm1) + hi(sp1));
+                all &= (hi(s0) ^ h1) >= 0 || abs(h1) < (4 << 27) - 8;   // (8: their lower halves)
+            }
+            return all;
+        };
+        bool wide = false;   // a momentum is larger than those scanned
         const bool whole = w == BX && h == BY;
 #pragma unroll 1
         for (; q < k1 + 2; ++q) {
@@ -451,6 +470,7 @@ struct RhsFixMarch {
                 }
             }
             if (q + 1 < k1 + 2 && q + 1 >= k0 + 3) landed(nslot);
+            bool grew = false;
             // The ring's fluxes of plane q+1 in FP64, beside the other threads' conversion of plane q.
             if (ring) {
                 if (xy_plane(q + 1)) ring_flux(sn);
@@ -467,22 +487,34 @@ struct RhsFixMarch {
                         if (!((m >> n) & 1u)) v[n] = kd == 1 ? 0ull : (u64)(u32)lds_int(sc + 60 + 4 * kd) << 52;
                     }
                 }
+                int room = 1;
 #pragma unroll
                 for (int n = 0; n < NE; ++n) {
                     const int kd = kind_of(n);
                     const int cu = lds_int(sc + 48 + 4 * kd);
                     if ((n + 1) * NC <= S::CELLS || cell + n * NC < S::CELLS) {
                         if ((n + 1) * NC > 4 * PLANE || n * NC < PLANE)
-                            bad |= (int)((hi32(v[n]) << 1) >> 21) - lds_int(sc + 60 + 4 * kd);
-                        sts1(sq + (cell + n * NC) * 8, to_fixed(v[n], cu, 0, bad));
+                            bad |= ((int)((hi32(v[n]) << 1) >> 21) - lds_int(sc + 60 + 4 * kd)) | (kd == 1 ? 0 : (int)hi32(v[n]));
+                        int s;
+                        sts1(sq + (cell + n * NC) * 8, to_fixed_by(v[n], cu, 0, s));
+                        bad |= s;
+                        if ((n + 1) * NC > PLANE && n * NC < 4 * PLANE) room = min(room, kd == 1 ? s : 1);
                     }
                 }
+                grew = room == 0 && !wide;
                 if (TMA) fence_proxy_async();
             }
             if (!ok) bad = -1;
             // Plane q in fixed point, its fluxes; a value out of range ends the segment before it is used.
-            if (__syncthreads_or(bad < 0)) break;
+            if (__syncthreads_or(bad < 0 || grew)) {
+                if (__syncthreads_or(bad < 0)) break;
+                wide = true;
+            }
             bad = 0;
+            if (wide && active && q - 2 >= k0 && !roomy()) {   // the next vote ends the segment, before this plane
+                note[5] = 1;
+                bad = -1;
+            }
             // Then plane q-2's result from integers and plane q+1's fluxes in FP64: independent, and in one
             // stretch of code where the whole tile takes part, so that the two pipes work at once.
             if (whole && q - 2 >= k0 && q + 1 < k1) {
@@ -505,10 +537,12 @@ struct RhsFixMarch {
             }
             cur = nslot;
         }
+        __syncthreads();
+        const int again = note[5];
         // Copies not waited for yet: planes after q + 1 that a segment cut short had under way.
         for (int p = max(q + 2, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
         if (!TMA) cp_async_wait_all();
-        return min(max(q - 2, k0), k1);
+        return min(max(q - 2 - again, k0), k1);
     }
 };
 
