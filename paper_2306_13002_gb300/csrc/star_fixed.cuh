@@ -137,8 +137,9 @@ struct StarFixMarch {
         const bool work = ty < h;
         const u32 rs = smem_addr(ring), mine = rs + ((ty + 4) * PX + tx + 4) * 8;
         const double* col0 = u + (i64)(k0 + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + g.halo);
-        auto below = [&](int q, int c) {   // the column's value q planes below k0
-            return valid(c) ? (u64)__double_as_longlong(__ldg(col0 - q * g.isz + c)) : 0ull;
+        auto below = [&](int q, int c) {   // the column's value q planes below k0 (0 for -0, which converts to -1)
+            const u64 v = valid(c) ? (u64)__double_as_longlong(__ldg(col0 - q * g.isz + c)) : 0ull;
+            return (v << 1) ? v : 0ull;
         };
         auto cells = [&](int slot, auto&& f) {   // f(bit, cell) over this thread's cells of a slot
             const u32 c = rs + (slot * PLANE + tid) * 8;

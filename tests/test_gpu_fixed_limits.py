@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from paper_2306_13002_gb300 import inputs
-from test_gpu_fixed import RHS_TILES, _check_rhs
+from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _star
 
 pytestmark = pytest.mark.gpu
 
@@ -29,3 +29,12 @@ def test_rhs_values_that_double_within_a_segment(signs, tile, dims, h):
     U[0], U[4] = 1.0, 8.0
     U[1:4] = s * np.where(z % 40 < 13, 0.95, 1.9)
     _check_rhs(U, tile, (signs, dims, h), h=h)
+
+
+@pytest.mark.parametrize("tile", TILES)
+def test_star_negative_zeros(tile):
+    """A field of zeros of both signs gives zeros."""
+    u = np.where(np.random.default_rng(33).random((29, 33, 45)) < 0.5, 0.0, -0.0)
+    a = np.random.default_rng(34).uniform(0.5, 1.5, u.shape)
+    assert not np.any(_star(u, a, TAYLOR, tile))
+    assert not np.any(_star(np.full(u.shape, -0.0), a, TAYLOR, tile))
