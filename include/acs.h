@@ -462,10 +462,11 @@ const char *acs_status_string(acs_status s);
 acs_status acs_wait_timeouts(unsigned int *count);
 
 /*
- * acs_wait_selftest - run the bounded-wait path once on the current device: one block of 32
- * threads, each waiting with the saturated kernels' own bounded wait (about one second of
+ * acs_wait_selftest - run the bounded-wait path once on the current device: one block of 64
+ * threads, 32 of them waiting with the saturated kernels' own bounded wait (about one second of
  * SM clock cycles) on an mbarrier phase that nothing completes, so every wait runs out. Writes
- * the number of waits that ran out to *timeouts (32 when the path works) and leaves the
+ * the number of waits that ran out to *timeouts, less the threads that then disagree about it (32
+ * when the path works), and leaves the
  * acs_wait_timeouts counter alone. No copy is issued, so nothing is left in flight. Enqueued on
  * `stream`, which it synchronises (takes about one second). ACS_ERR_INVALID for a NULL
  * timeouts, ACS_ERR_CUDA if the launch or the read fails.

@@ -568,14 +568,14 @@ __device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, do
     int kk = k0;
     for (int left = 4; kk < k1 && ok; --left) {
         const int done = m.segment(kk, phase, flying, ok);
-        __syncthreads();   // shared memory is free again
+        ok = block_ok(ok);   // (a barrier: shared memory is free again)
         left += (done - kk) / 16;
         const bool stop = done == kk || left <= 0;
         kk = done;
         if (stop) break;
     }
     if (TMA) {
-        if (tid == 0 && !ok)
+        if (tid == 0 && !ok)   // as star_fixed_march
             for (int s = 0; s < S::NSLOT; ++s)
                 if ((flying >> s) & 1u) mbar_wait_bounded(m.bar(s), (phase >> s) & 1u, tmo);
         __syncthreads();

@@ -416,7 +416,7 @@ __device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, c
     }
     for (int left = 4; kk < k1; --left) {
         const int done = m.segment(kk, phase, flying, ok);
-        __syncthreads();   // the ring and the notes are free again
+        ok = block_ok(ok);   // (a barrier: the ring and the notes are free again)
         left += (done - kk) / 16;
         if (done == kk || left <= 0 || !ok) {
             m.plain(done);
@@ -425,7 +425,8 @@ __device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, c
         kk = done;
     }
     if (TMA) {
-        // Copies may still be in flight after a wait that ran out: one more bounded wait each.
+        // Copies may still be in flight after a wait of thread 0 ran out (another thread's: it has seen them
+        // land): one more bounded wait each.
         if (tid == 0 && !ok)
             for (int s = 0; s < S::NSLOT; ++s)
                 if ((flying >> s) & 1u) mbar_wait_bounded(reinterpret_cast<uint64_t*>(bars + s), (phase >> s) & 1u, tmo);

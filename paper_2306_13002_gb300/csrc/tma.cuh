@@ -6,7 +6,8 @@
 // mbarrier's phase parity first. Every wait is bounded (about one second of clock64 cycles):
 // a wait that runs out is counted in a device counter whose address the launcher passes in
 // (read back by acs_wait_timeouts) and the thread carries on without further waits, so a lost
-// copy shows up as a wrong result and a counter, never as a hang.
+// copy shows up as a wrong result and a counter, never as a hang. No thread's own outcome may
+// decide which barriers it reaches (block_ok).
 #pragma once
 
 #include <cstdint>
@@ -65,6 +66,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
     }
     return true;
 }
+
+// Whether the waits of all threads of the block completed; a barrier. A wait can run out in some threads
+// only (a copy that lands between their limits), so what decides which barriers a thread reaches
+// next has to be the block's verdict, not the thread's own.
+__device__ __forceinline__ bool block_ok(bool ok) { return !__syncthreads_or(!ok); }
 
 // Box of a 3D tensor map at element coordinates (x, y, z) into shared memory at dst (128-byte
 // aligned), completing `bar`'s transaction count. x * 8 bytes must be a multiple of 16.
