@@ -40,14 +40,27 @@ __global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
     extern __shared__ __align__(128) double smem[];
     __shared__ long long s_unit;
     const BatchView b = batch_view(ws);
+    const bool leader = threadIdx.x == 0 && threadIdx.y == 0;
+    bool raw = false;
+    int left = 0;
+    BatchUnit u;
     for (;;) {
-        BatchUnit u;
-        if (!batch_next(b, counter, &s_unit, threadIdx.x == 0 && threadIdx.y == 0, u)) break;
+        if (!batch_next(b, counter, &s_unit, leader, u)) return;
         const BatchDesc& d = b.items[u.item];
         const Geom g = d.g;
-        rhs_fixed_march<BX, BY, false, ISO>(d.in0, d.out, g, kf, kc, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, nullptr,
-                                            nullptr);
+        left = rhs_fixed_march<BX, BY, false, ISO>(d.in0, d.out, g, kc, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, nullptr,
+                                                   nullptr, raw);
+        if (left < u.k1) break;
     }
+    // A block that met values that do not fit takes its further units in FP64 as well: what does not fit in
+    // one grid mostly does not in the others (the parameters decide), and the queue evens out the time.
+    u.k0 = left;
+    do {
+        const BatchDesc& d = b.items[u.item];
+        const Geom g = d.g;
+        rhs_rest<BX, BY, false, ISO>(d.in0, d.out, g, kf, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, nullptr, nullptr, raw);
+        raw = false;
+    } while (batch_next(b, counter, &s_unit, leader, u));
 }
 
 template <class K, class... A>

@@ -57,13 +57,9 @@ __device__ __forceinline__ void balanced_segments(const BalancedPlan& s, int b, 
     }
 }
 
-// The same segments one at a time (the march is then compiled once, not at each of the three calls).
-struct BalancedWalk {
-    int n;        // segments given so far
-    i64 L, L1;    // the share of the tops still to do
-};
-__device__ __forceinline__ bool balanced_next(const BalancedPlan& s, int b, BalancedWalk& w, i64& col, int& z0, int& z1) {
-    const int n = w.n++;
+// The n-th of the same segments, false past the last one (the march is then compiled once, not at each of
+// the three calls, and the count is all that lives across it).
+__device__ __forceinline__ bool balanced_segment(const BalancedPlan& s, int b, int n, i64& col, int& z0, int& z1) {
     if (n < s.f) {
         col = (i64)n * s.G + b;
         z0 = 0;
@@ -79,17 +75,22 @@ __device__ __forceinline__ bool balanced_next(const BalancedPlan& s, int b, Bala
         return n == s.f && s.P > 0;
     }
     const int H = s.Z - s.P, T = s.G - s.R, t = b - s.R;
-    if (n == s.f) {
-        w.L = (i64)s.R * H * t / T;
-        w.L1 = (i64)s.R * H * (t + 1) / T;
+    const i64 all = (i64)s.R * H;
+    i64 first, last;   // its share of the tops
+    if (all * T < (1ll << 31)) {   // (a 64-bit division takes a tenth of a plane step)
+        first = (int)all * t / T;
+        last = (int)all * (t + 1) / T;
+    } else {
+        first = all * t / T;
+        last = all * (t + 1) / T;
     }
-    if (w.L >= w.L1) return false;
-    const i64 c = w.L / H;
-    const int a = (int)(w.L - c * H);
+    if (first >= last) return false;
+    const i64 c = (all < (1ll << 31) ? (int)first / H : first / H) + (n - s.f), L = n == s.f ? first : c * H;
+    if (L >= last) return false;
+    const int a = (int)(L - c * H);
     col = c0 + c;
     z0 = s.P + a;
-    z1 = s.P + (int)min((i64)H, a + (w.L1 - w.L));
-    w.L += z1 - z0;
+    z1 = s.P + (int)min((i64)H, a + (last - L));
     return true;
 }
 

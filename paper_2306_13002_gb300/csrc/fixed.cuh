@@ -24,6 +24,19 @@ typedef unsigned int u32;
 // Exponents a segment may be scaled to: results and intermediate scales stay normal numbers.
 constexpr int kFixMinExp = 520, kFixMaxExp = 1600;
 
+// The thread's coordinates, read anew at every call: what is reckoned from them is then not carried in
+// registers across the loops over segments and units of work.
+__device__ __forceinline__ int tid_x() {
+    int t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
+}
+__device__ __forceinline__ int tid_y() {
+    int t;
+    asm volatile("mov.u32 %0, %%tid.y;" : "=r"(t));
+    return t;
+}
+
 // PTX shifts clamp amounts of 64 and more (the result is then 0).
 __device__ __forceinline__ u64 shr64(u64 v, int s) {
     u64 r;

@@ -107,15 +107,18 @@ __device__ __forceinline__ void load_plane(double* slot, const double* __restric
 // plane q with one tensor copy (`map`: the 4D tensor map of U, components outermost) that
 // completes on the slot's mbarrier, and the readers wait on it (bounded; timeouts counted in
 // *tmo). Plane q is fill number n = (q - k0 + 2) / 5 of its slot: phase parity n & 1.
-template <int BX, int BY, bool TMA, bool ISO = false>
+//
+// S with six slots (RhsFixShape): plane q in slot (q - k0 + 2) % 6, staged one step earlier. `staged`: the
+// first six planes (k0-2 .. k0+3, none past k1+1) are in the ring already, and no copy is in flight.
+template <int BX, int BY, bool TMA, bool ISO = false, class S = RhsShape<BX, BY>>
 __device__ __forceinline__ void rhs_march(const double* __restrict__ U, double* __restrict__ R, const Geom& g,
                                           const RhsConst& kc, int i0, int j0, int k0, int k1, double* smem,
-                                          const CUtensorMap* map, unsigned* tmo) {
-    using S = RhsShape<BX, BY>;
-    constexpr int PX = S::PX, PLANE = S::PLANE;
+                                          const CUtensorMap* map, unsigned* tmo, bool staged = false) {
+    constexpr int PX = S::PX, PLANE = S::PLANE, AHEAD = S::NSLOT - 2;   // step kk stages plane kk + AHEAD
+    static_assert(S::NSLOT == 5 || S::NSLOT == 6, "two planes ahead, or three");
     constexpr unsigned kSlotBytes = 5 * PLANE * sizeof(double);
     double* Us = smem;
-    double* Fxs = smem + S::U_ELEMS;
+    double* Fxs = smem + S::NSLOT * 5 * PLANE;
     double* Fys = Fxs + S::FX_ELEMS;
     double* Cs = Fys + S::FY_ELEMS;
     uint64_t* bars = reinterpret_cast<uint64_t*>(Cs + S::CONST_ELEMS);
@@ -135,9 +138,10 @@ __device__ __forceinline__ void rhs_march(const double* __restrict__ U, double* 
     const int i = i0 + tx, j = j0 + ty;
     const bool active = fluxer && tx < w && j < g.ny;
     const int own = fluxer ? (ty + 2) * PX + (tx + 2) : 2 * PX + 2;   // non-fluxers: any cell
-    auto sidx = [&](int q) -> int { return (q + S::NSLOT) % S::NSLOT; };
+    const int first = S::NSLOT == 5 ? -S::NSLOT : k0 - 2;   // a plane in slot 0
+    auto sidx = [&](int q) -> int { return (q - first) % S::NSLOT; };
     auto slot = [&](int q) -> double* { return Us + sidx(q) * (5 * PLANE); };
-    auto parity = [&](int q) -> unsigned { return (unsigned)((q - k0 + 2) / S::NSLOT) & 1u; };
+    auto parity = [&](int q) -> unsigned { return (unsigned)((q - k0 + 2) / S::NSLOT + staged) & 1u; };
     auto issue = [&](int q) {   // thread 0 only
         uint64_t* bar = bars + sidx(q);
         mbar_arrive_expect_tx(bar, kSlotBytes);
@@ -166,13 +170,18 @@ __device__ __forceinline__ void rhs_march(const double* __restrict__ U, double* 
             fence_mbar_init();
         }
         __syncthreads();
-        if (tid == 0 && ok)
-            for (int q = k0 - 2; q <= k0 + 2; ++q) issue(q);
-        for (int q = k0 - 2; q <= k0 + 2; ++q) wait_plane(q);
-    } else {
+        if (tid == 0 && ok && !staged)
+            for (int q = k0 - 2; q < k0 + AHEAD && q <= k1 + 1; ++q) issue(q);
+        if (!staged)
+            for (int q = k0 - 2; q <= k0 + 2; ++q) wait_plane(q);
+    } else if (!staged) {
         for (int q = k0 - 2; q <= k0 + 2; ++q) load_plane<BX, BY>(slot(q), U, g, i0, j0, q, tid);
         cp_async_commit();
         cp_async_wait_all();
+        if (S::NSLOT == 6) {   // in a group of its own, waited for in the next step
+            if (k0 + 3 <= k1 + 1) load_plane<BX, BY>(slot(k0 + 3), U, g, i0, j0, k0 + 3, tid);
+            cp_async_commit();
+        }
     }
     __syncthreads();
     const RhsRegs kr = stage_consts_read<RhsRegs>(Cs);
@@ -223,10 +232,13 @@ __device__ __forceinline__ void rhs_march(const double* __restrict__ U, double* 
             point_flux<ISO>(s[own], s[PLANE + own], s[2 * PLANE + own], s[3 * PLANE + own], s[4 * PLANE + own], k, pfx, pfy,
                        fzp);
         }
-        if (TMA)
-            wait_plane(kk + 2);   // plane kk+2 (issued one step earlier) has landed
-        else
+        if (TMA) {   // plane kk+2 has landed
+            if (!staged || kk + 2 > k0 + 3) wait_plane(kk + 2);
+        } else if (S::NSLOT == 5) {
             cp_async_wait_all();
+        } else {
+            cp_async_wait_group1();   // every group but the last step's, which brings plane kk+3
+        }
         __syncthreads();
 
         // (3) the right-hand side at plane kk.
@@ -277,21 +289,24 @@ __device__ __forceinline__ void rhs_march(const double* __restrict__ U, double* 
             fz0[c] = fzp[c];
         }
         __syncthreads();  // slot kk-2 and the flux planes are free again
-        // (5) bulk-load plane kk+3 into the slot of kk-2.
+        // (5) bulk-load plane kk+3 (six slots: kk+4) into the slot of kk-2.
         if (TMA) {
-            if (kk + 3 <= k1 + 1 && tid == 0 && ok) {
+            if (kk + AHEAD <= k1 + 1 && tid == 0 && ok) {
                 fence_proxy_async();
-                issue(kk + 3);
+                issue(kk + AHEAD);
             }
         } else {
-            if (kk + 3 <= k1 + 1) load_plane<BX, BY>(slot(kk + 3), U, g, i0, j0, kk + 3, tid);
+            if (kk + AHEAD <= k1 + 1) load_plane<BX, BY>(slot(kk + AHEAD), U, g, i0, j0, kk + AHEAD, tid);
             cp_async_commit();
         }
     }
     if (TMA) {
-        // A copy whose wait ran out may still be in flight: give it one more bounded wait
-        // before the slots are reused or the block exits. Then retire the barriers.
-        if (tid == 0 && !ok && lost != 0x7fffffff) mbar_wait_bounded(bars + sidx(lost), parity(lost), tmo);
+        // A copy whose wait ran out, and those issued after it, may still be in flight: give each one more
+        // bounded wait before the slots are reused or the block exits. Then retire the barriers.
+        if (tid == 0 && !ok && lost != 0x7fffffff) {
+            const int last = lost <= k0 + 2 ? k0 + AHEAD - 1 : lost + AHEAD - 3;
+            for (int q = lost; q <= last && q <= k1 + 1; ++q) mbar_wait_bounded(bars + sidx(q), parity(q), tmo);
+        }
         __syncthreads();
         if (tid == 0)
             for (int s = 0; s < S::NSLOT; ++s) mbar_inval(bars + s);

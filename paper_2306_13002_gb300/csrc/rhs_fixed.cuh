@@ -28,6 +28,9 @@
 
 namespace acs {
 
+// 2^n; 0 below the normal floats, infinity above.
+__device__ __forceinline__ float pow2f(int n) { return __int_as_float(min(max(n + 127, 0), 255) << 23); }
+
 // t * 2^e2 rounded to FP64 (half away from zero) with its sign flipped, on the integer pipes. No
 // branches here or in the flux: the five components' chains interleave.
 __device__ __forceinline__ double minus_from_fixed(i64 t, int e2) {
@@ -81,15 +84,14 @@ struct RhsFixShape {
     static constexpr int NT = BX * BY, NSLOT = 6;
     static constexpr int NR = 2 * (BX + BY), NC = NT - NR;   // threads of the flux ring, and of the cells
     static constexpr int NE = (CELLS + NC - 1) / NC;
-    static constexpr int FX = 4 * BY * (BX + 2), FY = 4 * (BY + 2) * BX;
-    static constexpr int CONST_ELEMS = 16;
+    static constexpr int FX_ELEMS = 4 * BY * (BX + 2), FY_ELEMS = 4 * (BY + 2) * BX;
+    static constexpr int CONST_ELEMS = RhsShape<BX, BY>::CONST_ELEMS;
     // ... constants of the launch, mbarriers, the scan's results, constants of the segment
-    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * CELLS + FX + FY + CONST_ELEMS + NSLOT + 4 + 10 + 3);
+    static constexpr size_t BYTES = sizeof(u64) * ((size_t)NSLOT * CELLS + FX_ELEMS + FY_ELEMS + CONST_ELEMS + NSLOT + 4 + 10 + 3);
     static constexpr int MINB = NT <= 128 ? 4 : 2;
     static_assert((CELLS * sizeof(u64)) % 128 == 0, "every ring slot 128-byte aligned");
     static_assert(NT >= 2 * (BX + BY) && (2 * BX) % 32 == 0, "flux ring needs 2(BX+BY) threads, y-ring whole warps");
     static_assert(sizeof(RhsConst) <= CONST_ELEMS * sizeof(double), "constant staging area");
-    static_assert(BYTES >= RhsShape<BX, BY>::BYTES, "the FP64 march runs in the same shared memory");
 };
 
 // A segment's constants, in shared memory: the march has few registers to spare.
@@ -111,6 +113,22 @@ __device__ __forceinline__ RhsJoin rhs_join(int ea, int ed) {
     return RhsJoin{min(e - ea, 63), min(e - ed, 63), e};
 }
 
+// Whether the dissipation of a point's momenta has room for certain, from the upper halves of its values in
+// three planes (addresses of rho's): 4.5 of the point's own and a quarter of the six at distance 2 are
+// at most 12 2^59, so it takes six nearest values of the other sign that sum to 4 2^59 to exceed 2^63. A
+// call of its own: inlined in the march, it took 30 us of 256^3 without being run.
+template <int PX, int PLANE>
+__device__ __noinline__ bool rhs_roomy(u32 below, u32 here, u32 above) {
+    bool all = true;
+#pragma unroll
+    for (int c = 1; c < 4; ++c) {
+        auto hi = [&](u32 a) { return lds_int(a + c * PLANE * 8 + 4); };
+        const int h1 = (hi(here - 8) + hi(here + 8) + hi(here - 8 * PX)) + (hi(here + 8 * PX) + hi(below) + hi(above));
+        all &= (hi(here) ^ h1) >= 0 || abs(h1) < (4 << 27) - 8;   // (8: their lower halves)
+    }
+    return all;
+}
+
 template <int BX, int BY, bool TMA, bool ISO>
 struct RhsFixMarch {
     using S = RhsFixShape<BX, BY>;
@@ -127,17 +145,18 @@ struct RhsFixMarch {
     unsigned* tmo;
 
     __device__ __forceinline__ uint64_t* bar(int slot) const {
-        return reinterpret_cast<uint64_t*>(smem + NSLOT * S::CELLS + S::FX + S::FY + S::CONST_ELEMS) + slot;
+        return reinterpret_cast<uint64_t*>(smem + NSLOT * S::CELLS + S::FX_ELEMS + S::FY_ELEMS + S::CONST_ELEMS) + slot;
     }
 
     __device__ __forceinline__ RhsScale* scales() const { return reinterpret_cast<RhsScale*>(bar(NSLOT) + 4); }
 
-    // Marches from plane k0; returns the first plane not finished. `phase`, `flying`, `ok`: as
+    // Marches from plane k0; returns the first plane not finished, or k0 - 1 if the scanned planes do not
+    // fit: the ring then holds planes k0-2 .. k0+3 (none past k1+1) as they are. `phase`, `flying`, `ok`: as
     // StarFixMarch::segment.
     __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
-        const int tid = threadIdx.y * BX + threadIdx.x;
-        const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX * 8;
-        // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E, [5] 1: a point's dissipation may not fit
+        const int tid = tid_y() * BX + tid_x();
+        const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX_ELEMS * 8;
+        // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E
         int* note = reinterpret_cast<int*>(bar(NSLOT));
         // Tiles cut by the grid's edges: points packed as in rhs_march, one halo column more than the
         // valid ones; rows up to the one past the last valid row.
@@ -151,17 +170,23 @@ struct RhsFixMarch {
 
         // The first NR threads compute the ring's fluxes; the others stage and convert the cells.
         const int cell = tid - S::NR;
-        u32 full = 0, core = 0;
-#pragma unroll
-        for (int n = 0; n < NE; ++n) {
-            const int e = cell + n * NC, r = e % PLANE;
-            const int yy = r / PX, xx = r - yy * PX;
-            const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2, mine = cell >= 0 && e < S::CELLS;
-            if (mine && xx < w + 4 && yy < h + 4 && (xin || yin)) full |= 1u << n;
-            if (mine && xin && yin) core |= 1u << n;
-        }
+        u32 full = 0, core = 0;   // one bit per cell: read by some point on the segment's planes, and on others
         const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 2 > g.nx || j0 + BY + 2 > g.ny);
-        if (TMA && !rim) full = ~0u;
+        auto masks = [&]() {
+            int xx = cell % PX, yy = cell / PX;
+#pragma unroll 1
+            for (int n = 0, e = cell; e >= 0 && e < S::CELLS; ++n, e += NC) {
+                const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2;
+                if (xx < w + 4 && yy < h + 4 && (xin || yin)) full |= 1u << n;
+                if (xin && yin) core |= 1u << n;
+                xx += NC % PX;
+                yy += NC / PX;
+                if (xx >= PX) xx -= PX, ++yy;
+                if (yy >= S::PY) yy -= S::PY;
+            }
+            if (TMA && !rim) full = ~0u;
+        };
+        if (!TMA) masks();
         auto keep = [&](int q) { return q >= k0 && q < k1 ? full : core; };
         auto slot_of = [&](int q) { return (q - k0 + 2) % NSLOT; };
         auto stage = [&](int q) {
@@ -216,35 +241,50 @@ struct RhsFixMarch {
         // Prologue: the first six planes under way; exponent ranges of the first five.
         int next = k0 - 2;
         for (; next < k0 + 4 && next < k1 + 2; ++next) stage(next);
-        if (tid < 6) note[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
+        if (tid < 5) note[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
         __syncthreads();
-        int rng[5] = {0, 0x7ff, 0, 0, 0x7ff};
-        if (!TMA) cp_async_wait_all();
+        u32 rng[5] = {0, ~0u, 0, 0, ~0u};   // of the exponents, shifted up
+        if (!TMA) {
+            cp_async_wait_all();
+            __syncthreads();
+        }
         const int scanned = min(5, next - k0 + 2);
-#pragma unroll 1
-        for (int p = 0; p < scanned; ++p) {
-            landed(p);
-            const u32 m = keep(k0 - 2 + p);
+        {
+            static_assert(PLANE <= 2 * S::NT, "two cells of a component and plane per thread");
+            bool in[2], mid[2];
 #pragma unroll
-            for (int n = 0; n < NE; ++n) {
-                if (cell < 0 || !((m >> n) & 1u) || cell + n * NC >= S::CELLS) continue;
-                const u64 v = lds1(rs + (p * S::CELLS + cell + n * NC) * 8);
-                const int e = (int)((hi32(v) << 1) >> 21), kd = kind_of(n);
-                if (kd == 0) {
-                    rng[0] = max(rng[0], e);
-                    rng[1] = min(rng[1], e);
-                } else if (kd == 1) {
-                    rng[2] = max(rng[2], e);
-                } else {
-                    rng[3] = max(rng[3], e);
-                    rng[4] = min(rng[4], e);
+            for (int i = 0; i < 2; ++i) {
+                const int r = tid + i * S::NT, yy = r / PX, xx = r - yy * PX;
+                const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2, is = r < PLANE;
+                in[i] = is && ((TMA && !rim) || (xx < w + 4 && yy < h + 4 && (xin || yin)));
+                mid[i] = is && xin && yin;
+            }
+            u32 at = rs + tid * 8 + 4;
+#pragma unroll 1
+            for (int p = 0; p < scanned; ++p) {
+                landed(p);
+                const bool inner = k0 - 2 + p >= k0 && k0 - 2 + p < k1;
+                const bool a0 = inner ? in[0] : mid[0], a1 = inner ? in[1] : mid[1];
+#pragma unroll
+                for (int c = 0; c < 5; ++c, at += PLANE * 8) {
+                    const u32 e0 = a0 ? (u32)lds_int(at) << 1 : 0u, e1 = a1 ? (u32)lds_int(at + S::NT * 8) << 1 : 0u;
+                    const u32 top = max(e0, e1), low = min(a0 ? e0 : ~0u, a1 ? e1 : ~0u);
+                    if (c == 0) {
+                        rng[0] = max(rng[0], top);
+                        rng[1] = min(rng[1], low);
+                    } else if (c < 4) {
+                        rng[2] = max(rng[2], top);
+                    } else {
+                        rng[3] = max(rng[3], top);
+                        rng[4] = min(rng[4], low);
+                    }
                 }
             }
         }
 #pragma unroll
         for (int n = 0; n < 5; ++n) {
             const bool mn = n == 1 || n == 4;
-            const int v = mn ? __reduce_min_sync(0xffffffffu, rng[n]) : __reduce_max_sync(0xffffffffu, rng[n]);
+            const int v = (int)((mn ? __reduce_min_sync(0xffffffffu, rng[n]) : __reduce_max_sync(0xffffffffu, rng[n])) >> 21);
             if ((tid & 31) == 0) {
                 if (mn)
                     atomicMin(note + n, v);
@@ -263,12 +303,16 @@ struct RhsFixMarch {
         // Exponents: |rho| in [2^rlo, 2^rhi), |m| < 2^mhi, |E| in [2^elo, 2^ehi), of all planes so far or,
         // where these range too far, of the scanned ones.
         int rhi = 0, rlo = 0, mhi = 0, ehi = 0, elo = 0, efm = 0, efe = 0;
-        bool fits = false;
+        bool fits = false, more = true;
 #pragma unroll 1
-        for (int t = 0; t < 2 && !fits; ++t) {
+        for (int t = 0; t < 2 && !fits && more; ++t) {
+            more = false;   // whether the planes before widen the ranges
 #pragma unroll
-            for (int n = 0; n < 5; ++n)
-                seen[n] = t ? note[n] : n == 1 || n == 4 ? min(seen[n], note[n]) : max(seen[n], note[n]);
+            for (int n = 0; n < 5; ++n) {
+                const int now = note[n];
+                seen[n] = t ? now : n == 1 || n == 4 ? min(seen[n], now) : max(seen[n], now);
+                more |= seen[n] != now;
+            }
             rhi = seen[0] - 1022;
             rlo = seen[1] - 1023 - 1;
             mhi = max(seen[2], 1023 + rlo - 60) - 1022;
@@ -279,20 +323,21 @@ struct RhsFixMarch {
             if (!fits) continue;
             // Bounds of the fluxes, and whether quantising against them stays below what FP64 rounds
             // anyway at the least rho and E: the dissipation (eps 18 U 2^-53) for the mass and energy
-            // components, the pressure ((gamma - 1) E 2^-53) for the momenta.
-            const float vmax = ldexpf(1.f, mhi - rlo), mv = ldexpf(vmax, mhi);
-            const float P = fabsf(fx.g1) * (ldexpf(1.f, ehi) + 1.5f * mv);
-            const float bm = (mv + P) * fx.smax * 1.01f, be = (ldexpf(1.f, ehi) + P) * vmax * fx.smax * 1.01f;
-            const float pl = fx.smin * fabsf(fx.g1) * ldexpf(1.f, elo);
-            fits = isfinite(bm) && isfinite(be) && fx.eps * ldexpf(1.f, rlo) >= fx.smax * ldexpf(0x1p-10f, mhi) &&
-                   fx.eps * ldexpf(1.f, elo) >= be * 0x1p-10f && pl >= bm * 0x1p-8f && pl * 0x1p5f >= fx.eps * ldexpf(1.f, mhi);
-            efm = ilogbf(bm) + 1;
-            efe = ilogbf(be) + 1;
+            // components, the pressure ((gamma - 1) E 2^-53) for the momenta. All relative to 2^ehi, so that
+            // the floats hold them whatever the unit of U is.
+            const float g1 = fabsf(fx.g1), vmax = pow2f(mhi - rlo), mv = pow2f(2 * mhi - rlo - ehi), el = pow2f(elo - ehi);
+            const float P = g1 * (1.f + 1.5f * mv);
+            const float bm = (mv + P) * fx.smax * 1.01f, be = (1.f + P) * vmax * fx.smax * 1.01f, pl = fx.smin * g1 * el;
+            fits = bm > 0x1p-100f && bm < 0x1p100f && be > 0x1p-100f && be < 0x1p100f && fx.eps >= fx.smax * vmax * 0x1p-10f &&
+                   fx.eps * el >= be * 0x1p-10f && pl >= bm * 0x1p-8f && pl * 0x1p5f >= fx.eps * pow2f(mhi - ehi);
+            efm = (__float_as_int(bm) >> 23) - 126 + ehi;
+            efe = (__float_as_int(be) >> 23) - 126 + ehi;
         }
         if (!fits) {
             for (int p = scanned; p < next - k0 + 2; ++p) landed(p);
-            return k0;
+            return k0 - 1;
         }
+        if (TMA) masks();
         // Conversion exponents (leading bit at 59) and the units of the sums. U has one more bit of room, so
         // that a flow may double on the way: the dissipation, 6/4 + 6 + 4.5 times the largest value, is
         // below 12 2^59 for values as scanned and for values of one sign (a negative rho or E ends the
@@ -320,7 +365,7 @@ struct RhsFixMarch {
 
         auto raw = [&](u32 at) { return __longlong_as_double((long long)lds1(at)); };
         auto flux = [&](u32 at, double* fxv, double* fyv, double* fzv) {
-            const RhsConst k = stage_consts_read<RhsConst>(smem + NSLOT * S::CELLS + S::FX + S::FY);
+            const RhsConst k = stage_consts_read<RhsConst>(smem + NSLOT * S::CELLS + S::FX_ELEMS + S::FY_ELEMS);
             const double rho = raw(at), mx = raw(at + PLANE * 8), my = raw(at + 2 * PLANE * 8), mz = raw(at + 3 * PLANE * 8),
                          E = raw(at + 4 * PLANE * 8);
             if (ISO)
@@ -429,21 +474,6 @@ struct RhsFixMarch {
 #pragma unroll
             for (int c = 0; c < 5; ++c) Rp[(i64)c * g.osc] = minus_from_fixed(z[c], ze[c]);
         };
-        // Whether the dissipation of this thread's momenta in plane q-2 has room for certain, from the upper
-        // halves of its values: 4.5 of the point's own and a quarter of the six at distance 2 are at most
-        // 12 2^59, so it takes six nearest values of the other sign that sum to 4 2^59 to exceed 2^63.
-        auto roomy = [&]() {
-            const u32 s0 = back(2) + own + 4, sm1 = back(3) + own + 4, sp1 = back(1) + own + 4;
-            bool all = true;
-#pragma unroll
-            for (int c = 1; c < 4; ++c) {
-                constexpr int C = PLANE * 8;
-                auto hi = [&](u32 a) { return lds_int(a + c * C); };
-                const int h1 = (hi(s0 - 8) + hi(s0 + 8) + hi(s0 - 8 * PX)) + (hi(s0 + 8 * PX) + hi(sm1) + hi(sp1));
-                all &= (hi(s0) ^ h1) >= 0 || abs(h1) < (4 << 27) - 8;   // (8: their lower halves)
-            }
-            return all;
-        };
         bool wide = false;   // a momentum is larger than those scanned
         const bool whole = w == BX && h == BY;
 #pragma unroll 1
@@ -497,24 +527,27 @@ struct RhsFixMarch {
                             bad |= ((int)((hi32(v[n]) << 1) >> 21) - lds_int(sc + 60 + 4 * kd)) | (kd == 1 ? 0 : (int)hi32(v[n]));
                         int s;
                         sts1(sq + (cell + n * NC) * 8, to_fixed_by(v[n], cu, 0, s));
-                        bad |= s;
-                        if ((n + 1) * NC > PLANE && n * NC < 4 * PLANE) room = min(room, kd == 1 ? s : 1);
+                        if (n * NC >= PLANE && (n + 1) * NC <= 4 * PLANE) {
+                            room = min(room, s);
+                        } else {
+                            bad |= s;
+                            if ((n + 1) * NC > PLANE && n * NC < 4 * PLANE && kd == 1) room = min(room, s);
+                        }
                     }
                 }
+                bad |= room;
                 grew = room == 0 && !wide;
                 if (TMA) fence_proxy_async();
             }
+            if (wide && active && q - 2 >= k0 && !rhs_roomy<PX, PLANE>(back(3) + own, back(2) + own, back(1) + own)) bad = -1;
             if (!ok) bad = -1;
-            // Plane q in fixed point, its fluxes; a value out of range ends the segment before it is used.
+            // Plane q in fixed point, its fluxes; a value out of range ends the segment before it is used, and so
+            // does a point of plane q-2 whose dissipation may not fit.
             if (__syncthreads_or(bad < 0 || grew)) {
                 if (__syncthreads_or(bad < 0)) break;
                 wide = true;
             }
             bad = 0;
-            if (wide && active && q - 2 >= k0 && !roomy()) {   // the next vote ends the segment, before this plane
-                note[5] = 1;
-                bad = -1;
-            }
             // Then plane q-2's result from integers and plane q+1's fluxes in FP64: independent, and in one
             // stretch of code where the whole tile takes part, so that the two pipes work at once.
             if (whole && q - 2 >= k0 && q + 1 < k1) {
@@ -537,26 +570,28 @@ struct RhsFixMarch {
             }
             cur = nslot;
         }
-        __syncthreads();
-        const int again = note[5];
         // Copies not waited for yet: planes after q + 1 that a segment cut short had under way.
         for (int p = max(q + 2, k0 + 3), s = slot_of(p); p < next; ++p, s = s + 1 == NSLOT ? 0 : s + 1) landed(s);
         if (!TMA) cp_async_wait_all();
-        return min(max(q - 2 - again, k0), k1);
+        return min(max(q - 2, k0), k1);
     }
 };
 
 // One block's work: the BX x BY column tile at (i0, j0), z-planes [k0, k1). Ends with all threads past
-// a barrier after their last shared-memory access. The planes of segments that do not fit run in the
-// FP64 march.
+// a barrier after their last shared-memory access. Returns the first plane that is left for the FP64
+// march (k1 if none); `raw`: the ring holds planes from two below that one on, as rhs_rest takes them.
+//
+// The FP64 march follows where nothing of this one lives any more, after a block's last unit. Called from
+// here it got what registers the loops over segments and units left it, and spilled: 256^3 with
+// values that never fit ran 3730 us in the balanced kernel, against 3255 for the FP64 kernel.
 template <int BX, int BY, bool TMA, bool ISO>
-__device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, double* __restrict__ R, const Geom& g,
-                                                const RhsConst& kf, const RhsConst& kc, const RhsFix& fx, int i0, int j0,
-                                                int k0, int k1, double* smem, const CUtensorMap* map, unsigned* tmo) {
+__device__ __forceinline__ int rhs_fixed_march(const double* __restrict__ U, double* __restrict__ R, const Geom& g,
+                                               const RhsConst& kc, const RhsFix& fx, int i0, int j0, int k0, int k1,
+                                               double* smem, const CUtensorMap* map, unsigned* tmo, bool& raw) {
     using S = RhsFixShape<BX, BY>;
     const int tid = threadIdx.y * BX + threadIdx.x;
     const RhsFixMarch<BX, BY, TMA, ISO> m{U, R, g, kc, fx, i0, j0, k1, smem, map, tmo};
-    stage_consts_write(smem + S::NSLOT * S::CELLS + S::FX + S::FY, kc, tid);
+    stage_consts_write(smem + S::NSLOT * S::CELLS + S::FX_ELEMS + S::FY_ELEMS, kc, tid);
     if (tid < 5) m.scales()->seen[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
     if (TMA && tid == 0) {
         for (int s = 0; s < S::NSLOT; ++s) mbar_init(m.bar(s), 1);
@@ -566,9 +601,12 @@ __device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, do
     u32 phase = 0, flying = 0;
     bool ok = !TMA || (smem_addr(smem) & 127u) == 0;
     int kk = k0;
+    raw = false;
     for (int left = 4; kk < k1 && ok; --left) {
         const int done = m.segment(kk, phase, flying, ok);
         ok = block_ok(ok);   // (a barrier: shared memory is free again)
+        raw = done < kk;
+        if (raw) break;
         left += (done - kk) / 16;
         const bool stop = done == kk || left <= 0;
         kk = done;
@@ -583,10 +621,23 @@ __device__ __forceinline__ void rhs_fixed_march(const double* __restrict__ U, do
             for (int s = 0; s < S::NSLOT; ++s) mbar_inval(m.bar(s));
         __syncthreads();
     }
-    if (kk < k1) {
-        rhs_march<BX, BY, TMA, ISO>(U, R, g, kf, i0, j0, kk, k1, smem, map, tmo);
-        __syncthreads();
-    }
+    raw = raw && ok;
+    return kk;
 }
+
+// The planes [k0, k1) of a column in the FP64 march.
+template <int BX, int BY, bool TMA, bool ISO>
+__device__ __forceinline__ void rhs_rest(const double* __restrict__ U, double* __restrict__ R, const Geom& g, const RhsConst& kf,
+                                         int i0, int j0, int k0, int k1, double* smem, const CUtensorMap* map, unsigned* tmo,
+                                         bool raw) {
+    rhs_march<BX, BY, TMA, ISO, RhsFixShape<BX, BY>>(U, R, g, kf, i0, j0, k0, k1, smem, map, tmo, raw);
+    __syncthreads();
+}
+
+// Planes a block leaves for the FP64 march.
+constexpr int kRhsLeft = 16;
+struct RhsLeft {
+    int i0, j0, from, to;
+};
 
 }  // namespace acs

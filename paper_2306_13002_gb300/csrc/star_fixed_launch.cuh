@@ -47,10 +47,9 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
                                const __grid_constant__ StarFix fx, const __grid_constant__ BalancedPlan plan,
                                const __grid_constant__ CUtensorMap map, unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
-    BalancedWalk walk{0, 0, 0};
     i64 col;
     int z0, z1;
-    while (balanced_next(plan, blockIdx.x, walk, col, z0, z1))
+    for (int n = 0; balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n)
         star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, (int)(col % plan.ntx) * BX,
                                           (int)(col / plan.ntx) * BY, z0, z1, smem, &map, tmo);
 }

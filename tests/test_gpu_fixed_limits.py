@@ -6,8 +6,10 @@ otherwise.
 import numpy as np
 import pytest
 
-from paper_2306_13002_gb300 import inputs
-from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _star
+import oracle
+from paper_2306_13002_gb300 import binding, inputs
+from _parity import to_dev
+from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _rhs_scale, _star
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +40,47 @@ def test_star_negative_zeros(tile):
     a = np.random.default_rng(34).uniform(0.5, 1.5, u.shape)
     assert not np.any(_star(u, a, TAYLOR, tile))
     assert not np.any(_star(np.full(u.shape, -0.0), a, TAYLOR, tile))
+
+
+@pytest.mark.parametrize("h", [(1.0, 1.0, 1.0), (1.0, 0.5, 2.0)])
+@pytest.mark.parametrize("flags", [0, 2])
+@pytest.mark.parametrize("kchunk", [1, 2, 3, 4, 5, 6, 7, 9, 14])
+def test_rhs_fp64_rest_from_the_scanned_planes(kchunk, flags, h):
+    """Values the scan refuses (a weak dissipation), in chunks as short as the planes it leaves in the ring and
+    longer, on whole and cut tiles."""
+    U = inputs.rhs_field(75, 50, 43, halo=2, seed=35)
+    _check_rhs(U, (16, 16, kchunk, flags), (kchunk, flags, h), eps=0.004, h=h)
+
+
+@pytest.mark.parametrize("flags", [1, 3])
+@pytest.mark.parametrize("every", [1, 7, 40])
+def test_rhs_fp64_rest_of_many_columns(every, flags):
+    """A balanced launch on a thin grid: 17 columns and more per block, all of them, most or a few with values
+    that do not fit."""
+    nx, ny, nz = 1150, 1144, 2
+    U = inputs.rhs_field(nx, ny, nz, halo=2, seed=36)
+    y, x = np.meshgrid(np.arange(ny + 4), np.arange(nx + 4), indexing="ij")
+    odd = ((x // 16) + 72 * (y // 16)) % every == 0
+    U[:, :, odd & (x % 16 == 3) & (y % 16 == 5)] *= 2.0 ** 11
+    _check_rhs(U, (16, 16, 0, flags), (every, flags))
+
+
+@pytest.mark.parametrize("eps,spiked", [(0.25, 0), (0.25, 3), (0.25, 8), (0.004, 0)])
+def test_rhs_batch_fp64_rest(eps, spiked):
+    """A batch with work for the fixed-point march, some or all of whose grids hold values that do not fit."""
+    host, grids = [], []
+    for q, (nx, ny, nz) in enumerate([(64, 48, 50), (49, 47, 61), (33, 70, 40), (80, 31, 45), (48, 48, 48), (65, 50, 37),
+                                      (40, 40, 60), (51, 62, 30), (17, 90, 50), (60, 60, 60)]):
+        U = inputs.rhs_field(nx, ny, nz, halo=2, seed=3700 + q)
+        if q < spiked:
+            U[:, 20:24, 10:15, 9:18] *= 2.0 ** 12
+        host.append(U)
+        grids.append((to_dev(U), None, torch.full((5, nz, ny, nx), float("nan"), dtype=torch.float64, device="cuda")))
+    ws = torch.zeros(binding.acs_batch_workspace_bytes(len(grids)) // 8 + 2, dtype=torch.float64, device="cuda")
+    plan = binding.acs_batch_prepare(binding.KIND_RHS, grids, ws)
+    for _ in range(2):
+        binding.acs_batch_launch(plan, {"eps": eps})
+    torch.cuda.synchronize()
+    for U, (_, _, R) in zip(host, grids):
+        bad = ~(np.abs(R.cpu().numpy() - oracle.rhs(U, eps=eps, threads=8)) <= 2.0 ** -46 * _rhs_scale(U, 1.4, eps, (1.0,) * 3))
+        assert not bad.any(), (U.shape, np.argwhere(bad)[:3])
