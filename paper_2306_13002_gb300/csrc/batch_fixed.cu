@@ -21,13 +21,17 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
         if (!batch_next(b, counter, &s_unit, threadIdx.x == 0, u)) break;
         const BatchDesc& d = b.items[u.item];
         const Geom g = d.g;
+        const int i0 = u.tx * BX, j0 = u.ty * BY;
+        bool raw;
         if (d.tma) {
             const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(ws + b.head->maps_off) + u.item;
             if (threadIdx.x == 0) tensormap_acquire(map);
-            star_fixed_march<BX, BY, true, ISO>(d.in0, d.in1, d.out, g, cf, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, map, tmo);
+            const int left = star_fixed_march<BX, BY, true, ISO>(d.in0, d.in1, d.out, g, cf, fx, i0, j0, u.k0, u.k1, smem, map, tmo, tid_x(), raw);
+            if (left < u.k1) star_rest<BX, BY, true>(d.in0, d.in1, d.out, g, cf, i0, j0, left, u.k1, map, tmo, raw);
         } else {
-            star_fixed_march<BX, BY, false, ISO>(d.in0, d.in1, d.out, g, cf, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem,
-                                                 nullptr, nullptr);
+            const int left = star_fixed_march<BX, BY, false, ISO>(d.in0, d.in1, d.out, g, cf, fx, i0, j0, u.k0, u.k1, smem,
+                                                                  nullptr, nullptr, tid_x(), raw);
+            if (left < u.k1) star_rest<BX, BY, false>(d.in0, d.in1, d.out, g, cf, i0, j0, left, u.k1, nullptr, nullptr, raw);
         }
     }
 }

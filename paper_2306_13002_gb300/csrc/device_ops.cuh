@@ -203,6 +203,8 @@ __device__ __forceinline__ void cp_async8_or_zero(unsigned smem_dst, const void*
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+// Waits until at most the two most recently committed groups are still in flight.
+__device__ __forceinline__ void cp_async_wait_group2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
 // Waits until at most the most recently committed group is still in flight.
 __device__ __forceinline__ void cp_async_wait_group1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 

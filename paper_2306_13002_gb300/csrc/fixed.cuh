@@ -37,6 +37,12 @@ __device__ __forceinline__ int tid_y() {
     return t;
 }
 
+// Planes a block leaves for the FP64 march.
+constexpr int kBlockLeft = 16;
+struct BlockLeft {
+    int i0, j0, from, to;
+};
+
 // PTX shifts clamp amounts of 64 and more (the result is then 0).
 __device__ __forceinline__ u64 shr64(u64 v, int s) {
     u64 r;

@@ -634,10 +634,4 @@ __device__ __forceinline__ void rhs_rest(const double* __restrict__ U, double* _
     __syncthreads();
 }
 
-// Planes a block leaves for the FP64 march.
-constexpr int kRhsLeft = 16;
-struct RhsLeft {
-    int i0, j0, from, to;
-};
-
 }  // namespace acs

@@ -30,28 +30,28 @@ __global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
                               const __grid_constant__ RhsFix fx, const __grid_constant__ BalancedPlan plan,
                               const __grid_constant__ CUtensorMap map, unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
-    __shared__ RhsLeft list[kRhsLeft];
+    __shared__ BlockLeft list[kBlockLeft];
     i64 col;
     int z0, z1, n = 0, count = 0;
     bool raw = false;
-    for (; count < kRhsLeft && balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n) {
+    for (; count < kBlockLeft && balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n) {
         const int i0 = (int)col % plan.ntx * BX, j0 = (int)col / plan.ntx * BY;
         const int left = rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kc, fx, i0, j0, z0, z1, smem, &map, tmo, raw);
         if (left < z1) {
-            if (threadIdx.x == 0 && threadIdx.y == 0) list[count] = RhsLeft{i0, j0, left, z1};
+            if (threadIdx.x == 0 && threadIdx.y == 0) list[count] = BlockLeft{i0, j0, left, z1};
             ++count;
         }
     }
     __syncthreads();
     // The listed planes, the last ones first (their ring may still hold them); a block with a full list
     // runs its other segments in FP64, too.
-    for (int i = count - 1; i >= 0 || count == kRhsLeft; --i, raw = false) {
-        RhsLeft l;
+    for (int i = count - 1; i >= 0 || count == kBlockLeft; --i, raw = false) {
+        BlockLeft l;
         if (i >= 0) {
             l = list[i];
         } else {
             if (!balanced_segment(plan, blockIdx.x, n++, col, z0, z1)) break;
-            l = RhsLeft{(int)col % plan.ntx * BX, (int)col / plan.ntx * BY, z0, z1};
+            l = BlockLeft{(int)col % plan.ntx * BX, (int)col / plan.ntx * BY, z0, z1};
         }
         rhs_rest<BX, BY, TMA, ISO>(U, R, g, kf, l.i0, l.j0, l.from, l.to, smem, &map, tmo, raw);
     }

@@ -26,6 +26,7 @@ namespace acs {
 // three) send the point to the FP64 form.
 constexpr u32 kStarBiasHi = 1u << 28;            // 2^60: the offset that keeps inputs unsigned
 constexpr u32 kStarSmallHi = 1u << 18;           // 2^50: the small-value bound
+constexpr int kStarSmallBits = 9;                // below E0 by more: small (2^50 is 2^-9 of 2^59)
 constexpr int kStarIsoLB = 29, kStarGenLB = 28;  // bits of Wl (see StarFix)
 
 // The sum at one point in FP64, from global memory: the saturated form's operations in their order.
@@ -78,16 +79,24 @@ struct StarFixMarch {
 
     __device__ __forceinline__ bool valid(int c) const { return ty < h && tx + c < w; }
 
-    // FP64 for the planes [k0, k1).
-    __device__ __forceinline__ void plain(int k0) const {
-        for (int kk = k0; kk < k1; ++kk)
-#pragma unroll 1
-            for (int c = 0; c < 2; ++c) {
-                if (!valid(c)) continue;
-                const i64 at = (i64)(kk + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + c + g.halo);
-                out[(i64)kk * g.osz + (i64)(j0 + ty) * g.osy + i0 + tx + c] =
-                    __ldg(a + at) * star_point(u + at, g.isy, g.isz, cf);
-            }
+    // The cells of a plane that some point reads, one bit each: a caller may leave the others (corners of the
+    // halo) unset. On planes past the segment's end only the columns themselves are read (core).
+    __device__ __forceinline__ void cells_read(u32& full, u32& core, u32 (&off)[NE]) const {
+        full = core = 0;
+#pragma unroll
+        for (int n = 0; n < NE; ++n) {
+            const int e = tid + n * NT;
+            const int yy = e / PX, xx = e - yy * PX;
+            const bool xin = xx >= 4 && xx < w + 4, yin = yy >= 4 && yy < h + 4;
+            const bool in = xx < w + 8 && yy < h + 8 && e < PLANE && (xin || yin);
+            off[n] = in ? (u32)(yy * (int)g.isy + xx) : 0u;
+            if (in) full |= 1u << n;
+            if (xin && yin) core |= 1u << n;
+        }
+    }
+    // Tensor copies bring every cell: only tiles at the grid's rim drop the ones not read.
+    __device__ __forceinline__ bool at_rim() const {
+        return TMA && (i0 == 0 || j0 == 0 || i0 + BX + 4 > g.nx || j0 + BY + 4 > g.ny);
     }
 
     // Stages plane q (raw values) into its slot: one tensor copy, or this thread's cells with
@@ -112,26 +121,16 @@ struct StarFixMarch {
         }
     }
 
-    // Marches from plane k0 at one scale; returns the first plane it did not finish.
-    // `phase`: the parity of each slot's next tensor copy (one bit per slot; every thread waits
+    // Marches from plane k0 at one scale; returns the first plane it did not finish, or k0 - 1 if the planes
+    // do not suit a scale: the ring then holds planes k0 .. k0+5 (none past k1+3) as they are.
+    // `crowded`: it ended since its list was full. `phase`: the parity of each slot's next tensor copy (one bit per slot; every thread waits
     // for every copy once); `flying`: the slots with a copy not waited for yet. `ok` turns false when a
     // wait runs out.
-    __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
-        // The cells of a plane that some point reads: a caller may leave the others (corners of the
-        // halo) unset. On planes past the segment's end only the columns themselves are read.
-        u32 full = 0, core = 0, off[NE];
-#pragma unroll
-        for (int n = 0; n < NE; ++n) {
-            const int e = tid + n * NT;
-            const int yy = e / PX, xx = e - yy * PX;
-            const bool xin = xx >= 4 && xx < w + 4, yin = yy >= 4 && yy < h + 4;
-            const bool in = xx < w + 8 && yy < h + 8 && e < PLANE && (xin || yin);
-            off[n] = in ? (u32)(yy * (int)g.isy + xx) : 0u;
-            if (in) full |= 1u << n;
-            if (xin && yin) core |= 1u << n;
-        }
-        // Tensor copies bring every cell: only tiles at the grid's rim drop the ones not read.
-        const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 4 > g.nx || j0 + BY + 4 > g.ny);
+    __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok, bool& crowded) const {
+        crowded = false;
+        u32 full, core, off[NE];
+        cells_read(full, core, off);
+        const bool rim = at_rim();
         if (TMA && !rim) full = ~0u;
         auto keep = [&](int q) { return q < k1 ? full : core; };
         const bool work = ty < h;
@@ -190,7 +189,20 @@ struct StarFixMarch {
         top = note[0];
         const bool zero = top == 0;
         int E0 = (int)(top >> 20);
-        const bool fits = zero || (E0 >= kFixMinExp && E0 <= kFixMaxExp);   // not if a wait ran out, either
+        if (!zero && (E0 < kFixMinExp || E0 > kFixMaxExp)) return k0 - 1;   // so, too, if a wait ran out
+        if (!zero) {
+            // Mostly small values: the list would be longer than the rest is worth.
+            int seen = 0, few = 0;
+            for (int q = 0; q < next - k0 && k0 + q < k1; ++q)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (!valid(c)) continue;
+                    ++seen;
+                    few += (int)((u32)lds_int(mine + q * (PLANE * 8) + c * 8 + 4) << 1 >> 21) < E0 - kStarSmallBits;
+                }
+            const int crowd = __syncthreads_count(2 * few > seen), all = __syncthreads_count(seen > 0);
+            if (2 * crowd > all) return k0 - 1;
+        }
         if (zero) E0 = kFixMinExp;
         int bad = 0;
         constexpr u32 bias = kStarBiasHi + kStarSmallHi;
@@ -211,14 +223,12 @@ struct StarFixMarch {
             if (TMA) fence_proxy_async();
         };
         int kk = k0;
-        if (fits) {
 #pragma unroll 1
-            for (int q = 0; q < next - k0; ++q) convert(q, k0 + q);
+        for (int q = 0; q < next - k0; ++q) convert(q, k0 + q);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int c = 0; c < 2; ++c) past[q][c] = to_fixed(past[q][c], E0, bias, bad);
-        }
+            for (int c = 0; c < 2; ++c) past[q][c] = to_fixed(past[q][c], E0, bias, bad);
         const FixOut fo = fix_out(E0 - 1023 - 59 + fx.shift, fx.neg != 0);
         const u32 small = zero ? 0u : 2 * kStarSmallHi;
         // + 1: the two floors in the joined sum lose half a unit each on average.
@@ -233,7 +243,7 @@ struct StarFixMarch {
         int cur = 0;   // the slot of plane kk
         __syncthreads();
 #pragma unroll 1
-        for (; fits && kk < k1; kk += 2) {
+        for (; kk < k1; kk += 2) {
             const bool two = kk + 1 < k1;
             double av[2][2];
 #pragma unroll
@@ -371,6 +381,7 @@ av[j][c] *= from_fixed((i64)sum, fo);
         // The listed points (of finished planes), by all threads.
         __syncthreads();
         const u32 listed = min(note[1], (u32)S::LIST);
+        crowded = note[1] > (u32)S::LIST;
         for (u32 n = tid; n < listed; n += NT) {
             const int x = list[n] % BX, y = list[n] / BX % BY, q = k0 + (int)(list[n] / (BX * BY));
             if (q >= kk) continue;
@@ -381,17 +392,20 @@ av[j][c] *= from_fixed((i64)sum, fo);
     }
 };
 
-// One block's work: the BX x BY column tile at (i0, j0), z-planes [k0, k1). Ends with all threads
-// past a barrier after their last shared-memory read. A segment that meets a value beyond its scale
-// (or too many points below it) ends early and the next one starts with a scale of its own;
-// after several short ones the rest of the planes is evaluated in FP64.
+// One block's work: the BX x BY column tile at (i0, j0), z-planes [k0, k1). Ends with all threads past a
+// barrier after their last shared-memory access. A segment that meets a value beyond its scale (or too
+// many points below it) ends early and the next one starts with a scale of its own. Returns the first
+// plane that is left for star_rest (k1 if none): after several short segments, after one that filled its
+// list within 16 planes (an eighth of its points), or where the planes at hand do not suit a scale;
+// `raw`: the ring then holds them.
 template <int BX, int BY, bool TMA, bool ISO>
-__device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, const double* __restrict__ a,
-                                                 double* __restrict__ out, const Geom& g, const StarCoef& cf,
-                                                 const StarFix& fx, int i0, int j0, int k0, int k1, double* smem,
-                                                 const CUtensorMap* map, unsigned* tmo) {
+__device__ __forceinline__ int star_fixed_march(const double* __restrict__ u, const double* __restrict__ a,
+                                                double* __restrict__ out, const Geom& g, const StarCoef& cf,
+                                                const StarFix& fx, int i0, int j0, int k0, int k1, double* smem,
+                                                const CUtensorMap* map, unsigned* tmo, int tid, bool& raw) {
     using S = StarFixShape<BX, BY>;
-    const int tid = threadIdx.x;
+    raw = false;
+    if (g.isy >= (1 << 22)) return k0;   // staging offsets are 32 bits
     // A tile cut by the grid's x edge packs its column pairs into the first threads (see star_march).
     const int w = min(BX, g.nx - i0), h = min(BY, g.ny - j0), wp = (w + 1) / 2;
     u64* ring = reinterpret_cast<u64*>(align128(smem));
@@ -410,19 +424,16 @@ __device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, c
     u32 phase = 0, flying = 0;
     bool ok = true;
     int kk = k0;
-    if (g.isy >= (1 << 22)) {   // staging offsets are 32 bits
-        m.plain(k0);
-        kk = k1;
-    }
-    for (int left = 4; kk < k1; --left) {
-        const int done = m.segment(kk, phase, flying, ok);
+    for (int left = 4; kk < k1 && ok; --left) {
+        bool crowded;
+        const int done = m.segment(kk, phase, flying, ok, crowded);
         ok = block_ok(ok);   // (a barrier: the ring and the notes are free again)
+        raw = done < kk;
+        if (raw) break;
+        const bool stop = done == kk || (crowded && done - kk < 16);
         left += (done - kk) / 16;
-        if (done == kk || left <= 0 || !ok) {
-            m.plain(done);
-            break;
-        }
         kk = done;
+        if (stop || left <= 0) break;
     }
     if (TMA) {
         // Copies may still be in flight after a wait of thread 0 ran out (another thread's: it has seen them
@@ -435,6 +446,153 @@ __device__ __forceinline__ void star_fixed_march(const double* __restrict__ u, c
             for (int s = 0; s < S::NSLOT; ++s) mbar_inval(reinterpret_cast<uint64_t*>(bars + s));
         __syncthreads();
     }
+    raw = raw && ok;
+    return kk;
+}
+
+// The planes [k0, k1) of a column in FP64, with star_march's operations in their order: two neighbours along x
+// per thread and the ring of eight planes above, staged three steps ahead. A function of its own: inlined, it
+// cost the fixed-point march registers (384^3 595 -> 645 us). `raw`: planes k0 .. k0+5 are in
+// slots 0 .. 5, and no copy is in flight. Bound by the FP64 pipe like star_march; a field whose every
+// point comes here (384^3, see star_fixed_march) runs as fast as in that kernel.
+template <int BX, int BY, bool TMA>
+__device__ __noinline__ void star_rest(const double* __restrict__ u, const double* __restrict__ a, double* __restrict__ out,
+                                          const Geom& g, const StarCoef& cfc, int i0, int j0, int k0, int k1,
+                                          const CUtensorMap* map, unsigned* tmo, bool raw) {
+    extern __shared__ __align__(128) double smem[];
+    using S = StarFixShape<BX, BY>;
+    constexpr int PX = S::PX, PLANE = S::PLANE, HELD = 6;
+    static_assert(S::LIST * sizeof(u32) >= sizeof(StarCoef), "the weights take the list's place");
+    const int tid = tid_x();
+    const int w = min(BX, g.nx - i0), h = min(BY, g.ny - j0), wp = (w + 1) / 2;
+    const int tx = 2 * (w == BX ? tid % (BX / 2) : tid % wp), ty = w == BX ? tid / (BX / 2) : tid / wp;
+    const bool v0 = ty < h && tx < w, v1 = ty < h && tx + 1 < w;
+    double* ring = align128(smem);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(ring + S::NSLOT * PLANE);
+    double* Cs = reinterpret_cast<double*>(bars + S::NSLOT + 1);
+    const u32 own = v0 ? ((ty + 4) * PX + tx + 4) * 8 : (4 * PX + 4) * 8, rs = smem_addr(ring);
+    const int top = k1 + 3;   // the last plane needed
+    auto slot = [&](int q) { return (q - k0) & 7; };
+    // Fills of a slot are counted from the barriers' start: the planes at hand are none.
+    auto parity = [&](int q) { return (u32)(((q - k0) >> 3) - (raw && slot(q) < HELD)) & 1u; };
+    bool ok = true;
+    int lost = 0x7fffffff, issued = 0;   // thread 0: the plane whose wait ran out, the last one under way
+    auto stage = [&](int q) {
+        if (TMA) {
+            if (tid == 0 && ok) {
+                fence_proxy_async();
+                mbar_arrive_expect_tx(bars + slot(q), PLANE * 8);
+                tma_load_3d(ring + slot(q) * PLANE, map, bars + slot(q), i0 - 4 + g.halo, j0 - 4 + g.halo, q + g.halo);
+                issued = q;
+            }
+        } else {
+            const double* base = u + (i64)(q + g.halo) * g.isz + (i64)(j0 - 4 + g.halo) * g.isy + (i0 - 4 + g.halo);
+            const int xlim = min(PX, g.nx + 8 - i0), ylim = min(S::PY, g.ny + 8 - j0);
+#pragma unroll 1
+            for (int e = tid; e < PLANE; e += S::NT) {
+                const int yy = e / PX, xx = e - yy * PX;
+                if (xx < xlim && yy < ylim) cp_async8(ring + slot(q) * PLANE + e, base + (i64)yy * g.isy + xx);
+            }
+        }
+    };
+    auto landed = [&](int q) {
+        if (!TMA || !ok) return;
+        ok = mbar_wait_bounded(bars + slot(q), parity(q), tmo);
+        if (!ok) lost = q;
+    };
+    stage_consts_write(Cs, cfc, tid);
+    if (TMA) {
+        if (tid == 0) {
+            for (int s = 0; s < S::NSLOT; ++s) mbar_init(bars + s, 1);
+            fence_mbar_init();
+        }
+        __syncthreads();
+    }
+    // (Element-wise: planes k0 .. k0+4 in one group, each further one in a group of its own.)
+    for (int q = raw ? k0 + HELD : k0; q <= k0 + 6; ++q) {
+        if (q <= top) stage(q);
+        if (!TMA && q >= k0 + 4) cp_async_commit();
+    }
+    if (!raw) {
+        for (int q = k0; q <= k0 + 4; ++q) landed(q);
+        if (!TMA) cp_async_wait_group2();
+    }
+    __syncthreads();
+    const StarCoef cf = stage_consts_read<StarCoef>(Cs);
+    const Pipe& p = cf.pp;
+    auto pair = [&](u32 at, double (&v)[2]) {
+        const U64x2 t = lds2(at);
+        v[0] = __longlong_as_double((long long)t.x);
+        v[1] = __longlong_as_double((long long)t.y);
+    };
+    double zq[9][2];   // the columns' values at planes kk-4 .. kk+4
+    const i64 at0 = (i64)(k0 + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + g.halo);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        zq[m][0] = v0 ? __ldg(u + at0 + (m - 4) * g.isz) : 0.0;
+        zq[m][1] = v1 ? __ldg(u + at0 + (m - 4) * g.isz + 1) : 0.0;
+    }
+#pragma unroll
+    for (int m = 4; m < 9; ++m) pair(rs + slot(k0 + m - 4) * (PLANE * 8) + own, zq[m]);
+    const double* ap = a + at0;
+    double* op = out + (i64)k0 * g.osz + (i64)(j0 + ty) * g.osy + i0 + tx;
+#pragma unroll 1
+    for (int kk = k0; kk < k1; ++kk) {
+        if (kk + 7 <= top) stage(kk + 7);   // into the slot of plane kk-1
+        if (!TMA) cp_async_commit();
+        if (v0) {
+            const u32 s0 = rs + slot(kk) * (PLANE * 8) + own;
+            double row[10];
+#pragma unroll
+            for (int x = 0; x < 10; x += 2) {
+                double v[2];
+                pair(s0 + (x - 4) * 8, v);
+                row[x] = v[0];
+                row[x + 1] = v[1];
+            }
+            double t[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                t[c] = pmul(cf.c0, zq[4][c], p);
+#pragma unroll
+                for (int o = 1; o <= 4; ++o) t[c] = fma(cf.c[o - 1], padd(row[4 + c + o], row[4 + c - o], p), t[c]);
+            }
+#pragma unroll
+            for (int o = 1; o <= 4; ++o) {
+                double yp[2], ym[2];
+                pair(s0 + o * PX * 8, yp);
+                pair(s0 - o * PX * 8, ym);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) t[c] = fma(cf.c[4 + o - 1], padd(yp[c], ym[c], p), t[c]);
+            }
+#pragma unroll
+            for (int o = 1; o <= 4; ++o)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) t[c] = fma(cf.c[8 + o - 1], padd(zq[4 + o][c], zq[4 - o][c], p), t[c]);
+            op[0] = pmul(__ldg(ap), t[0], p);
+            if (v1) op[1] = pmul(__ldg(ap + 1), t[1], p);
+        }
+        ap += g.isz;
+        op += g.osz;
+        if (kk + 5 <= top && !(raw && kk + 5 < k0 + HELD)) landed(kk + 5);
+        if (!TMA) cp_async_wait_group2();   // every group but the last two steps': plane kk+5 is there
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) zq[m][c] = zq[m + 1][c];
+        if (kk + 1 < k1) pair(rs + slot(kk + 5) * (PLANE * 8) + own, zq[8]);
+    }
+    if (TMA) {
+        if (tid == 0 && !ok && lost != 0x7fffffff)   // copies that may still be in flight: one more bounded wait each
+            for (int q = lost; q <= issued; ++q) mbar_wait_bounded(bars + slot(q), parity(q), tmo);
+        __syncthreads();
+        if (tid == 0)
+            for (int s = 0; s < S::NSLOT; ++s) mbar_inval(bars + s);
+    } else {
+        cp_async_wait_all();
+    }
+    __syncthreads();
 }
 
 }  // namespace acs

@@ -35,9 +35,10 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
                       const __grid_constant__ Geom g, const __grid_constant__ StarCoef cf,
                       const __grid_constant__ StarFix fx, int kchunk, const __grid_constant__ CUtensorMap map, unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
-    const int k0 = blockIdx.z * kchunk;
-    star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, blockIdx.x * BX, blockIdx.y * BY, k0,
-                                      min(k0 + kchunk, g.nz), smem, &map, tmo);
+    const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY, k0 = blockIdx.z * kchunk, k1 = min(k0 + kchunk, g.nz);
+    bool raw;
+    const int left = star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, i0, j0, k0, k1, smem, &map, tmo, threadIdx.x, raw);
+    if (left < k1) star_rest<BX, BY, TMA>(u, a, out, g, cf, i0, j0, left, k1, &map, tmo, raw);
 }
 
 template <int BX, int BY, int MINB, bool TMA, bool ISO>
@@ -47,11 +48,30 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
                                const __grid_constant__ StarFix fx, const __grid_constant__ BalancedPlan plan,
                                const __grid_constant__ CUtensorMap map, unsigned* tmo) {
     extern __shared__ __align__(128) double smem[];
+    __shared__ BlockLeft list[kBlockLeft];
     i64 col;
-    int z0, z1;
-    for (int n = 0; balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n)
-        star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, (int)(col % plan.ntx) * BX,
-                                          (int)(col / plan.ntx) * BY, z0, z1, smem, &map, tmo);
+    int z0, z1, n = 0, count = 0;
+    bool raw = false;
+    for (; count < kBlockLeft && balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n) {
+        const int i0 = (int)col % plan.ntx * BX, j0 = (int)col / plan.ntx * BY;
+        const int left = star_fixed_march<BX, BY, TMA, ISO>(u, a, out, g, cf, fx, i0, j0, z0, z1, smem, &map, tmo, threadIdx.x, raw);
+        if (left < z1) {
+            if (threadIdx.x == 0) list[count] = BlockLeft{i0, j0, left, z1};
+            ++count;
+        }
+    }
+    __syncthreads();
+    // As in rhs_fixed_balanced_kernel.
+    for (int i = count - 1; i >= 0 || count == kBlockLeft; --i, raw = false) {
+        BlockLeft l;
+        if (i >= 0) {
+            l = list[i];
+        } else {
+            if (!balanced_segment(plan, blockIdx.x, n++, col, z0, z1)) break;
+            l = BlockLeft{(int)col % plan.ntx * BX, (int)col / plan.ntx * BY, z0, z1};
+        }
+        star_rest<BX, BY, TMA>(u, a, out, g, cf, l.i0, l.j0, l.from, l.to, &map, tmo, raw);
+    }
 }
 
 template <int BX, int BY, int MINB, bool TMA, bool ISO>

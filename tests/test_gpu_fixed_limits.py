@@ -8,8 +8,8 @@ import pytest
 
 import oracle
 from paper_2306_13002_gb300 import binding, inputs
-from _parity import to_dev
-from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _rhs_scale, _star
+from _parity import padded_dev, to_dev
+from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _field, _rhs_scale, _star, _star_scale
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +84,59 @@ def test_rhs_batch_fp64_rest(eps, spiked):
     for U, (_, _, R) in zip(host, grids):
         bad = ~(np.abs(R.cpu().numpy() - oracle.rhs(U, eps=eps, threads=8)) <= 2.0 ** -46 * _rhs_scale(U, 1.4, eps, (1.0,) * 3))
         assert not bad.any(), (U.shape, np.argwhere(bad)[:3])
+
+
+@pytest.mark.parametrize("bxy", [(16, 8), (32, 8), (64, 4), (16, 16)])
+@pytest.mark.parametrize("flags", [0, 2])
+@pytest.mark.parametrize("kind", ["lumps", "growing", "pulse", "tiny"])
+@pytest.mark.parametrize("kchunk", [1, 2, 3, 5, 6, 7, 8, 9, 20])
+def test_star_fp64_rest(kchunk, kind, flags, bxy):
+    """Planes left for FP64: by the scan (mostly small values, values below the scales' range), by several
+    short segments, by a full list; chunks as short as the planes a scan leaves in the ring and longer."""
+    nx, ny, nz = 75, 34, 41
+    u = _field("plain" if kind == "tiny" else kind, (nz + 8, ny + 8, nx + 8), 38)
+    a = np.random.default_rng(39).uniform(-1.0, 1.0, u.shape)
+    s = 2.0 ** -900 if kind == "tiny" else 1.0
+    got, ref = _star(u * s, a, TAYLOR, (*bxy, kchunk, flags)) / s, oracle.stencil(u, a, TAYLOR, threads=4)
+    bad = ~(np.abs(got - ref) <= 2.0 ** -46 * _star_scale(u, a, TAYLOR))
+    assert not bad.any(), (int(bad.sum()), np.argwhere(bad)[:3])
+
+
+@pytest.mark.parametrize("flags", [1, 3])
+@pytest.mark.parametrize("every", [1, 7, 50])
+def test_star_fp64_rest_of_many_columns(every, flags):
+    """A balanced launch on a thin grid: 17 columns and more per block, all of them, some or a few with values
+    that do not suit a scale."""
+    nx, ny, nz = 2310, 1150, 2
+    rng = np.random.default_rng(40)
+    shape = (nz + 8, ny + 8, nx + 8)
+    u = rng.uniform(-1.0, 1.0, shape)
+    y, x = np.meshgrid(np.arange(shape[1]), np.arange(shape[2]), indexing="ij")
+    odd = ((x // 16) + 145 * (y // 8)) % every == 0
+    u[:, odd] *= 2.0 ** rng.integers(-60, 1, (shape[0], int(odd.sum())))
+    a = rng.uniform(-1.0, 1.0, shape)
+    got, ref = _star(u, a, TAYLOR, (16, 8, 0, flags)), oracle.stencil(u, a, TAYLOR, threads=8)
+    bad = ~(np.abs(got - ref) <= 2.0 ** -46 * _star_scale(u, a, TAYLOR))
+    assert not bad.any(), (int(bad.sum()), np.argwhere(bad)[:3])
+
+
+@pytest.mark.parametrize("pitch", [0, 1])
+def test_star_batch_fp64_rest(pitch):
+    """A batch of which some grids are pulses, some uniform and some values far apart; both stagings."""
+    host, grids = [], []
+    for q, (nx, ny, nz) in enumerate([(64, 48, 50), (50, 46, 61), (34, 70, 40), (80, 31, 45), (48, 48, 48), (16, 90, 50)]):
+        shape = (nz + 8, ny + 8, nx + 8)
+        u = _field(("plain", "pulse", "lumps", "zeros", "growing", "wave")[q], shape, 41 + q)
+        a = np.random.default_rng(50 + q).uniform(-1.0, 1.0, shape)
+        ud, ad = padded_dev(u, nx + 8 + pitch), padded_dev(a, nx + 8 + pitch)
+        host.append((u, a))
+        grids.append((ud, ad, torch.full((nz, ny, nx), float("nan"), dtype=torch.float64, device="cuda")))
+    ws = torch.zeros(binding.acs_batch_workspace_bytes(len(grids)) // 8 + 2, dtype=torch.float64, device="cuda")
+    for c in (None, [[w / (h * h) for w in binding.TAYLOR8] for h in (1.0, 0.8, 1.25)]):
+        plan = binding.acs_batch_prepare(binding.KIND_STENCIL, grids, ws)
+        binding.acs_batch_launch(plan, c)
+        torch.cuda.synchronize()
+        cn = TAYLOR if c is None else np.array(c)
+        for (u, a), (_, _, out) in zip(host, grids):
+            bad = ~(np.abs(out.cpu().numpy() - oracle.stencil(u, a, cn, threads=4)) <= 2.0 ** -46 * _star_scale(u, a, cn))
+            assert not bad.any(), (u.shape, int(bad.sum()), np.argwhere(bad)[:3])
