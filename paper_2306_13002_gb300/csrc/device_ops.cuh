@@ -144,10 +144,11 @@ struct RhsFix {
 // The weights as integers for the fixed-point star march (star_fixed.cuh): c = (wh 2^LB + wl) 2^-w
 // with wh signed, index 0 the centre, then one axis (kind 1: the three axes share their weights,
 // LB 29) or three (kind 2, LB 28). The joined sum counts in units of 2^(LB + 29 - w) = 2^shift of
-// the inputs' unit; `neg`: the weights were negated to make the centre's negative. kind 0: the
+// the inputs' unit; `neg`: the weights were negated to make the centre's negative; `small`: the
+// upper half of the small-value bound, `zmask` 0: the +z neighbour does not count for it. kind 0: the
 // weights do not suit (star_fix).
 struct StarFix {
-    unsigned wh[13], wl[13];
+    unsigned wh[13], wl[13], small, zmask;
     int shift, kind, neg;
 };
 

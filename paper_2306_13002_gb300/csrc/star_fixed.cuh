@@ -22,11 +22,16 @@
 
 namespace acs {
 
-// Inputs smaller than 2^-10 of the segment's scale (u(p) and its +x and +y neighbours, all
-// three) send the point to the FP64 form.
+// A point is small if u(p) and its +x, +y and +z neighbours, all four, are below 2^53 units (2^-6 to 2^-7 of
+// the segment's largest value): it is evaluated in FP64. The conversion's errors (0.3 unit of each input,
+// so mostly the centre weight's share, 2.7 units for Taylor weights) are then no larger than FP64's
+// roundings at any other point, relative to its sum of |terms|: a host emulation of both sums gives,
+// with all inputs just above the bound, 4.5e-17 against 8.1e-17 (of one sign and alike 2.9e-17 against
+// 4.0e-17), and with one input there and the others far below, 1.5e-16 (+x or +y) and 1.1e-16 (centre)
+// against 1.4e-16 to 1.7e-16. Weights whose nearest ones are a smaller share of the centre's raise the bound by
+// that (StarFix::small), or leave +z out.
 constexpr u32 kStarBiasHi = 1u << 28;            // 2^60: the offset that keeps inputs unsigned
-constexpr u32 kStarSmallHi = 1u << 18;           // 2^50: the small-value bound
-constexpr int kStarSmallBits = 9;                // below E0 by more: small (2^50 is 2^-9 of 2^59)
+constexpr u32 kStarSmallHi = 1u << 21;           // 2^53
 constexpr int kStarIsoLB = 29, kStarGenLB = 28;  // bits of Wl (see StarFix)
 
 // The sum at one point in FP64, from global memory: the saturated form's operations in their order.
@@ -193,19 +198,20 @@ struct StarFixMarch {
         if (!zero) {
             // Mostly small values: the list would be longer than the rest is worth.
             int seen = 0, few = 0;
+            const int low = ISO ? 6 : 59 - (63 - __clz((int)fx.small));   // 2^53: 6 below the leading bit
             for (int q = 0; q < next - k0 && k0 + q < k1; ++q)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
                     if (!valid(c)) continue;
                     ++seen;
-                    few += (int)((u32)lds_int(mine + q * (PLANE * 8) + c * 8 + 4) << 1 >> 21) < E0 - kStarSmallBits;
+                    few += (int)((u32)lds_int(mine + q * (PLANE * 8) + c * 8 + 4) << 1 >> 21) < E0 - low;
                 }
             const int crowd = __syncthreads_count(2 * few > seen), all = __syncthreads_count(seen > 0);
             if (2 * crowd > all) return k0 - 1;
         }
         if (zero) E0 = kFixMinExp;
         int bad = 0;
-        constexpr u32 bias = kStarBiasHi + kStarSmallHi;
+        const u32 bound = ISO ? kStarSmallHi : fx.small, bias = kStarBiasHi + bound;
         // This thread's cells of plane q from raw to fixed point, in place.
         auto convert = [&](int slot, int q) {
             if (zero) {
@@ -230,7 +236,7 @@ struct StarFixMarch {
 #pragma unroll
             for (int c = 0; c < 2; ++c) past[q][c] = to_fixed(past[q][c], E0, bias, bad);
         const FixOut fo = fix_out(E0 - 1023 - 59 + fx.shift, fx.neg != 0);
-        const u32 small = zero ? 0u : 2 * kStarSmallHi;
+        const u32 small = zero ? 0u : 2 * bound;
         // + 1: the two floors in the joined sum lose half a unit each on average.
         const u64 round = zero ? 0 : 1;
         const i64 at0 = (i64)(k0 + g.halo) * g.isz + (i64)(j0 + ty + g.halo) * g.isy + (i0 + tx + g.halo);
@@ -298,7 +304,7 @@ struct StarFixMarch {
                             if (o == 1) {
                                 nh[c] = hi32(row[4 + c]);
                                 nl[c] = lo32(row[4 + c]);
-                                least = min(least, nh[c] ^ kStarBiasHi);
+                                least = min(least, (nh[c] ^ kStarBiasHi) | (hi32(xp) ^ kStarBiasHi) | (hi32(yp) ^ kStarBiasHi));
                             }
                             if (ISO) {
                                 const u64 sm = (xp + xm + yp) + (ym + zp + zm);
@@ -343,14 +349,14 @@ av[j][c] *= from_fixed((i64)sum, fo);
                     past[1][c] = here[0][c];
                     past[0][c] = here[1][c];
                 }
-                if (least < small) {   // a point whose neighbours are small, too, goes on the list
+                if (least < small) {   // some of the four points may go on the list
 #pragma unroll 1
                     for (int p = 0; p < 4; ++p) {
                         const int j = p >> 1, c = p & 1;
                         if (!(c ? v1 : v0) || (j && !two)) continue;
-                        const u32 q = mine + (((cur + j) & 7) * PLANE + c) * 8;
+                        const u32 q = mine + (((cur + j) & 7) * PLANE + c) * 8, qz = mine + (((cur + j + 1) & 7) * PLANE + c) * 8;
                         if (((hi32(lds1(q)) ^ kStarBiasHi) | (hi32(lds1(q + 8)) ^ kStarBiasHi) |
-                             (hi32(lds1(q + PX * 8)) ^ kStarBiasHi)) >= small)
+                             (hi32(lds1(q + PX * 8)) ^ kStarBiasHi) | ((hi32(lds1(qz)) ^ kStarBiasHi) & (ISO ? ~0u : fx.zmask))) >= small)
                             continue;
                         const u32 at = atomicAdd(note + 1, 1u);
                         if (at < (u32)S::LIST)

@@ -42,6 +42,13 @@ void star_fix(const StarCoef& c, StarFix& fx) {
     put(0, (iso ? -6 : -2) * total);
     fx.shift = LB + 29 - w;
     fx.neg = sg < 0.0;
+    // The bound's reasoning takes a point's sum of |terms| for at least a nearest weight times the bound; Taylor
+    // weights with the same spacing on every axis have 0.187 of the centre's there. Up to a power of
+    // two (but for a tenth), 2^4 at most by the tests above (2^57, an eighth of the scale).
+    double least = std::fmin(std::fabs(c.c[0]), std::fabs(c.c[4]));
+    fx.zmask = std::fabs(c.c[8]) >= 0.5 * least ? ~0u : 0u;
+    if (fx.zmask) least = std::fmin(least, std::fabs(c.c[8]));
+    fx.small = kStarSmallHi << (least < 0.187 * mid ? std::ilogb(1.8 * 0.187 * mid / least) : 0);
     fx.kind = iso ? 1 : 2;
 }
 

@@ -140,3 +140,73 @@ def test_star_batch_fp64_rest(pitch):
         for (u, a), (_, _, out) in zip(host, grids):
             bad = ~(np.abs(out.cpu().numpy() - oracle.stencil(u, a, cn, threads=4)) <= 2.0 ** -46 * _star_scale(u, a, cn))
             assert not bad.any(), (u.shape, int(bad.sum()), np.argwhere(bad)[:3])
+
+
+@pytest.mark.parametrize("tile", TILES)
+@pytest.mark.parametrize("h", [(1.0, 1.0, 1.0), (1.0, 0.8, 1.25), (1.0, 1.0, 0.4)])
+def test_star_points_far_below_the_scale_are_as_exact_as_fp64(tile, h):
+    """Single values of 1 to 2^-12 among values of 2^-20, no two in reach of one point: a point's error, relative
+    to its sum of |terms|, whatever the block's largest value is. An FP64 sum of one such value in any place
+    has 1.3e-16 to 1.7e-16 (root mean square; emulated), at most 8.1e-16. 2.2e-16 and 1.3e-15 leave room for
+    weights that share the bound to the nearest power of two (a factor of 1.4)."""
+    nz, ny, nx = 68, 62, 70
+    rng = np.random.default_rng(42)
+    u = rng.uniform(-1.0, 1.0, (nz + 8, ny + 8, nx + 8)) * 2.0 ** -20
+    z, y, x = np.meshgrid(*(np.arange(0, n, 9) for n in u.shape), indexing="ij")
+    big = rng.uniform(1.0, 2.0, z.shape) * 2.0 ** -rng.integers(1, 13, z.shape) * rng.choice([-1.0, 1.0], z.shape)
+    u[z, y, x] = np.where(rng.random(z.shape) < 0.25, 1.0, big)
+    a = np.ones(u.shape)
+    c = np.array([[w / (s * s) for w in binding.TAYLOR8] for s in h])
+    got = _star(u, a, c, tile)
+    L = np.longdouble
+    v, ref, scale = u.astype(L), np.zeros(got.shape, L), np.zeros(got.shape)
+    for d in range(3):
+        for o in range(1, 5):
+            s = [slice(4, -4)] * 3
+            p, m = list(s), list(s)
+            n = u.shape[2 - d]
+            p[2 - d], m[2 - d] = slice(4 + o, n - 4 + o), slice(4 - o, n - 4 - o)
+            ref += L(c[d][o - 1]) * (v[tuple(p)] - 2 * v[tuple(s)] + v[tuple(m)])
+            scale += abs(c[d][o - 1]) * (np.abs(u[tuple(p)]) + 2 * np.abs(u[tuple(s)]) + np.abs(u[tuple(m)]))
+    err = (np.abs(got.astype(L) - ref) / scale).astype(np.float64)
+    octave = np.floor(np.log2(scale / np.abs(c).max())).astype(int)
+    for k in range(-12, 1):
+        e = err[octave == k]
+        assert e.size > 50 and np.sqrt(np.mean(e * e)) <= 2.2e-16 and e.max() <= 1.3e-15, (k, e.size, np.sqrt(np.mean(e * e)), e.max())
+
+
+@pytest.mark.parametrize("tile", TILES)
+@pytest.mark.parametrize("h", [(1.0, 1.0, 1.0), (1.0, 0.8, 1.25)])
+def test_star_points_near_the_small_value_bound(tile, h):
+    """Values of 2^-9 to 2^-3 alone in small balls of a field of ordinary ones, so that the block keeps its
+    scale: the points whose only large term is their own value or their +x, +y or +z neighbour's. Bounds
+    as above."""
+    n, L = 96, np.longdouble
+    c = np.array([[w / (s * s) for w in binding.TAYLOR8] for s in h])
+    got, errs = None, []
+    for seed in range(4):
+        rng = np.random.default_rng(4300 + seed)
+        u = rng.uniform(-1.001, 1.001, (n + 8,) * 3)
+        i = 16 + 24 * np.stack(np.meshgrid(*[np.arange(4)] * 3, indexing="ij")).reshape(3, -1) + rng.integers(-3, 4, (3, 64))
+        z, y, x = np.meshgrid(*[np.arange(n + 8)] * 3, indexing="ij", sparse=True)
+        for k, j, m in i.T:
+            ball = (z - k) ** 2 + (y - j) ** 2 + (x - m) ** 2 <= 36
+            u[ball] *= 2.0 ** -20
+        u[tuple(i)] = rng.uniform(1.0, 2.0, 64) * 2.0 ** -rng.integers(4, 10, 64) * rng.choice([-1.0, 1.0], 64)
+        got = _star(u, np.ones(u.shape), c, tile)
+        for off in ((0, 0, 0), (0, 0, -1), (0, -1, 0), (-1, 0, 0)):
+            p = i + np.array(off)[:, None]
+            ref, scale = np.zeros(64, L), np.zeros(64)
+            for d in range(3):
+                for o in range(1, 5):
+                    s = np.zeros((3, 1), int)
+                    s[2 - d] = o
+                    a, b, m = u[tuple(p + s)], u[tuple(p)], u[tuple(p - s)]
+                    ref += L(c[d][o - 1]) * (a.astype(L) - 2 * b.astype(L) + m.astype(L))
+                    scale += abs(c[d][o - 1]) * (np.abs(a) + 2 * np.abs(b) + np.abs(m))
+            e = (np.abs(got[tuple(p - 4)].astype(L) - ref) / scale).astype(np.float64)
+            errs.append(np.stack([np.floor(np.log2(np.abs(u[tuple(i)]))), e]))
+    octave, e = np.concatenate(errs, axis=1)
+    for k in range(-9, -3):
+        v = e[octave == k]
+        assert v.size > 50 and np.sqrt(np.mean(v * v)) <= 2.2e-16 and v.max() <= 1.3e-15, (k, np.sqrt(np.mean(v * v)), v.max())
