@@ -152,7 +152,8 @@ static size_t batch_table_bytes(int n) { return kHeader + desc_bytes(n) + sizeof
 size_t batch_ws_bytes(int n) { return n < 1 ? 0 : batch_table_bytes(n) + 128 + sizeof(CUtensorMap) * (size_t)n; }
 
 // Host half of acs_batch_prepare: geometry already validated; builds the packed image.
-acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int kind, const acs_tile& tile,
+// Clears ACS_TILE_TMA in the tile if not every grid can be staged so.
+acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int kind, acs_tile& tile,
                       uintptr_t ws_addr, std::vector<unsigned char>& image, long long& total) {
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
@@ -221,6 +222,7 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
             set_error("%s", "");
         }
     }
+    if (!tma) tile.flags &= ~ACS_TILE_TMA;
     if (tma) {
         const uintptr_t first = (ws_addr + batch_table_bytes(n) + 127) & ~(uintptr_t)127;
         h.maps_off = (int)(first - ws_addr);

@@ -9,7 +9,7 @@
 namespace acs {
 namespace {
 
-template <int BX, int BY, bool ISO, int MINB>
+template <int BX, int BY, bool TMA, bool ISO, int MINB>
 __global__ void __launch_bounds__(BX* BY / 2, MINB)
     batch_star_fixed_kernel(const unsigned char* __restrict__ ws, unsigned long long* counter,
                             const __grid_constant__ StarCoef cf, const __grid_constant__ StarFix fx, unsigned* tmo) {
@@ -22,17 +22,15 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
         const BatchDesc& d = b.items[u.item];
         const Geom g = d.g;
         const int i0 = u.tx * BX, j0 = u.ty * BY;
-        bool raw;
-        if (d.tma) {
-            const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(ws + b.head->maps_off) + u.item;
+        const CUtensorMap* map = nullptr;
+        if (TMA) {
+            map = reinterpret_cast<const CUtensorMap*>(ws + b.head->maps_off) + u.item;
             if (threadIdx.x == 0) tensormap_acquire(map);
-            const int left = star_fixed_march<BX, BY, true, ISO>(d.in0, d.in1, d.out, g, cf, fx, i0, j0, u.k0, u.k1, smem, map, tmo, tid_x(), raw);
-            if (left < u.k1) star_rest<BX, BY, true>(d.in0, d.in1, d.out, g, cf, i0, j0, left, u.k1, map, tmo, raw);
-        } else {
-            const int left = star_fixed_march<BX, BY, false, ISO>(d.in0, d.in1, d.out, g, cf, fx, i0, j0, u.k0, u.k1, smem,
-                                                                  nullptr, nullptr, tid_x(), raw);
-            if (left < u.k1) star_rest<BX, BY, false>(d.in0, d.in1, d.out, g, cf, i0, j0, left, u.k1, nullptr, nullptr, raw);
         }
+        bool raw;
+        const int left = star_fixed_march<BX, BY, TMA, ISO>(d.in0, d.in1, d.out, g, cf, fx, i0, j0, u.k0, u.k1, smem, map, tmo,
+                                                            tid_x(), raw);
+        if (left < u.k1) star_rest<BX, BY, TMA>(d.in0, d.in1, d.out, g, cf, i0, j0, left, u.k1, map, tmo, raw);
     }
 }
 
@@ -52,8 +50,8 @@ __global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
         if (!batch_next(b, counter, &s_unit, leader, u)) return;
         const BatchDesc& d = b.items[u.item];
         const Geom g = d.g;
-        left = rhs_fixed_march<BX, BY, false, ISO>(d.in0, d.out, g, kc, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, nullptr,
-                                                   nullptr, raw);
+        left = rhs_fixed_march<BX, BY, false, ISO, true>(d.in0, d.out, g, kc, fx, u.tx * BX, u.ty * BY, u.k0, u.k1, smem, nullptr,
+                                                   nullptr, threadIdx.y * BX + threadIdx.x, raw);
         if (left < u.k1) break;
     }
     // A block that met values that do not fit takes its further units in FP64 as well: what does not fit in
@@ -84,10 +82,10 @@ acs_status launch_star_t(const BatchPlanHost& p, unsigned long long* counter, co
     unsigned* tmo = wait_timeout_counter();
     if (!tmo) return fail(ACS_ERR_CUDA, "cannot address the wait-timeout counter");
     using S = StarFixShape<BX, BY>;
-    return fx.kind == 1 ? launch_batch(batch_star_fixed_kernel<BX, BY, true, MINB>, dim3(S::NT), S::BYTES, p, s,
-                                       "batch_star_fixed_kernel", counter, sc, fx, tmo)
-                        : launch_batch(batch_star_fixed_kernel<BX, BY, false, MINB>, dim3(S::NT), S::BYTES, p, s,
-                                       "batch_star_fixed_kernel", counter, sc, fx, tmo);
+    auto run = [&](auto kernel) { return launch_batch(kernel, dim3(S::NT), S::BYTES, p, s, "batch_star_fixed_kernel", counter, sc, fx, tmo); };
+    if (p.tile.flags & ACS_TILE_TMA)   // all grids have tensor maps (batch_pack)
+        return fx.kind == 1 ? run(batch_star_fixed_kernel<BX, BY, true, true, MINB>) : run(batch_star_fixed_kernel<BX, BY, true, false, MINB>);
+    return fx.kind == 1 ? run(batch_star_fixed_kernel<BX, BY, false, true, MINB>) : run(batch_star_fixed_kernel<BX, BY, false, false, MINB>);
 }
 
 template <int BX, int BY>

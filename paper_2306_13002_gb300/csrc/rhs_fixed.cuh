@@ -153,8 +153,7 @@ struct RhsFixMarch {
     // Marches from plane k0; returns the first plane not finished, or k0 - 1 if the scanned planes do not
     // fit: the ring then holds planes k0-2 .. k0+3 (none past k1+1) as they are. `phase`, `flying`, `ok`: as
     // StarFixMarch::segment.
-    __device__ __forceinline__ int segment(int k0, u32& phase, u32& flying, bool& ok) const {
-        const int tid = tid_y() * BX + tid_x();
+    __device__ __forceinline__ int segment(int k0, int tid, u32& phase, u32& flying, bool& ok) const {
         const u32 rs = smem_addr(smem), fxs = rs + NSLOT * S::CELLS * 8, fys = fxs + S::FX_ELEMS * 8;
         // [0] max rho, [1] min rho, [2] max m, [3] max E, [4] min E
         int* note = reinterpret_cast<int*>(bar(NSLOT));
@@ -171,7 +170,8 @@ struct RhsFixMarch {
         // The first NR threads compute the ring's fluxes; the others stage and convert the cells.
         const int cell = tid - S::NR;
         u32 full = 0, core = 0;   // one bit per cell: read by some point on the segment's planes, and on others
-        const bool rim = TMA && (i0 == 0 || j0 == 0 || i0 + BX + 2 > g.nx || j0 + BY + 2 > g.ny);
+        // (Away from the rim all cells are values of the flow: both stagings bring and convert the corners, too.)
+        const bool rim = i0 == 0 || j0 == 0 || i0 + BX + 2 > g.nx || j0 + BY + 2 > g.ny;
         auto masks = [&]() {
             int xx = cell % PX, yy = cell / PX;
 #pragma unroll 1
@@ -184,7 +184,7 @@ struct RhsFixMarch {
                 if (xx >= PX) xx -= PX, ++yy;
                 if (yy >= S::PY) yy -= S::PY;
             }
-            if (TMA && !rim) full = ~0u;
+            if (!rim) full = ~0u;
         };
         if (!TMA) masks();
         auto keep = [&](int q) { return q >= k0 && q < k1 ? full : core; };
@@ -256,7 +256,7 @@ struct RhsFixMarch {
             for (int i = 0; i < 2; ++i) {
                 const int r = tid + i * S::NT, yy = r / PX, xx = r - yy * PX;
                 const bool xin = xx >= 2 && xx < w + 2, yin = yy >= 2 && yy < h + 2, is = r < PLANE;
-                in[i] = is && ((TMA && !rim) || (xx < w + 4 && yy < h + 4 && (xin || yin)));
+                in[i] = is && (!rim || (xx < w + 4 && yy < h + 4 && (xin || yin)));
                 mid[i] = is && xin && yin;
             }
             u32 at = rs + tid * 8 + 4;
@@ -505,7 +505,7 @@ struct RhsFixMarch {
             if (ring) {
                 if (xy_plane(q + 1)) ring_flux(sn);
             } else {   // plane q to fixed point, in place
-                const u32 m = rim || !TMA || !xy ? keep(q) : ~0u;
+                const u32 m = rim || !xy ? keep(q) : ~0u;
                 u64 v[NE];
 #pragma unroll
                 for (int n = 0; n < NE; ++n)
@@ -584,12 +584,15 @@ struct RhsFixMarch {
 // The FP64 march follows where nothing of this one lives any more, after a block's last unit. Called from
 // here it got what registers the loops over segments and units left it, and spilled: 256^3 with
 // values that never fit ran 3730 us in the balanced kernel, against 3255 for the FP64 kernel.
-template <int BX, int BY, bool TMA, bool ISO>
+//
+// `tid`: the thread's number. How it comes about decides what the compiler carries in registers across the
+// loops, and is as measured: read anew per segment (FRESH) in the batch kernel (32 grids 390 us, 425 otherwise),
+// read once by tid_x and tid_y in the balanced kernel (256^3 1113 us, 1160).
+template <int BX, int BY, bool TMA, bool ISO, bool FRESH = false>
 __device__ __forceinline__ int rhs_fixed_march(const double* __restrict__ U, double* __restrict__ R, const Geom& g,
                                                const RhsConst& kc, const RhsFix& fx, int i0, int j0, int k0, int k1,
-                                               double* smem, const CUtensorMap* map, unsigned* tmo, bool& raw) {
+                                               double* smem, const CUtensorMap* map, unsigned* tmo, int tid, bool& raw) {
     using S = RhsFixShape<BX, BY>;
-    const int tid = threadIdx.y * BX + threadIdx.x;
     const RhsFixMarch<BX, BY, TMA, ISO> m{U, R, g, kc, fx, i0, j0, k1, smem, map, tmo};
     stage_consts_write(smem + S::NSLOT * S::CELLS + S::FX_ELEMS + S::FY_ELEMS, kc, tid);
     if (tid < 5) m.scales()->seen[tid] = tid == 1 || tid == 4 ? 0x7ff : 0;
@@ -603,7 +606,7 @@ __device__ __forceinline__ int rhs_fixed_march(const double* __restrict__ U, dou
     int kk = k0;
     raw = false;
     for (int left = 4; kk < k1 && ok; --left) {
-        const int done = m.segment(kk, phase, flying, ok);
+        const int done = m.segment(kk, FRESH ? tid_y() * BX + tid_x() : tid, phase, flying, ok);
         ok = block_ok(ok);   // (a barrier: shared memory is free again)
         raw = done < kk;
         if (raw) break;

@@ -19,7 +19,8 @@ __global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
     extern __shared__ __align__(128) double smem[];
     const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY, k0 = blockIdx.z * kchunk, k1 = min(k0 + kchunk, g.nz);
     bool raw;
-    const int left = rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kc, fx, i0, j0, k0, k1, smem, &map, tmo, raw);
+    const int tid = TMA ? threadIdx.y * BX + threadIdx.x : tid_y() * BX + tid_x();   // (as measured: 1207 / 1243, 1383 / 1427 us)
+    const int left = rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kc, fx, i0, j0, k0, k1, smem, &map, tmo, tid, raw);
     if (left < k1) rhs_rest<BX, BY, TMA, ISO>(U, R, g, kf, i0, j0, left, k1, smem, &map, tmo, raw);
 }
 
@@ -36,7 +37,7 @@ __global__ void __launch_bounds__(BX* BY, RhsFixShape<BX, BY>::MINB)
     bool raw = false;
     for (; count < kBlockLeft && balanced_segment(plan, blockIdx.x, n, col, z0, z1); ++n) {
         const int i0 = (int)col % plan.ntx * BX, j0 = (int)col / plan.ntx * BY;
-        const int left = rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kc, fx, i0, j0, z0, z1, smem, &map, tmo, raw);
+        const int left = rhs_fixed_march<BX, BY, TMA, ISO>(U, R, g, kc, fx, i0, j0, z0, z1, smem, &map, tmo, tid_y() * BX + tid_x(), raw);
         if (left < z1) {
             if (threadIdx.x == 0 && threadIdx.y == 0) list[count] = BlockLeft{i0, j0, left, z1};
             ++count;

@@ -84,8 +84,11 @@ struct StarFixMarch {
 
     __device__ __forceinline__ bool valid(int c) const { return ty < h && tx + c < w; }
 
-    // The cells of a plane that some point reads, one bit each: a caller may leave the others (corners of the
-    // halo) unset. On planes past the segment's end only the columns themselves are read (core).
+    __device__ __forceinline__ bool at_rim() const { return i0 == 0 || j0 == 0 || i0 + BX + 4 > g.nx || j0 + BY + 4 > g.ny; }
+    // The cells of a plane that count, one bit each. In tiles at the grid's rim those that some point reads: a
+    // caller may leave the others (corners of the halo) unset. Elsewhere all of them, since tensor copies
+    // bring them all and both stagings have to find the same scale. On planes past the segment's end only
+    // the columns themselves (core).
     __device__ __forceinline__ void cells_read(u32& full, u32& core, u32 (&off)[NE]) const {
         full = core = 0;
 #pragma unroll
@@ -93,17 +96,12 @@ struct StarFixMarch {
             const int e = tid + n * NT;
             const int yy = e / PX, xx = e - yy * PX;
             const bool xin = xx >= 4 && xx < w + 4, yin = yy >= 4 && yy < h + 4;
-            const bool in = xx < w + 8 && yy < h + 8 && e < PLANE && (xin || yin);
+            const bool in = xx < w + 8 && yy < h + 8 && e < PLANE && (xin || yin || (!TMA && !at_rim()));
             off[n] = in ? (u32)(yy * (int)g.isy + xx) : 0u;
             if (in) full |= 1u << n;
             if (xin && yin) core |= 1u << n;
         }
     }
-    // Tensor copies bring every cell: only tiles at the grid's rim drop the ones not read.
-    __device__ __forceinline__ bool at_rim() const {
-        return TMA && (i0 == 0 || j0 == 0 || i0 + BX + 4 > g.nx || j0 + BY + 4 > g.ny);
-    }
-
     // Stages plane q (raw values) into its slot: one tensor copy, or this thread's cells with
     // cp.async (zeros for the cells no point reads).
     __device__ __forceinline__ void stage(int q, int slot, const u32 (&off)[NE], u32 keep, u32& flying) const {
@@ -135,7 +133,7 @@ struct StarFixMarch {
         crowded = false;
         u32 full, core, off[NE];
         cells_read(full, core, off);
-        const bool rim = at_rim();
+        const bool rim = TMA && at_rim();
         if (TMA && !rim) full = ~0u;
         auto keep = [&](int q) { return q < k1 ? full : core; };
         const bool work = ty < h;

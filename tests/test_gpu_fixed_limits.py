@@ -9,7 +9,7 @@ import pytest
 import oracle
 from paper_2306_13002_gb300 import binding, inputs
 from _parity import padded_dev, to_dev
-from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _field, _rhs_scale, _star, _star_scale
+from test_gpu_fixed import RHS_TILES, TAYLOR, TILES, _check_rhs, _field, _rhs, _rhs_scale, _star, _star_scale
 
 pytestmark = pytest.mark.gpu
 
@@ -210,3 +210,32 @@ def test_star_points_near_the_small_value_bound(tile, h):
     for k in range(-9, -3):
         v = e[octave == k]
         assert v.size > 50 and np.sqrt(np.mean(v * v)) <= 2.2e-16 and v.max() <= 1.3e-15, (k, np.sqrt(np.mean(v * v)), v.max())
+
+
+@pytest.mark.parametrize("kchunk,flags", [(0, 1), (5, 0), (17, 0), (64, 0)])
+@pytest.mark.parametrize("kind", ["wave", "slope", "pulse", "growing", "corner"])
+def test_stagings_agree_bitwise_where_scales_differ(kind, kchunk, flags):
+    """Tensor copies and element-wise staging take the same scales, also where a block's largest value is in a
+    corner of its halo, which no point reads."""
+    def fields(n, halo):
+        shape = tuple(v + 2 * halo for v in (60, 66, 104))
+        z, y, x = np.meshgrid(*(np.arange(v) for v in shape), indexing="ij")
+        base = np.random.default_rng(44).uniform(0.6, 1.0, (n,) + shape)
+        if kind == "slope":
+            return base * 2.0 ** (0.11 * (x + 1.7 * y) - 0.05 * z)
+        if kind == "corner":    # larger values at the crossings of every second tile's edges
+            return base * np.where((((x - halo) % 16) // 2 == 0) & (((y - halo) % 8) // 2 == 0), 5.0, 1.0)
+        return np.stack([_field(kind, shape, 45 + q) for q in range(n)]) if kind != "wave" else base * _field("wave", shape, 0)
+
+    u = fields(1, 4)[0]
+    a = np.random.default_rng(46).uniform(-1.0, 1.0, u.shape)
+    for bx, by in ((16, 8), (32, 8), (16, 16)):
+        for c in (TAYLOR, np.array([[w * s for w in binding.TAYLOR8] for s in (1.0, 1.5, 0.7)])):
+            t, e = (_star(u, a, c, (bx, by, kchunk, flags | f)) for f in (binding.TILE_TMA, 0))
+            assert np.array_equal(t, e), (bx, by, int((t != e).sum()))
+    U = fields(5, 2)
+    U[0] = np.abs(U[0]) + 0.5
+    U[4] = np.abs(U[4]) + 1.0
+    for h in ((1.0, 1.0, 1.0), (1.0, 1.5, 2.0)):
+        t, e = (_rhs(U, (16, 16, kchunk, flags | f), 1.4, 0.25, h) for f in (binding.TILE_TMA, 0))
+        assert np.array_equal(t, e), (h, int((t != e).sum()))
