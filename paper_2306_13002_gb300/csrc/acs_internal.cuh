@@ -35,6 +35,8 @@ acs_status ensure_smem(const void* fn, size_t bytes);
 acs_status launch_rhs_plain(const double* U, double* R, const Geom& g, const RhsConst& k, cudaStream_t s);
 acs_status launch_rhs_saturated(const double* U, double* R, const Geom& g, const RhsConst& k,
                                 const acs_tile& t, cudaStream_t s);
+// Whether that launch is the fixed-point march's, which has 16 x 16 columns whatever the tile.
+bool rhs_takes_fixed(const Geom& g, const RhsConst& k, const acs_tile& t);
 // The RHS in fixed point (rhs_fixed.cuh): its constants (kc: kf with |s_d|), and the launch.
 void rhs_fix(const RhsConst& kf, RhsFix& fx, RhsConst& kc);
 acs_status launch_rhs_fixed(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
@@ -59,7 +61,6 @@ acs_status launch_stencil_saturated(const double* u, const double* a, double* ou
                                     const StarCoef& c, const acs_tile& t, cudaStream_t s);
 
 // Host view of a prepared batch (mirrors acs_batch_plan).
-constexpr int kBatchPlain = 0x100;   // in a plan's tile.flags: too little work for the fixed-point RHS march
 struct BatchPlanHost {
     unsigned char* ws;
     size_t ws_bytes;

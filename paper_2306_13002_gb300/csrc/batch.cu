@@ -98,47 +98,40 @@ long long resident_t() {
     return (long long)per_sm * num_sms();
 }
 
-template <int KIND>
 acs_status dispatch(const BatchPlanHost& p, unsigned long long* counter, const RhsConst& rk, const StarCoef& sc,
                     cudaStream_t s) {
+    constexpr int K = ACS_KIND_STENCIL;
     const int bx = p.tile.bx, by = p.tile.by;
-    if (KIND == ACS_KIND_RHS) {
-        if (bx == 32 && by == 8) return launch_batch_t<32, 8, KIND>(p, counter, rk, sc, s);
-        if (bx == 32 && by == 4) return launch_batch_t<32, 4, KIND>(p, counter, rk, sc, s);
-        if (bx == 32 && by == 16) return launch_batch_t<32, 16, KIND>(p, counter, rk, sc, s);
-        if (bx == 16 && by == 8) return launch_batch_t<16, 8, KIND>(p, counter, rk, sc, s);
-        if (bx == 16 && by == 16) return launch_batch_t<16, 16, KIND>(p, counter, rk, sc, s);
-        if (bx == 64 && by == 4) return launch_batch_t<64, 4, KIND>(p, counter, rk, sc, s);
+    if (p.kind == ACS_KIND_RHS) {   // always 16 x 16 columns (batch_prepare_host)
+        if (bx == 16 && by == 16) return launch_batch_t<16, 16, ACS_KIND_RHS>(p, counter, rk, sc, s);
     } else {
-        if (bx == 32 && by == 8) return launch_batch_t<32, 8, KIND>(p, counter, rk, sc, s);
-        if (bx == 32 && by == 4) return launch_batch_t<32, 4, KIND>(p, counter, rk, sc, s);
-        if (bx == 32 && by == 16) return launch_batch_t<32, 16, KIND>(p, counter, rk, sc, s);
-        if (bx == 64 && by == 4) return launch_batch_t<64, 4, KIND>(p, counter, rk, sc, s);
-        if (bx == 64 && by == 8) return launch_batch_t<64, 8, KIND>(p, counter, rk, sc, s);
-        if (bx == 16 && by == 16) return launch_batch_t<16, 16, KIND>(p, counter, rk, sc, s);
-        if (bx == 16 && by == 8) return launch_batch_t<16, 8, KIND>(p, counter, rk, sc, s);
+        if (bx == 32 && by == 8) return launch_batch_t<32, 8, K>(p, counter, rk, sc, s);
+        if (bx == 32 && by == 4) return launch_batch_t<32, 4, K>(p, counter, rk, sc, s);
+        if (bx == 32 && by == 16) return launch_batch_t<32, 16, K>(p, counter, rk, sc, s);
+        if (bx == 64 && by == 4) return launch_batch_t<64, 4, K>(p, counter, rk, sc, s);
+        if (bx == 64 && by == 8) return launch_batch_t<64, 8, K>(p, counter, rk, sc, s);
+        if (bx == 16 && by == 16) return launch_batch_t<16, 16, K>(p, counter, rk, sc, s);
+        if (bx == 16 && by == 8) return launch_batch_t<16, 8, K>(p, counter, rk, sc, s);
     }
     return fail(ACS_ERR_UNSUPPORTED, "batch tile %dx%d is not built", bx, by);
 }
 
+// (Of the FP64 kernel, whose blocks per SM the chunk rules of batch_pack were measured with; which kernel runs
+// is known at the launch only.)
 long long resident_batch_blocks(int kind, const acs_tile& t) {
+    constexpr int K = ACS_KIND_STENCIL;
     long long r = 0;
     const int bx = t.bx, by = t.by;
     if (kind == ACS_KIND_RHS) {
-        if (bx == 32 && by == 8) r = resident_t<32, 8, ACS_KIND_RHS>();
-        if (bx == 32 && by == 4) r = resident_t<32, 4, ACS_KIND_RHS>();
-        if (bx == 32 && by == 16) r = resident_t<32, 16, ACS_KIND_RHS>();
-        if (bx == 16 && by == 8) r = resident_t<16, 8, ACS_KIND_RHS>();
         if (bx == 16 && by == 16) r = resident_t<16, 16, ACS_KIND_RHS>();
-        if (bx == 64 && by == 4) r = resident_t<64, 4, ACS_KIND_RHS>();
     } else {
-        if (bx == 32 && by == 8) r = resident_t<32, 8, ACS_KIND_STENCIL>();
-        if (bx == 32 && by == 4) r = resident_t<32, 4, ACS_KIND_STENCIL>();
-        if (bx == 32 && by == 16) r = resident_t<32, 16, ACS_KIND_STENCIL>();
-        if (bx == 64 && by == 4) r = resident_t<64, 4, ACS_KIND_STENCIL>();
-        if (bx == 64 && by == 8) r = resident_t<64, 8, ACS_KIND_STENCIL>();
-        if (bx == 16 && by == 16) r = resident_t<16, 16, ACS_KIND_STENCIL>();
-        if (bx == 16 && by == 8) r = resident_t<16, 8, ACS_KIND_STENCIL>();
+        if (bx == 32 && by == 8) r = resident_t<32, 8, K>();
+        if (bx == 32 && by == 4) r = resident_t<32, 4, K>();
+        if (bx == 32 && by == 16) r = resident_t<32, 16, K>();
+        if (bx == 64 && by == 4) r = resident_t<64, 4, K>();
+        if (bx == 64 && by == 8) r = resident_t<64, 8, K>();
+        if (bx == 16 && by == 16) r = resident_t<16, 16, K>();
+        if (bx == 16 && by == 8) r = resident_t<16, 8, K>();
     }
     // unknown (no device, or an unbuilt tile rejected later): the former estimate
     return r > 0 ? r : (long long)num_sms() * (kind == ACS_KIND_RHS ? 2 : 4);
@@ -153,7 +146,7 @@ size_t batch_ws_bytes(int n) { return n < 1 ? 0 : batch_table_bytes(n) + 128 + s
 
 // Host half of acs_batch_prepare: geometry already validated; builds the packed image.
 // Clears ACS_TILE_TMA in the tile if not every grid can be staged so.
-acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int kind, acs_tile& tile,
+acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int kind, acs_tile& tile, bool plain,
                       uintptr_t ws_addr, std::vector<unsigned char>& image, long long& total) {
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
@@ -172,7 +165,7 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     long long planes = 0;
     for (int q = 0; q < n; ++q) planes += unit_count(q, 1);
     const bool rhs = kind == ACS_KIND_RHS;
-    const bool plain = (tile.flags & kBatchPlain) != 0;   // the FP64 march, which starts at once
+    // plain: the FP64 march, which starts at once
     const int kc = plain ? std::min(tile.kchunk, 16)
                          : (int)std::min<long long>(tile.kchunk, std::max<long long>(rhs ? 8 : 16, planes / (resident * (rhs ? 2 : 1))));
     // Guided z-chunks: the grids at the end of the order, whose units make up the last two
@@ -207,6 +200,7 @@ acs_status batch_pack(const acs_batch_item* items, const Geom* geo, int n, int k
     h.bx = tile.bx;
     h.by = tile.by;
     h.kchunk = tile.kchunk;
+    h.plain = plain;
     BatchDesc* d = reinterpret_cast<BatchDesc*>(image.data() + kHeader);
     long long* prefix = reinterpret_cast<long long*>(image.data() + kHeader + desc_bytes(n));
     // Tensor maps of a star-stencil batch staged by TMA: at the first 128-byte aligned device
@@ -261,17 +255,18 @@ acs_status batch_prepare_host(const acs_batch_item* items, const Geom* geo, int 
     // Columns of an RHS batch are 16 x 16, the shape the fixed-point march is built for (whether the
     // parameters suit it is known at the launch only).
     acs_tile tile = asked;
+    bool plain = false;
     if (kind == ACS_KIND_RHS) {
         tile.bx = tile.by = 16;
         // Few planes per resident block: the FP64 march (4 grids with sides of 16 to 60, 3.2 planes: 87 us
         // against 95 to 105; 12 grids, 8.9 planes: 223 against 165).
         long long planes = 0;
         for (int q = 0; q < n; ++q) planes += (i64)((geo[q].nx + 15) / 16) * ((geo[q].ny + 15) / 16) * geo[q].nz;
-        if (planes < 5 * resident_batch_blocks(kind, tile)) tile.flags |= kBatchPlain;
+        plain = planes < 5 * resident_batch_blocks(kind, tile);
     }
     std::vector<unsigned char> image;
     long long total = 0;
-    acs_status st = batch_pack(items, geo, n, kind, tile, (uintptr_t)ws, image, total);
+    acs_status st = batch_pack(items, geo, n, kind, tile, plain, (uintptr_t)ws, image, total);
     if (st != ACS_OK) return st;
     if (image.size() > ws_bytes) return fail(ACS_ERR_WORKSPACE, "workspace %zu bytes < %zu needed", ws_bytes, image.size());
     if (cudaMemcpyAsync(ws, image.data(), image.size(), cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -291,8 +286,7 @@ acs_status batch_launch(const BatchPlanHost& p, const RhsConst& rk, const StarCo
     if (cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return launch_status("cudaMemsetAsync");
     acs_status st;
     if (batch_fixed_launch(p, counter, rk, sc, s, st)) return st;
-    if (p.kind == ACS_KIND_RHS) return dispatch<ACS_KIND_RHS>(p, counter, rk, sc, s);
-    return dispatch<ACS_KIND_STENCIL>(p, counter, rk, sc, s);
+    return dispatch(p, counter, rk, sc, s);
 }
 
 }  // namespace acs

@@ -19,7 +19,8 @@ struct BatchHeader {
     unsigned long long counter;
     long long total;
     int n, kind, bx, by, kchunk, maps_off;   // maps_off: byte offset of the tensor maps (0: none)
-    long long pad1[3];
+    int plain, pad;                          // plain: too little work for the fixed-point RHS march
+    long long pad1[2];
 };
 static_assert(sizeof(BatchHeader) == 64, "batch header is 64 bytes");
 

@@ -139,21 +139,31 @@ size_t rhs_smem_bytes(int bx, int by) {
     return 0;
 }
 
+// The fixed-point march is built for 16 x 16 columns (larger ones leave room for one block on an SM,
+// 16 x 8 ran 1.4 times slower) and takes any requested tile but on grids that fill these columns much
+// worse, such as a few rows of long lines. It starts four planes before its first result (the FP64
+// march one), so it needs a few planes per resident block: 64^3 (3.4 planes) 70.3 -> 43.0 us, 48^3
+// (1.4) 42.6 -> 43.4, 32^3 (0.4) 17.5 -> 22.0.
+static bool fills_fixed(const Geom& g, const RhsFix& fx, const acs_tile& t) {
+    auto padded = [&](int bx, int by) { return (i64)((g.nx + bx - 1) / bx * bx) * ((g.ny + by - 1) / by * by); };
+    const i64 work = padded(16, 16) / 256 * g.nz;
+    return fx.ok && rhs_tile_supported(t.bx, t.by) && work >= 4 * (i64)num_sms() &&
+           padded(16, 16) <= padded(t.bx, t.by) + padded(t.bx, t.by) / 2;
+}
+
+bool rhs_takes_fixed(const Geom& g, const RhsConst& k, const acs_tile& t) {
+    RhsFix fx;
+    RhsConst kc;
+    rhs_fix(k, fx, kc);
+    return fills_fixed(g, fx, t);
+}
+
 acs_status launch_rhs_saturated(const double* U, double* R, const Geom& g, const RhsConst& k, const acs_tile& t,
                                 cudaStream_t s) {
     RhsFix fx;
     RhsConst kc;
     rhs_fix(k, fx, kc);
-    // The fixed-point march is built for 16 x 16 columns (larger ones leave room for one block on an SM,
-    // 16 x 8 ran 1.4 times slower) and takes any requested tile but on grids that fill these columns much
-    // worse, such as a few rows of long lines. It starts four planes before its first result (the FP64
-    // march one), so it needs a few planes per resident block: 64^3 (3.4 planes) 71.6 -> 46.7 us, 48^3
-    // (1.4) 42.6 -> 43.4, 32^3 (0.4) 17.5 -> 22.0.
-    auto padded = [&](int bx, int by) { return (i64)((g.nx + bx - 1) / bx * bx) * ((g.ny + by - 1) / by * by); };
-    const i64 work = padded(16, 16) / 256 * g.nz;
-    if (fx.ok && rhs_tile_supported(t.bx, t.by) && work >= 4 * (i64)num_sms() &&
-        padded(16, 16) <= padded(t.bx, t.by) + padded(t.bx, t.by) / 2)
-        return launch_rhs_fixed(U, R, g, k, kc, fx, t, s);
+    if (fills_fixed(g, fx, t)) return launch_rhs_fixed(U, R, g, k, kc, fx, t, s);
     if (t.bx == 32 && t.by == 8) return launch_t<32, 8>(U, R, g, k, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 4) return launch_t<32, 4>(U, R, g, k, t.kchunk, t.flags, s);
     if (t.bx == 32 && t.by == 16) return launch_t<32, 16>(U, R, g, k, t.kchunk, t.flags, s);

@@ -43,6 +43,7 @@ std::string key_of(int kind, const Geom* g, int n) {
 const int kRhsTiles[][2] = {{32, 8}, {32, 4}, {32, 16}, {16, 8}, {16, 16}, {64, 4}};
 const int kStarTiles[][2] = {{32, 8}, {32, 4}, {32, 16}, {64, 4}, {64, 8}, {16, 16}, {16, 8}};
 constexpr int kNumRhsTiles = (int)(sizeof(kRhsTiles) / sizeof(kRhsTiles[0]));
+const int kFixedRhsTile[][2] = {{16, 16}};   // the columns of the fixed-point RHS and of RHS batches
 constexpr int kNumStarTiles = (int)(sizeof(kStarTiles) / sizeof(kStarTiles[0]));
 // z-chunk candidates; kBalanced stands for the balanced schedule (ACS_TILE_BALANCED).
 constexpr int kBalanced = -1;
@@ -158,8 +159,16 @@ bool tuned_tile(int kind, const Geom& g, acs_tile* t) {
 acs_status tune_rhs(const double* U, double* R, const Geom& g, const RhsConst& k, cudaStream_t s, acs_tile* best,
                     float* best_ms) {
     static const int staging[] = {0, ACS_TILE_TMA};   // element-wise cp.async or TMA plane copies
+    // Tiles that all run the fixed-point march's columns are tried (and recorded) as those, once.
+    int tiles[kNumRhsTiles][2], n = 0;
+    for (int q = 0; q < kNumRhsTiles; ++q) {
+        const int bx = kRhsTiles[q][0], by = kRhsTiles[q][1];
+        if ((bx != 16 || by != 16) && rhs_takes_fixed(g, k, acs_tile{bx, by, 0, 0})) continue;
+        tiles[n][0] = bx;
+        tiles[n++][1] = by;
+    }
     return tune_grid(
-        ACS_KIND_RHS, g, kRhsTiles, kNumRhsTiles, staging, 2,
+        ACS_KIND_RHS, g, tiles, n, staging, 2,
         [&](const acs_tile& c) { return launch_rhs_saturated(U, R, g, k, c, s); }, s, best, best_ms);
 }
 
@@ -176,8 +185,8 @@ acs_status tune_batch(const acs_batch_item* items, const Geom* geo, int n, int k
                       float* best_ms) {
     Timer t;
     if (!t.init()) return launch_status("cudaEventCreate");
-    const int(*tiles)[2] = kind == ACS_KIND_RHS ? kRhsTiles : kStarTiles;
-    const int ntiles = kind == ACS_KIND_RHS ? kNumRhsTiles : kNumStarTiles;
+    const int(*tiles)[2] = kind == ACS_KIND_RHS ? kFixedRhsTile : kStarTiles;
+    const int ntiles = kind == ACS_KIND_RHS ? 1 : kNumStarTiles;
     acs_tile bt = {0, 0, 0, 0};
     float bms = 1e30f;
     static const int chunks[] = {4, 6, 8, 12, 16, 32};
@@ -190,12 +199,13 @@ acs_status tune_batch(const acs_batch_item* items, const Geom* geo, int n, int k
             BatchPlanHost plan;
             acs_status st = batch_prepare_host(items, geo, n, kind, cand, ws, ws_bytes, s, plan);
             if (st != ACS_OK) return st;
+            if (f && !(plan.tile.flags & ACS_TILE_TMA)) continue;   // staged element-wise, as tried before
             float ms = 0.f;
             st = time_best([&]() { return batch_launch(plan, rk, sc, s); }, s, t, ms);
             if (st != ACS_OK) return st;
             if (ms < bms) {
                 bms = ms;
-                bt = cand;
+                bt = plan.tile;
             }
           }
         }

@@ -239,3 +239,47 @@ def test_stagings_agree_bitwise_where_scales_differ(kind, kchunk, flags):
     for h in ((1.0, 1.0, 1.0), (1.0, 1.5, 2.0)):
         t, e = (_rhs(U, (16, 16, kchunk, flags | f), 1.4, 0.25, h) for f in (binding.TILE_TMA, 0))
         assert np.array_equal(t, e), (h, int((t != e).sum()))
+
+
+def _rhs_grids(sides, seed):
+    out = []
+    for q, (nx, ny, nz) in enumerate(sides):
+        U = inputs.rhs_field(nx, ny, nz, halo=2, seed=seed + q)
+        out.append((to_dev(U), None, torch.full((5, nz, ny, nx), float("nan"), dtype=torch.float64, device="cuda")))
+    return out
+
+
+@pytest.mark.parametrize("sides", [[(16, 16, 16), (20, 18, 5)], [(64, 48, 50)] * 6])
+@pytest.mark.parametrize("tile", [None, (32, 8, 12), (16, 16, 32)])
+def test_rhs_batch_plan_tile_prepares_the_same_plan(tile, sides):
+    """A prepared plan's tile is the shape that runs, and prepares it again: batches with little work, which
+    run the FP64 march, and others."""
+    grids = _rhs_grids(sides, 4700)
+    ws = torch.zeros(binding.acs_batch_workspace_bytes(len(grids)) // 8 + 2, dtype=torch.float64, device="cuda")
+
+    def run(t):
+        plan = binding.acs_batch_prepare(binding.KIND_RHS, grids, ws, tile=t)
+        binding.acs_batch_launch(plan)
+        torch.cuda.synchronize()
+        return plan, [R.clone() for _, _, R in grids]
+
+    p, first = run(tile)
+    assert (p.tile.bx, p.tile.by, p.tile.flags) == (16, 16, 0)
+    again, second = run((p.tile.bx, p.tile.by, p.tile.kchunk, p.tile.flags))
+    assert again.total_units == p.total_units
+    assert all(torch.equal(x, y) for x, y in zip(first, second))
+    binding.acs_batch_run_static(binding.KIND_RHS, grids, tile=(p.tile.bx, p.tile.by, p.tile.kchunk, p.tile.flags))
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, R) for x, (_, _, R) in zip(first, grids))
+
+
+def test_autotuners_name_the_columns_that_run():
+    """Grids and batches the fixed-point RHS takes run in 16 x 16 columns: so do the tuners' winners."""
+    try:
+        (U, _, R), = _rhs_grids([(96, 64, 48)], 4800)
+        assert tuple(binding.acs_autotune_rhs(U, R)[0])[:2] == (16, 16)
+        grids = _rhs_grids([(64, 48, 50)] * 4, 4900)
+        ws = torch.zeros(binding.acs_batch_workspace_bytes(len(grids)) // 8 + 2, dtype=torch.float64, device="cuda")
+        assert tuple(binding.acs_autotune_batch(binding.KIND_RHS, grids, ws)[0])[:2] == (16, 16)
+    finally:
+        binding.acs_tune_cache_clear()
