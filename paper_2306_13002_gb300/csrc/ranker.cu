@@ -170,6 +170,7 @@ __global__ void mlp_grad_adam(const float* __restrict__ X, const float* __restri
 // is kept, and two cluster barriers with a trip through the L2 per epoch.
 constexpr int kTrainBlocks = 8, kTrainThreads = 512, kTrainH = 64, kTrainRows = kTrainH / kTrainBlocks;
 constexpr int kSamples = 4;               // samples a thread works on at once
+constexpr int kTrainMost = 2;             // parameters besides W2 per thread
 constexpr int kTrainPad = kTrainH + 1;   // row pitch of the activations a thread reads along
 
 struct TrainShape {
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(kTrainThreads)
     if (tid < 128)
         for (int q = 0; q < 4; ++q) p4[q] = prm[L.W2 + (size_t)(j0 + jq + q / 2) * H + k2 + q % 2];
     const int others = kTrainRows * F + 3 * kTrainRows + (blk == 0 ? 1 : 0);
-    constexpr int kOther = kTrainThreads - 128, kMost = 2;   // others <= 8 * 93 + 25
+    constexpr int kOther = kTrainThreads - 128, kMost = kTrainMost;   // others <= kOther * kMost (train_fits)
     size_t po[kMost];
     float pv[kMost], mv[kMost], vv[kMost];
     for (int r = 0; r < kMost; ++r) {
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(kTrainThreads)
 
 // Whether the one-launch training takes this model and training set.
 bool train_fits(int n, int F, int H) {
-    return H == kTrainH && n >= kTrainBlocks && kTrainRows * F + 3 * kTrainRows + 1 <= 2 * (kTrainThreads - 128) &&
+    return H == kTrainH && n >= kTrainBlocks && kTrainRows * F + 3 * kTrainRows + 1 <= kTrainMost * (kTrainThreads - 128) &&   // F <= 92
            TrainShape(n, F).floats * sizeof(float) <= 227 * 1024;
 }
 

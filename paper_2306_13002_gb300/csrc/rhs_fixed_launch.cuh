@@ -87,20 +87,16 @@ acs_status launch_rhs_fixed_t(const double* U, double* R, const Geom& g, const R
     return launch_status("rhs_fixed_kernel");
 }
 
-template <int BX, int BY, bool ISO>
-acs_status launch_rhs_fixed_tile(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
+// 16 x 16 columns, with the tile's schedule and staging.
+template <bool ISO>
+acs_status launch_rhs_fixed_form(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
                                  const RhsFix& fx, const acs_tile& t, cudaStream_t s) {
+    constexpr int BX = 16, BY = 16;
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
     if ((t.flags & ACS_TILE_TMA) && encode_plane_map(U, g, 5, BX + 4, BY + 4, &map) == ACS_OK)
         return launch_rhs_fixed_t<BX, BY, true, ISO>(U, R, g, kf, kc, fx, t.kchunk, t.flags, map, s);
     return launch_rhs_fixed_t<BX, BY, false, ISO>(U, R, g, kf, kc, fx, t.kchunk, t.flags, map, s);
-}
-
-template <bool ISO>
-acs_status launch_rhs_fixed_form(const double* U, double* R, const Geom& g, const RhsConst& kf, const RhsConst& kc,
-                                 const RhsFix& fx, const acs_tile& t, cudaStream_t s) {
-    return launch_rhs_fixed_tile<16, 16, ISO>(U, R, g, kf, kc, fx, t, s);
 }
 
 }  // namespace
