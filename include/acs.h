@@ -44,8 +44,15 @@
  *    human-readable reason for the last failure of the calling thread.
  *  - Inputs and outputs must not overlap in memory (ACS_ERR_ALIAS).
  *  - The saturated kernels add neighbours in 64-bit fixed point, with one exponent per block of
- *    planes, where the values' ranges allow it, and in FP64 elsewhere. Results are as near to the
- *    exact value as FP64's or nearer; their last bits may depend on the launch shape.
+ *    planes, where the values' ranges allow it, and in FP64 elsewhere. Measured against exact values,
+ *    the errors (root mean square, relative to a point's sum of |terms|) are no larger than FP64's,
+ *    also among points far below the block's largest value. What has no such bound: where FP64's
+ *    terms cancel exactly (a fluid at rest under uniform pressure), momenta far below the block's
+ *    largest keep an absolute error of a few 2^-59 of that.
+ *  - The last bits of a saturated result depend on the exponents of its block, hence on the tile,
+ *    the z-chunks, the schedule (which follows the number of SMs) and the slabs of host-streamed
+ *    calls, and on values up to a tile away. Mirrored or negated inputs need not give mirrored or
+ *    negated last bits. The same call on the same device gives the same bits every time.
  *  - The saturated RHS computes 1/rho with a refined hardware reciprocal estimate for
  *    normal |rho| in [2^-1000, 2^1001), faithful (within 1 ulp of the correctly rounded 1/rho),
  *    and falls back to an IEEE division otherwise.
@@ -135,7 +142,7 @@ typedef struct acs_tile {
  * (acs_batch_prepare, acs_autotune_batch: per grid; RHS batches and acs_batch_run_static reject
  * it). Used where the layout allows it (16-byte aligned input, row, plane and component strides
  * that are multiples of 2 elements, even halo); other layouts, and batches with such a
- * grid, are staged element-wise, with the same results. Waits on the mbarriers are bounded (about one
+ * grid, are staged element-wise, with the same results for the same tile and z-chunks. Waits on the mbarriers are bounded (about one
  * second); one that runs out is counted (acs_wait_timeouts) and the call's results are then
  * wrong, but the kernel ends. */
 #define ACS_TILE_TMA 2
@@ -157,9 +164,13 @@ acs_status acs_rhs_plain(const double *U, double *R, const acs_grid *g, const ac
  * sum(U at +-2) - 4 sum(U at +-1) + 18 U, and every plane of U staged in shared memory ahead of
  * the arithmetic (bulk load). Grids of more than two planes per resident block with positive spacing
  * and dissipation form the fluxes in FP64 (23 operations per point with equal spacing, 30 without)
- * and the differences and the dissipation in fixed point, in blocks whose values' ranges suit it; the
+ * and the differences and the dissipation in fixed point, in blocks whose values suit it; the
  * others run in FP64 throughout (114 operations with equal spacing within 2^-65 .. 2^63, where -1/(2h)
- * is folded into the fluxes, else 116). All forms equal the as-written definition over the reals
+ * is folded into the fluxes, else 116), about three times as long. Values suit it if rho and E are
+ * positive and keep within a factor of 2^7 in a block, and if the bounds on the fluxes that follow from
+ * them, times 1/(2h), are at most 2^10 times the dissipation eps E (eps rho) and 2^8 times the pressure's
+ * share: for states near 1 and eps = 0.25, spacings of about 0.1 (uniform noise) or 0.05 (smooth flow)
+ * and more, and axes that differ by up to 8; for eps = 0.03, a spacing of 1. All forms equal the as-written definition over the reals
  * and differ from it only by rounding. Same arguments as acs_rhs_plain plus
  *   tile     launch shape or NULL (the autotuned shape for this grid size if acs_autotune_rhs
  *            recorded one, else 16 x 16 with the balanced schedule and TMA plane staging where
@@ -222,7 +233,9 @@ acs_status acs_stencil_plain(const double *u, const double *a, double *out, cons
  *   C0 = -2 sum c (folded on the host), u planes staged in shared memory and reused by the 9
  *   z-offsets as the block marches along z. Weights of alternating sign (second-derivative weights
  *   of every order) are summed exactly in block-scaled 64-bit fixed point and rounded once, others in
- *   FP64 with FMA throughout; points and blocks whose values do not fit the scale fall back to FP64.
+ *   FP64 with FMA throughout. Points whose own value and next neighbours are below about 2^-6 of
+ *   their block's largest value, and blocks with many of them (localized fields), run in FP64: a field
+ *   of such blocks only takes the FP64 kernel's time, about four times as long.
  *   tile   launch shape or NULL (the autotuned shape for this grid size if
  *          acs_autotune_stencil recorded one, else a shape by weights and layout, z-chunks from the
  *          grid size, TMA plane staging where the layout allows it).
@@ -275,7 +288,8 @@ size_t acs_batch_workspace_bytes(int n);
  * batch are 16 x 16 whatever the tile); tile->flags may be ACS_TILE_TMA for a star-stencil batch,
  * which encodes a tensor map per grid into the workspace if every grid of the batch can be staged so
  * (even row and plane pitch, 16-byte aligned; otherwise all are staged element-wise). Long z-chunks
- * are shortened for batches with little work per resident block. On success fills `plan`.
+ * are shortened for batches with little work per resident block. On success fills `plan`; plan->tile
+ * is the shape that runs, and prepares the same plan if it is passed back.
  */
 acs_status acs_batch_prepare(const acs_batch_item *items, int n, int kind, const acs_tile *tile, void *ws,
                              size_t ws_bytes, acs_batch_plan *plan, acs_stream stream);

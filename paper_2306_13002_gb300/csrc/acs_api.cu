@@ -380,8 +380,8 @@ acs_status batch_params(int kind, const void* params, RhsConst& rk, StarCoef& sc
 const acs_tile kDefaultRhsTile = {16, 16, 0, ACS_TILE_BALANCED | ACS_TILE_TMA};
 const acs_tile kDefaultStarTile = {32, 8, 0, ACS_TILE_TMA};
 // The star stencil's tile without one asked for. Fixed-point march, 32 x 8 / 16 x 8 / 16 x 16: same weights
-// on every axis and tensor copies 605 / 591 / 601 us at 384^3 (4.49 / 4.38 / 4.47 ms at 768^3), element-wise
-// 660 / 699 / 679; weights of its own per axis 876 / 902 / 860 (6.57 / 6.73 / 6.45 ms).
+// on every axis and tensor copies 561 / 562 / 563 us at 384^3 (4.17 / 4.17 / 4.18 ms at 768^3), element-wise
+// 589 / 649 / 585; weights of its own per axis 788 / 844 / 781 (5.91 / 6.33 / 5.86 ms).
 acs_tile default_star_tile(const Geom& g, const StarCoef& cf, const double* u) {
     StarFix fx;
     star_fix(cf, fx);
@@ -391,8 +391,8 @@ acs_tile default_star_tile(const Geom& g, const StarCoef& cf, const double* u) {
     return kDefaultStarTile;
 }
 // Batches: the marches start a few planes before their first result, so chunks are long (64 star grids:
-// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16; 32 RHS grids: 397 us with chunks of
-// 32, 412 with 24, 434 with 16, 496 with 8); batches with less work take shorter ones (batch_pack).
+// 245 us with 16 x 8 x 32, 266 with 16 x 8 x 16, 268 with 32 x 8 x 16, and 235 as it is now; 32 RHS grids: 397 us
+// with chunks of 32, 412 with 24, 434 with 16, 496 with 8, and 390 now); batches with less work take shorter ones (batch_pack).
 acs_tile default_batch_tile(int kind, int staging) {
     return kind == ACS_KIND_STENCIL ? acs_tile{16, 8, 32, staging} : acs_tile{16, 16, 32, 0};
 }

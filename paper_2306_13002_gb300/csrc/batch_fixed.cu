@@ -1,6 +1,6 @@
 // The batched persistent launch with the fixed-point marches (star_fixed.cuh, rhs_fixed.cuh): the same
-// queue of units as batch_kernel. Measured on GB300: 64 star grids with sides of 16 to 160 680 -> 244 us,
-// 32 RHS grids with sides of 16 to 96 912 -> 398 us (small grids: a third of the steps of an RHS unit are
+// queue of units as batch_kernel. Measured on GB300: 64 star grids with sides of 16 to 160 680 -> 235 us,
+// 32 RHS grids with sides of 16 to 96 912 -> 390 us (small grids: a third of the steps of an RHS unit are
 // its start, and its element-wise staging has to serve any row pitch).
 #include "batch_desc.cuh"
 #include "rhs_fixed.cuh"

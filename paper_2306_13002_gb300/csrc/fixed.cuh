@@ -4,14 +4,15 @@
 // mostly adds neighbours runs 5 to 8 times longer on the FP64 pipe than it takes to add the same
 // numbers as 64-bit integers (two 32-bit instructions per sum of three terms). The marches that use
 // this header convert every input once, when its plane is staged, to
-//     q = trunc(v / d) + bias,   d = 2^(E0 - 1023 - 59),
+//     q = floor(v / d) + bias,   d = 2^(E0 - 1023 - 59),
 // with one exponent E0 per block and segment (the largest exponent staged), |v / d| < 2^60. Integer
 // sums are exact, so the only errors are the conversion's (less than d per input, 2^-59 of the
 // segment's largest value) and the final rounding. FP64 rounds every partial sum to 53 bits.
 //
-// Values far below the block's largest lose their low bits in this form, so each march also
-// has a per-point test of the local magnitude and evaluates the points that fail it in FP64, and
-// leaves the fixed-point form when an input exceeds E0 or is not finite.
+// Values far below the block's largest lose their low bits in this form. The star march tests each point for
+// it and evaluates those that fail in FP64; the RHS march takes only planes whose values keep ranges that
+// leave its errors below FP64's. Both leave the form when an input exceeds E0 or is not finite. What a
+// block leaves runs in a staged FP64 march at its end.
 #pragma once
 
 #include "device_ops.cuh"

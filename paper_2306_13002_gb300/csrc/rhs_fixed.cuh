@@ -11,16 +11,20 @@
 // Scales: one exponent each for rho, the momenta and E, from the first planes of a segment, with
 // the ranges of rho and E below them (they enter the bounds of the fluxes, and a point's own values
 // must not lose their low bits); the fluxes' scales follow from these bounds. A plane that leaves
-// the ranges ends the segment.
+// the ranges ends the segment. The rule compares the bounds with the dissipation and the pressure (see
+// segment), so it takes spacings near 1 (0.1 to 1 for the uniform and smooth states of perf/cases.py with a
+// dissipation of 0.25, down to 0.03 with a spacing of 1) and refuses much finer or more uneven ones.
 //
-// Measured on GB300: 256^3 3237 us in FP64 (114 operations per point, 94 % of the FP64 pipe) -> 1160 us
-// (element-wise staging 1268), three spacings 3270 -> 1384, 162^3 with three spacings 999 -> 441, 512^3 of a
-// smooth flow 25.7 -> 8.5 ms, 128^3 420 -> 178. Error against 64 bits (2-norm): uniform state 2.2e-16 ->
-// 4.9e-17, smooth flow 2.4e-15 -> 5.7e-16. What bounds it now: a warp's own chains. About 1200
-// instructions per point (29 of them FP64, ring included: 67 % of that pipe's time) issue at 44 % of
-// the peak rate, 16 warps per SM being what two rings of six planes and 128 registers leave room
-// for; the stalls are FP64 and shared-memory results (2.5 cycles per instruction), fixed latencies (1.8)
-// and the two barriers per plane (1.1).
+// Measured on GB300: 256^3 3237 us in FP64 (114 operations per point, 94 % of the FP64 pipe) -> 1113 us
+// (element-wise staging 3403 -> 1252), three spacings 3293 -> 1410, 162^3 with three spacings 999 -> 444, 512^3
+// of a smooth flow 25.7 -> 8.4 ms, 128^3 420 -> 168. Values that are refused: 256^3 3254 -> 3260, 128^3 420 -> 424,
+// 64^3 70.3 -> 74.1 (the scan, 4 us per block). Error against 64 bits (2-norm): uniform state 2.2e-16 -> 4.9e-17,
+// smooth flow 2.4e-15 -> 5.7e-16; no larger than FP64's in any octave of the points' own magnitudes, up to
+// the ends of the ranges (momenta from 2^-30 to 2^-3, rho and E over 2^6). What bounds it now: a warp's own
+// chains. About 1200 instructions per point (29 of them FP64, ring included: 70 % of that pipe's time) issue
+// at 46 % of the peak rate, 16 warps per SM being what two rings of six planes and 128 registers leave room
+// for; the stalls are FP64 and shared-memory results (2.1 cycles per instruction), fixed latencies (1.7)
+// and the two barriers per plane (1.2).
 #pragma once
 
 #include "fixed.cuh"
