@@ -283,3 +283,22 @@ def test_autotuners_name_the_columns_that_run():
         assert tuple(binding.acs_autotune_batch(binding.KIND_RHS, grids, ws)[0])[:2] == (16, 16)
     finally:
         binding.acs_tune_cache_clear()
+
+
+@pytest.mark.parametrize("fixed,prm", [
+    (True, {}), (True, {"eps": 0.03}), (True, {"eps": 0.1, "h": (0.37, 0.37, 0.37)}), (True, {"h": (0.1, 0.1, 0.1)}),
+    (True, {"h": (1.0, 0.5, 2.0)}), (True, {"h": (1.0, 1.0, 8.0)}), (True, {"gamma": 5.0 / 3.0}), (True, {"gamma": 0.5}),
+    (False, {"eps": 0.01}), (False, {"h": (1.0 / 64,) * 3}), (False, {"h": (1.0, 1.0, 16.0)}), (False, {"gamma": 1.0}),
+    (False, {"eps": 1e-9}), (False, {"h": (1e-5, 1.0, 1.0)}),
+])
+def test_rhs_which_march_ran(fixed, prm):
+    """A grid too small for the fixed-point march runs in FP64, and what a block leaves runs the same operations in
+    the same order: a slab of a larger grid, taken alone, has the larger one's bits if and only if that ran in FP64.
+    Both within the bound of the exact value."""
+    U = inputs.rhs_field(83, 70, 61, halo=2, seed=60)
+    args = (prm.get("gamma", 1.4), prm.get("eps", 0.25), prm.get("h", (1.0, 1.0, 1.0)))
+    for tile in (None, (16, 16, 20, 2), (16, 16, 20, 0)):
+        whole, slab = _rhs(U, tile, *args), _rhs(U[:, 20:44], None, *args)
+        same = whole[:, 20:40] == slab
+        assert same.mean() < 0.9 if fixed else same.all(), (tile, same.mean())
+        _check_rhs(U, tile, str(prm), *args)
