@@ -2,6 +2,7 @@
 // compile one of its two weight forms.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -11,8 +12,8 @@ namespace acs {
 namespace {
 
 // z-chunk of a launch: the work per resident slot plus a third of a chunk for the uneven end, each
-// chunk paying about three plane steps for its prologue (384^3, 32 x 8: chunks of 64 run 632 us, of
-// 128 686 us, though both fill 95 % of their waves).
+// chunk paying about three plane steps for its prologue (384^3, 32 x 8: chunks of 64 ran 632 us, of
+// 128 686 us, though both fill 95 % of their waves; 561 us now).
 int star_fixed_kchunk(int nz, i64 columns, i64 slots) {
     static const int cand[] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128};
     int best = nz;
@@ -25,6 +26,13 @@ int star_fixed_kchunk(int nz, i64 columns, i64 slots) {
             best_cost = cost;
             best = kc < nz ? kc : nz;
         }
+    }
+    // A launch of one wave: the columns in as many parts as there are slots for, so that the SMs hold the same
+    // number of blocks (160^3 of shells, where FP64 runs all of it, in chunks of 32 and 27: 16 x 8 204 -> 188 us,
+    // 16 x 16 with distinct weights 222 -> 189, FP64 kernel 186; uniform values 59 -> 53 and 78 -> 70).
+    if (columns * ((nz + best - 1) / best) <= slots) {
+        const int parts = (int)(slots / columns);
+        best = std::max(std::min(best, 4), (nz + parts - 1) / parts);
     }
     return best < 1 ? 1 : best;
 }
