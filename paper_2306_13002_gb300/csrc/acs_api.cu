@@ -381,12 +381,13 @@ const acs_tile kDefaultRhsTile = {16, 16, 0, ACS_TILE_BALANCED | ACS_TILE_TMA};
 const acs_tile kDefaultStarTile = {32, 8, 0, ACS_TILE_TMA};
 // The star stencil's tile without one asked for. Fixed-point march, 32 x 8 / 16 x 8 / 16 x 16: same weights
 // on every axis and tensor copies 561 / 562 / 563 us at 384^3 (4.17 / 4.17 / 4.18 ms at 768^3), element-wise
-// 589 / 649 / 585; weights of its own per axis 788 / 844 / 781 (5.91 / 6.33 / 5.86 ms).
+// 589 / 649 / 585; weights of its own per axis 788 / 844 / 781 (5.91 / 6.33 / 5.86 ms), element-wise 852 / 974 / 936.
 acs_tile default_star_tile(const Geom& g, const StarCoef& cf, const double* u) {
     StarFix fx;
     star_fix(cf, fx);
     const bool copies = ((g.isy | g.isz | g.halo) & 1) == 0 && (uintptr_t)u % 16 == 0;
-    if (fx.kind == 2) return acs_tile{16, 16, 0, ACS_TILE_TMA};
+    auto padded = [&](int bx, int by) { return (i64)((g.nx + bx - 1) / bx * bx) * ((g.ny + by - 1) / by * by); };
+    if (fx.kind == 2 && (copies || 10 * padded(16, 16) < 9 * padded(32, 8))) return acs_tile{16, 16, 0, ACS_TILE_TMA};
     if (fx.kind == 1 && copies) return acs_tile{16, 8, 0, ACS_TILE_TMA};
     return kDefaultStarTile;
 }

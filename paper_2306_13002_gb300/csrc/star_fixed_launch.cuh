@@ -32,7 +32,8 @@ int star_fixed_kchunk(int nz, i64 columns, i64 slots) {
     // 16 x 16 with distinct weights 222 -> 189, FP64 kernel 186; uniform values 59 -> 53 and 78 -> 70).
     if (columns * ((nz + best - 1) / best) <= slots) {
         const int parts = (int)(slots / columns);
-        best = std::max(std::min(best, 4), (nz + parts - 1) / parts);
+        const int even = ((nz + parts - 1) / parts + 1) & ~1;   // (the march takes two planes at a time)
+        best = std::max(std::min(best, 4), std::min(even, best));
     }
     return best < 1 ? 1 : best;
 }
