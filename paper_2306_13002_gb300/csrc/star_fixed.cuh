@@ -9,7 +9,7 @@
 //
 // Measured on GB300, tensor copies: 384^3 with 16 x 8 tiles 2388 us in FP64 (26 operations per point, 98 %
 // of the FP64 pipe) -> 562 us; 768^3, a smooth wave with distinct weights per axis, 19.0 -> 6.33 ms. Fields
-// whose every point is left to FP64 (values 2^40 apart): 384^3 2405 -> 2420, 160^3 186 -> 189, 61 x 47 x 53
+// whose every point is left to FP64 (values 2^40 apart): 384^3 2405 -> 2420, 160^3 186 -> 195, 61 x 47 x 53
 // 21.0 -> 20.8.
 // Error against 64 bits (2-norm): uniform values 3.1e-16 -> 8.1e-17, a smooth wave 5.8e-15 -> 9.6e-17. What
 // bounds it now: about 240 instructions per point (127 on the ALU pipe, 63 on the FMA pipe) issued at 56 % of

@@ -28,8 +28,8 @@ int star_fixed_kchunk(int nz, i64 columns, i64 slots) {
         }
     }
     // A launch of one wave: the columns in as many parts as there are slots for, so that the SMs hold the same
-    // number of blocks (160^3 of shells, where FP64 runs all of it, in chunks of 32 and 27: 16 x 8 204 -> 188 us,
-    // 16 x 16 with distinct weights 222 -> 189, FP64 kernel 186; uniform values 59 -> 53 and 78 -> 70).
+    // number of blocks (160^3 of shells, where FP64 runs all of it, in chunks of 32 and 28: 16 x 8 204 -> 195 us,
+    // 16 x 16 with distinct weights 222 -> 195, FP64 kernel 186; uniform values 59 -> 53 and 78 -> 70).
     if (columns * ((nz + best - 1) / best) <= slots) {
         const int parts = (int)(slots / columns);
         const int even = ((nz + parts - 1) / parts + 1) & ~1;   // (the march takes two planes at a time)
